@@ -15,15 +15,16 @@
 // routed by their wedge count W (a count is at most W too): one warp with a
 // 6 KB table (k_c4_warp) or an 8 KB one (k_c4_warp_big), four warps
 // (k_c4_mid, packed or split tables), a 512-thread CTA (k_c4_cta), or, for the largest
-// roots, and for every root with more than WL_MAXD in-neighbours, a
-// 1024-thread CTA that counts the root's key range tile by tile in shared
-// memory (k_c4_tiled). The other tables are open-addressing hash
+// roots, and for every root with more than WL_MAXD in-neighbours, a CTA with
+// a directly indexed counter per key in shared memory (k_c4_tiled). The other tables are open-addressing hash
 // tables in shared memory, either split (key and count arrays) or packed
 // (key << cb | count in one 32-bit word, cb = 32 - bits(n - 1) count bits,
 // usable while W < 2^cb - 1), which holds twice the keys in the same space.
 // Each table is emptied once per CTA; afterwards a warp sweeps the region
 // its root used, and a CTA empties the slots it filled (kept in a 16-bit
 // `touched` list).
+#include <type_traits>
+
 #include "kernels.h"
 
 namespace niorca {
@@ -658,59 +659,179 @@ __global__ void __launch_bounds__(CC_THREADS) k_c4_cta(Graph g, VAcc *vacc, cons
 //
 // Roots with more wedges than the hash tiers take (W > teamw): one CTA per
 // root, largest roots first. The keys w of a root u are the vertices below
-// u; the CTA cuts them into tiles of TK consecutive ids and counts each
-// tile's wedges in shared memory (16-bit counters while the root has fewer
-// than 65535 in-neighbours, as no count exceeds that; 32-bit ones, half as
-// many keys, above). A root's wedges through its in-neighbour v are the
-// entries of row v below u, ascending, so the wedges that fall into a tile
-// are a run of that row: every in-neighbour keeps a cursor (the start of its
-// next run), the end of its wedge prefix and the key at the cursor. A tile
-// first finds every in-neighbour's run (a galloping search from the cursor,
-// one thread per in-neighbour) and its offset in the concatenation of the
-// tile's runs (a prefix sum across the CTA); every warp then takes an equal
-// slice of that concatenation, weighted so that each chunk of 32
-// in-neighbours also counts for its overhead, and neither hub rows nor many
-// short runs leave warps waiting.
-// It counts the slice's wedges, credits C(c, 2) to every key w and to u
-// from the counts, walks the slice again adding c - 1 per wedge to its
-// middle vertex, moves the cursors past the runs, and clears. The next tile
-// starts at the smallest key any cursor points at, so key ranges without
-// wedges are skipped.
-// The cursors of all these roots (their in-degrees sum to at most |E|) live
-// in the region of the per-edge triangle counts, which nothing reads after
-// the aggregate stage and which is sized 8 m bytes for them: 16 bytes per
-// in-neighbour, |E| = m / 2 of them.
-constexpr int CK_THREADS = 1024;
-constexpr int CK_NW = CK_THREADS / 32;
-constexpr size_t CK_OTHER = CK_NW * sizeof(SegTab) + CK_NW * 32 * 8 + 64 * 4;   // segment tables, sums, scalars
-// Counter words (204 KB; tiles of 104448 keys with 16-bit counters). Larger
-// tiles pay, as every tile costs passes over the in-neighbours: on R-MAT 22
-// the tier took 598 ms with 48K words, 587 with 50K, 567 with 51K, and
-// 571-572 with 51.5K and with all the 227 KB the rest leaves (52928).
-constexpr int CK_WORDS = 51 * 1024;
+// u; their counters are packed words in shared memory, indexed by w.
+//
+// Counter stream. A count c_uw is at most the degree of w, and ids are
+// ordered by degree class, so an id range has a fixed counter width (zones,
+// ck_zones: 2 bits for degrees 2-3, 3 for 4-7, ... 10 for 256-1023, 16
+// above; a root whose counts could pass 16 bits takes the last zone with
+// 32-bit counters, c4_wide_top). Vertices of degree 0 and 1 are on no cycle
+// and have no counter. All counters form one stream of words, from the
+// highest id down; a group is the part of it that fits the shared memory.
+//
+// The layout is the same for every root, so each column entry's counter
+// (byte address in its group, shift, width) is computed once (`enc`), as are
+// the position in every row where each group starts (`index`, group by
+// group over the vertices) and the position of every root in its
+// in-neighbours' rows (`ends`): k_c4_tiled_plan. They live in the
+// triangle-count region, which nothing reads after the hash tiers.
+//
+// A root takes group after group: it counts its wedges that end in the
+// group (the entries of row v in the group's id range and below u are a
+// contiguous run), walks them again adding c - 1 per wedge to the middle
+// vertex, then sweeps the counters, crediting C(c, 2) to every key and to u,
+// and clears them. A walk takes the runs in batches of one per thread
+// (loaded one batch ahead): a run of at most CK_TINY entries is walked by
+// its thread; the others are listed in shared memory with the prefix sums of
+// their windows of 32 entries, and every warp takes an equal share of the
+// windows. A window lies in one run: a warp finds the runs of 32 windows at
+// once (one window per lane, into a shared list) and then spends a load, two
+// shifts and an atomic on each window, CK_UNROLL of them in flight.
+//
+// Measured (GB300, the tier's time): R-MAT 22 364 -> 114 ms, R-MAT 18
+// 5.34 -> 1.83 ms, R-MAT 14 0.34 -> 0.12 ms, G(1501, 0.5) 1.34 -> 0.48 ms,
+// against tiles of 104448 16-bit counters whose runs were concatenated and
+// looked up entry by entry (63 and 88 instructions per 32 wedges in the two
+// walks). It is bound by shared memory now: on R-MAT 21 the LSU data pipe is
+// 68% busy (3.4 wavefronts per 32 random counter updates) and 60% of the
+// sectors hit L2. Two 512-thread CTAs per SM with half the counters took
+// twice the time (every group passes over all in-neighbours).
+constexpr int CK_TINY = 4;
 constexpr int CK_NARROW_MAXD = 65534;               // in-degree up to which 16-bit counters cannot overflow
-constexpr int CK_INF = 0x7fffffff;
-// Weight of a chunk's overhead in elements when the walks are cut into warp
-// slices: equal element counts left the warps of a tile with many short runs
-// waiting at the tile barriers for the warp with the most chunks (R-MAT 22:
-// 566 ms with equal elements; 430, 398, 372, 363, 367, 371, 392 ms with
-// weights 32, 64, 128, 256, 384, 512, 1024).
-constexpr int CK_ALPHA = 256;
-constexpr size_t CK_SMEM = (size_t)CK_WORDS * 4 + CK_OTHER;
-static_assert(CK_SMEM <= 227 * 1024, "k_c4_tiled shared memory");
+constexpr int CK_WORDS = 48 * 1024;                 // counter words of a 1024-thread CTA
+constexpr int CK_SMALL_N = 12288;                   // graphs whose 16-bit counters fit 24 KB: 256-thread CTAs
+constexpr int CK_MAX_GROUPS = 64;                   // groups up to which there may be an index
+constexpr int CK_ENDS_MAXD = 8192;                  // in-degree of a root up to which `ends` holds its positions
+constexpr int CK_UNROLL = 16;                       // windows a warp has in flight (R-MAT 22: 125 ms with 8)
+constexpr int CK_ZONES = 8;
+constexpr size_t ck_smem(int threads, int words) {
+    // counters; per thread: run start, length, window prefix, vertex and a window; warp totals, zones, scalars
+    return (size_t)words * 4 + (size_t)threads * 24 + (size_t)(threads / 32) * 8 + (CK_ZONES + 1) * 16 + 32;
+}
+static_assert(ck_smem(1024, CK_WORDS) <= 227 * 1024, "k_c4_tiled shared memory");
 
-// Root order of the key-tiled tier: the queued roots (list 4, their wedge
-// counts in list 1) sorted by decreasing wedge count (64 buckets, two per
-// octave) into list 0, and the prefix sums of their in-degrees (the offsets
-// of their cursors) into list 2. One CTA.
-__global__ void __launch_bounds__(1024) k_c4_tiled_plan(Graph g, int *lists, int *counters) {
+// Counter widths of the zones.
+__host__ __device__ constexpr int ck_bits(int zone) {
+    return zone == 0 ? 16 : zone == 1 ? 10 : zone == 2 ? 8 : 8 - zone + 1;
+}
+
+// Zone z: ids [lo, hi), `per` counters of `bits` bits in a word, stream words
+// from `off` on (a multiple of 4). Id w has word off + (hi - 1 - w) / per and
+// field (hi - 1 - w) % per. Zones run from the highest ids down.
+struct __align__(16) CkZone {
+    int lo, hi, off, fmt;
+    __device__ __forceinline__ int per() const { return fmt & 0xff; }
+    __device__ __forceinline__ int bits() const { return fmt >> 8; }
+};
+
+// The zones, from the first id of the class of each zone's lowest degree;
+// z[CK_ZONES].off is the length of the stream. One thread.
+__device__ __forceinline__ void ck_zones(const int *coff, int ntiles, int n, CkZone *z) {
+    const int deg[CK_ZONES] = {1024, 256, 64, 32, 16, 8, 4, 2};
+    int hi = n, off = 0;
+#pragma unroll
+    for (int i = 0; i < CK_ZONES; ++i) {
+        CkZone q;
+        q.hi = hi;
+        q.lo = min(coff[deg_class(deg[i]) * ntiles], hi);
+        q.off = off;
+        const int bits = ck_bits(i), per = 32 / bits;
+        q.fmt = per | bits << 8;
+        off += ((hi - q.lo + per - 1) / per + 3) & ~3;
+        hi = q.lo;
+        z[i] = q;
+    }
+    z[CK_ZONES].lo = z[CK_ZONES].hi = hi;
+    z[CK_ZONES].off = off;
+    z[CK_ZONES].fmt = 1;
+}
+
+// Lowest id with a counter before stream word e.
+__device__ __forceinline__ int ck_low_id(const CkZone *z, long long e) {
+    int lo = z[0].hi;
+    for (int i = 0; i < CK_ZONES && z[i].off < e; ++i)
+        lo = (int)max((long long)z[i].lo, z[i].hi - (e - z[i].off) * z[i].per());
+    return lo;
+}
+
+// Where the plan's arrays lie in the triangle-count region (2 m ints): enc
+// (m ints), ends (m 16-bit offsets from the split of the in-neighbour's
+// row; an out-degree is at most sqrt(1.25 m) < 2^16), index (groups x n
+// ints, when there is room).
+struct CkPlan {
+    int *enc;
+    unsigned short *ends;
+    int *index;
+    int groups;
+    bool indexed;
+};
+__device__ __forceinline__ CkPlan ck_plan(int *region, const CkZone *z, int words, int n, int m) {
+    CkPlan P;
+    P.enc = region;
+    P.ends = reinterpret_cast<unsigned short *>(region + m);
+    P.index = region + m + (m + 1) / 2;
+    P.groups = (z[CK_ZONES].off + words - 1) / words;
+    P.indexed = P.groups <= CK_MAX_GROUPS && (long long)P.groups * n <= m / 2;
+    return P;
+}
+
+// CTA 0: root order of the key-tiled tier: the queued roots (list 4, their
+// wedge counts in list 1) sorted by decreasing wedge count (64 buckets, two
+// per octave) into list 0, and the prefix sums of their in-degrees into list
+// 2. Every other CTA: enc, ends and index.
+__global__ void __launch_bounds__(1024) k_c4_tiled_plan(Graph g, int *lists, int *counters, const int *coff, int ntiles,
+                                                        int words, int *region) {
     pdl_begin();
     __shared__ int hist[64], base[64];
     __shared__ int wsum[32];
+    __shared__ CkZone z[CK_ZONES + 1];
+    __shared__ int glo[CK_MAX_GROUPS];
     if (degree_overflow(counters)) return;
     const int nt = counters[CNT_C4_TEAM];
     if (nt == 0) return;
     const int *roots = lists + 4 * (size_t)g.n, *wts = lists + (size_t)g.n;
+    if (blockIdx.x > 0) {
+        if (threadIdx.x == 0) ck_zones(coff, ntiles, g.n, z);
+        __syncthreads();
+        const CkPlan P = ck_plan(region, z, words, g.n, g.m);
+        if ((int)threadIdx.x < min(P.groups, CK_MAX_GROUPS))
+            glo[threadIdx.x] = ck_low_id(z, (long long)(threadIdx.x + 1) * words);
+        __syncthreads();
+        const int first = z[CK_ZONES].lo;   // rows below have degree 0 or 1
+        const int b = blockIdx.x - 1;
+        const long long t0 = b * (long long)blockDim.x + threadIdx.x, stride = (long long)(gridDim.x - 1) * blockDim.x;
+        for (long long p = t0; p < g.m; p += stride) {
+            const int w = g.ncol[p];
+            int i = 0;
+            while (i < CK_ZONES && w < z[i].lo) ++i;
+            if (i == CK_ZONES) {   // no counter, and below every run of a sorted row
+                P.enc[p] = 0;
+                continue;
+            }
+            const CkZone q = z[i];
+            const unsigned k = (unsigned)(q.hi - 1 - w), per = (unsigned)q.per(), word = k / per;
+            const unsigned at = (unsigned)q.off + word, local = at - at / (unsigned)words * (unsigned)words;
+            P.enc[p] = (int)(local << 12 | (unsigned)(32 - q.bits()) << 5 | (k - word * per) * (unsigned)q.bits());
+        }
+        if (P.indexed)
+            for (int i = 0; i < P.groups; ++i) {
+                const int key = glo[i];
+                for (long long v = first + t0; v < g.n; v += stride) {
+                    const int4 rv = g.rinfo[v];
+                    P.index[(size_t)i * g.n + v] = lower_bound(g.ncol, rv.x, rv.z, key);
+                }
+            }
+        for (int r = b * 4 + (threadIdx.x >> 8); r < nt; r += (gridDim.x - 1) * 4) {   // 256 threads per root
+            const int u = roots[r];
+            const int4 ru = g.rinfo[u];
+            if (ru.y - ru.x > CK_ENDS_MAXD) continue;
+            for (int p = ru.x + (threadIdx.x & 255); p < ru.y; p += 256) {
+                const int4 rv = g.rinfo[g.ncol[p]];
+                P.ends[p] = (unsigned short)min(lower_bound(g.ncol, rv.y, rv.z, u) - rv.y, 65535);
+            }
+        }
+        return;
+    }
     int *sorted = lists, *offs = lists + 2 * (size_t)g.n;
     auto bucket = [](int w) {
         const int e = 31 - __clz(max(w, 1));
@@ -750,265 +871,349 @@ __global__ void __launch_bounds__(1024) k_c4_tiled_plan(Graph g, int *lists, int
     }
 }
 
-// First position p in [cur, end) with a[p] >= key, given a[cur] < key
-// (a ascending): doubling steps from cur, then a binary search.
-__device__ __forceinline__ int gallop(const int *__restrict__ a, int cur, int end, int key) {
-    int lo = cur, step = 1, hi = end;
-    for (;;) {
-        const int pr = lo + step;
-        if (pr >= end) break;
-        if (a[pr] >= key) {
-            hi = pr;
-            break;
-        }
-        lo = pr;
-        step <<= 1;
+// What a CTA keeps in shared memory.
+struct CkShared {
+    unsigned char *cnt;        // a group's counters, and four words that stay 0
+    int *st, *len, *win, *v;   // a batch's listed runs: start, length, first window, vertex
+    int2 *wnd;                 // the warp's 32 windows: first entry, entries
+    int *wwin, *wrun;          // windows and listed runs of every warp's part of the batch
+    CkZone *z;
+    int *any, *job;
+    long long *twice;          // sum of c - 1 over the root's wedges
+    // adds one to / reads the counter of a column entry (see k_c4_tiled_plan:
+    // byte address << 10 | (32 - bits) << 5 | shift; shifts wrap at 32)
+    __device__ __forceinline__ void add(unsigned e) const {
+        atomicAdd(reinterpret_cast<unsigned *>(cnt + (e >> 10)), __funnelshift_l(0u, 1u, e));
     }
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (a[mid] < key) lo = mid; else hi = mid;
+    __device__ __forceinline__ unsigned get(unsigned e) const {
+        const unsigned x = *reinterpret_cast<const unsigned *>(cnt + (e >> 10));
+        const unsigned r = e >> 5;
+        return __funnelshift_r(__funnelshift_l(0u, x, r - e), 0u, r);
     }
-    return hi;
-}
-
-template <bool WIDE>
-struct TileCounts {
-    unsigned *c;
-    __device__ __forceinline__ void add(int k) const {
-        if (WIDE) atomicAdd(&c[k], 1u);
-        else atomicAdd(&c[k >> 1], 1u << ((k & 1) << 4));
-    }
-    __device__ __forceinline__ int get(int k) const {
-        return WIDE ? (int)c[k] : (int)((c[k >> 1] >> ((k & 1) << 4)) & 0xffffu);
-    }
-    static constexpr int keys_per_word = WIDE ? 1 : 2;
 };
 
-// One root of the key-tiled tier, the whole CTA. st: one int4 per
-// in-neighbour {cursor, end of its wedge prefix, offset of its run in the
-// tile's concatenation of runs, key at the cursor}. The offsets are scanned
-// per warp over a contiguous range of R in-neighbours (R a multiple of 32,
-// so a chunk never straddles two ranges); woff[r] turns range r's offsets
-// into offsets in the whole tile.
-template <bool WIDE>
-__device__ __forceinline__ void c4_tiled_root(const Graph &g, VAcc *vacc, int u, int4 *st, unsigned *cnt,
-                                              SegTab *segs, long long *pvs, int *ssm) {
+// Credits C(c, 2) to every key with c >= 2 of the group's stream words
+// [max(gw0, from), to), zone by zone from Z on, and clears the words. Most
+// words of the narrow zones hold no count above 1: four words are tested at
+// once, and only the fields that pass are visited; a word of the wide zones
+// has at most four fields, each taken with constant shifts.
+template <int THREADS, int Z>
+__device__ __forceinline__ void ck_sweep(const CkShared &S, VAcc *vacc, int gw0, int from, int to) {
+    constexpr int BITS = ck_bits(Z), PER = 32 / BITS;
+    constexpr unsigned FIELD = (1u << BITS) - 1u;
+    constexpr unsigned GE2 = [] {   // the bits that are set in some field of 2 or more
+        unsigned m = 0;
+        for (int f = 0; f < PER; ++f) m |= (FIELD - 1u) << (f * BITS);
+        return m;
+    }();
+    const CkZone z = S.z[Z];
+    const int ws = max(max(z.off, gw0), from), we = min(S.z[Z + 1].off, to);
+    for (int s = ws + 4 * (int)threadIdx.x; s < we; s += 4 * THREADS) {
+        uint4 *const at = reinterpret_cast<uint4 *>(S.cnt + 4 * (size_t)(s - gw0));
+        const uint4 x4 = *at;
+        const unsigned some = x4.x | x4.y | x4.z | x4.w;
+        if (!some) continue;
+        *at = make_uint4(0, 0, 0, 0);
+        if (!(some & GE2)) continue;
+        const unsigned xs[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            unsigned m = xs[h] & GE2;
+            if (!m) continue;
+            const int w = z.hi - 1 - (s + h - z.off) * PER;   // key of field 0, the others descend from it
+            VAcc *const p = vacc + w;
+            if constexpr (PER <= 4) {
+#pragma unroll
+                for (int f = 0; f < PER; ++f) {
+                    const unsigned c = (xs[h] >> (f * BITS)) & FIELD;   // below 2^16: c (c - 1) fits 32 bits
+                    if (c >= 2 && w - f >= z.lo) add64(&p[-f].C4, (long long)(c * (c - 1u) / 2u));
+                }
+            } else {
+                while (m) {
+                    const int f = (31 - __clz(m)) / BITS;
+                    m &= ~(FIELD << (f * BITS));
+                    const unsigned c = (xs[h] >> (f * BITS)) & FIELD;
+                    if (w - f >= z.lo) add64(&p[-f].C4, (long long)(c * (c - 1u) / 2u));
+                }
+            }
+        }
+    }
+    if constexpr (Z + 1 < CK_ZONES) ck_sweep<THREADS, Z + 1>(S, vacc, gw0, from, to);
+}
+
+// One root, the whole CTA: the keys below ulim (u, or for a root with
+// c4_wide_top the first id of zone 0).
+template <int THREADS>
+__device__ __forceinline__ void c4_tiled_root(const Graph &g, VAcc *vacc, int u, int ulim, int words, const CkPlan &P,
+                                              const CkShared &S) {
+    constexpr int NW = THREADS / 32, U = CK_UNROLL;
     const int lane = lane_id(), wid = threadIdx.x >> 5;
+    const int *__restrict__ col = g.ncol;
+    const int *__restrict__ enc = P.enc, *__restrict__ encl = P.enc + lane;
+    const unsigned none = (unsigned)words << 12;
+    const int *__restrict__ index = P.index;
     const int4 ru = g.rinfo[u];
     const int b = ru.x, din = ru.y - ru.x;
-    const int nch = (din + 31) >> 5;
-    constexpr int TK = CK_WORDS * TileCounts<WIDE>::keys_per_word;
-    const TileCounts<WIDE> T{cnt};
-    SegTab &seg = segs[wid];
-    long long *pv = pvs + wid * 32;
-    int *woff = ssm, *s_next = ssm + 32, *s_tot = ssm + 33;
-    const int RC = (din + 32 * CK_NW - 1) / (32 * CK_NW), R = RC * 32;   // chunks, in-neighbours per warp range
-    auto offset = [&](int p) { return st[p].z + woff[p / R]; };   // p's run offset in the tile
-    // cursors: each in-neighbour v's wedge prefix [row start, position of u in N+(v))
-    int mn = CK_INF;
-    for (int p = threadIdx.x; p < din; p += CK_THREADS) {
-        const int v = g.ncol[b + p];
-        const int4 rv = g.rinfo[v];
-        const int e = lower_bound(g.ncol, rv.y, rv.z, u);
-        const int nx = rv.x < e ? g.ncol[rv.x] : CK_INF;
-        st[p] = make_int4(rv.x, e, 0, nx);
-        mn = min(mn, nx);
-    }
-    pv[lane] = 0;
-    mn = -warp_max(-mn);
-    if (threadIdx.x == 0) *s_next = CK_INF;
-    __syncthreads();
-    if (lane == 0) atomicMin(s_next, mn);
-    __syncthreads();
-    int lo = *s_next;
+    const int first = S.z[CK_ZONES].lo;
     long long su = 0;
-    // The wedges of elements [e0, e1) of the tile's concatenation of runs,
-    // chunk by chunk of 32 in-neighbours: f(act, q, w) per wedge, done(v)
-    // after each chunk.
-    // Slices by weight: each chunk of 32 in-neighbours counts CK_ALPHA
-    // elements of overhead ahead of its elements (its cursor loads, table
-    // and window setup), so that a slice across many short runs gets fewer
-    // elements. weighted() gives the chunk holding weighted position wp and
-    // the element there.
-    auto weighted = [&](long long wp, int total, long long &e) {
-        int c = 0, top = nch;
-        while (top - c > 1) {
-            const int mid = (c + top) >> 1;
-            if (offset(mid * 32) + (long long)CK_ALPHA * mid <= wp) c = mid; else top = mid;
+    if (ulim <= first) return;
+    int lim_word = 0;   // the stream word of id ulim - 1, the first one the root may use
+    for (int i = 0; i < CK_ZONES; ++i)
+        if (ulim - 1 >= S.z[i].lo) {
+            lim_word = S.z[i].off + (max(S.z[i].hi - ulim, 0)) / S.z[i].per();
+            break;
         }
-        const long long zc = offset(c * 32);
-        const long long zn = c + 1 < nch ? offset((c + 1) * 32) : total;
-        const long long x = wp - zc - (long long)CK_ALPHA * c - CK_ALPHA;
-        e = zc + (x > 0 ? x : 0);
-        if (e > zn) e = zn;
-        return c;
-    };
-    auto visit = [&](long long e0, long long e1, int total, int c0, auto f, auto done) {
-        if (e0 >= e1) return;
-        int c = c0;
-        int r = c / RC, left = RC - (c - r * RC);   // warp range of chunk c, chunks left in it
-        for (; c < nch; ++c) {
-            const int p = c * 32 + lane;
-            int v = -1, cur = 0, end = 0, z = total;
-            if (p < din) {
-                const int4 s4 = st[p];
-                cur = s4.x, end = s4.y, z = s4.z + woff[r];
-                v = g.ncol[b + p];
+    const int g0 = lim_word / words;
+    for (int gi = g0; gi < P.groups; ++gi) {
+        const int glo = P.indexed ? 0 : ck_low_id(S.z, (long long)(gi + 1) * words);
+        const int ghi = P.indexed || gi == g0 ? ulim : ck_low_id(S.z, (long long)gi * words);
+        auto vertex = [&](int e) { return e < din ? col[b + e] : -1; };
+        auto run = [&](int e, int v) {   // {start, end} of the run of in-neighbour e, v
+            if (v < first) return make_int2(0, 0);   // none, or a row of one entry
+            if (P.indexed) {
+                const int x = index[(size_t)gi * g.n + v];
+                if (gi > g0) return make_int2(x, index[(size_t)(gi - 1) * g.n + v]);
+                const int4 rv = g.rinfo[v];
+                if (ulim < u) return make_int2(x, lower_bound(col, x, rv.z, ulim));
+                return make_int2(x, din <= CK_ENDS_MAXD ? rv.y + (int)P.ends[b + e] : lower_bound(col, rv.y, rv.z, u));
             }
-            const int cbase = __shfl_sync(FULL, z, 0);
-            if (cbase >= e1) break;
-            int znext = __shfl_down_sync(FULL, z, 1);
-            if (lane == 31) znext = p + 1 < din ? st[p + 1].z + woff[left == 1 ? r + 1 : r] : total;
-            if (--left == 0) {
-                ++r;
-                left = RC;
-            }
-            // the run, never past the in-neighbour's wedge prefix
-            const int len = p < din ? min(max(znext - z, 0), end - cur) : 0;
-            int pre;
-            const int tot = seg_build(seg, cur, len, pre);
-            const int from = (int)max(e0 - cbase, 0ll), to = (int)min(e1 - cbase, (long long)tot);
-            if (from < to)
-                seg_visit<4, true>(g.ncol, seg, pre, len, to, from, 32, [&](bool ok, int q, int, int w) { f(ok, q, w); });
-            __syncwarp();
-            done(v);
-            __syncwarp();
-        }
-    };
-    while (lo < u) {
-        const int hi = min(lo + TK, u);
-        const int nk = hi - lo;
-        // A. every in-neighbour's run inside [lo, hi) (a galloping search from
-        // its cursor) and the run's offset in the tile's concatenation: each
-        // warp scans its range with a running carry, then one scan of the
-        // warps' totals
-        {
-            int carry = 0;
-            const int r0 = wid * R, r1 = min(r0 + R, din);
-            for (int p0 = r0; p0 < r1; p0 += 32) {
-                const int p = p0 + lane;
-                int len = 0;
-                if (p < r1) {
-                    const int4 s4 = st[p];
-                    if (s4.w < hi) len = gallop(g.ncol, s4.x, s4.y, hi) - s4.x;
+            const int4 rv = g.rinfo[v];
+            const int x = lower_bound(col, rv.x, rv.z, glo);
+            return make_int2(x, lower_bound(col, x, rv.z, ghi));
+        };
+        // One walk over the group's runs. MID: sum c - 1 per run into the
+        // middle vertices; else count.
+        auto walk = [&](auto mid) {
+            constexpr bool MID = decltype(mid)::value;
+            bool any = false;
+            int v = vertex((int)threadIdx.x);
+            int2 r = run((int)threadIdx.x, v);
+            int vn = vertex(THREADS + (int)threadIdx.x);
+            for (int e0 = 0; e0 < din; e0 += THREADS) {
+                const int e = e0 + (int)threadIdx.x;
+                const int len = r.y - r.x;
+                const bool list = len > CK_TINY;
+                // list the batch's longer runs with their first windows
+                const int nwin = list ? (len + 31) >> 5 : 0;
+                const unsigned bal = __ballot_sync(FULL, list);
+                const int incl = warp_inclusive_scan(nwin);
+                if (lane == 31) {
+                    S.wwin[wid] = incl;
+                    S.wrun[wid] = __popc(bal);
                 }
-                const int incl = warp_inclusive_scan(len);
-                if (p < r1) st[p].z = carry + incl - len;
-                carry += __shfl_sync(FULL, incl, 31);
-            }
-            if (lane == 0) woff[wid] = carry;
-            __syncthreads();
-            if (wid == 0) {   // the warps' totals, CK_NW of them
-                const int x = lane < CK_NW ? woff[lane] : 0;
-                const int xi = warp_inclusive_scan(x);
-                if (lane < CK_NW) woff[lane] = xi - x;
-                if (lane == 31) *s_tot = xi;
-            }
-            __syncthreads();
-        }
-        const int total = *s_tot;
-        // every warp takes an equal slice of the tile's weighted wedges (the
-        // same slice for both walks)
-        const long long wt = (long long)total + (long long)CK_ALPHA * nch;
-        long long e0, e1;
-        const int c0 = weighted(wt * wid / CK_NW, total, e0);
-        weighted(wt * (wid + 1) / CK_NW, total, e1);
-        if (wid == CK_NW - 1) e1 = total;
-        // 1. count the tile's wedges
-        visit(e0, e1, total, c0, [&](bool ok, int, int w) {
-            if (ok && (unsigned)(w - lo) < (unsigned)nk) T.add(w - lo);   // always, for a simple graph
-        }, [](int) {});
-        __syncthreads();
-        // 2. C(c, 2) to every key with c >= 2 and to u (the counts are only read from here on)
-        const int nw4 = (nk + 4 * T.keys_per_word - 1) / (4 * T.keys_per_word);
-        for (int i = threadIdx.x; i < nw4; i += CK_THREADS) {
-            const uint4 q = reinterpret_cast<const uint4 *>(cnt)[i];
-            if (!(q.x | q.y | q.z | q.w)) continue;
-            const unsigned qw[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-#pragma unroll
-                for (int h = 0; h < T.keys_per_word; ++h) {
-                    const int c = WIDE ? (int)qw[j] : (int)((qw[j] >> (16 * h)) & 0xffffu);
-                    if (c >= 2) {
-                        const int k = (4 * i + j) * T.keys_per_word + h;
-                        su += c2(c);
-                        add64(&vacc[lo + k].C4, c2(c));
+                __syncthreads();   // and the batch before is done with the list
+                const int tw = lane < NW ? S.wwin[lane] : 0, tr = lane < NW ? S.wrun[lane] : 0;
+                const int iw = warp_inclusive_scan(tw), ir = warp_inclusive_scan(tr);
+                const int total = __shfl_sync(FULL, iw, 31), nlist = __shfl_sync(FULL, ir, 31);
+                const int w0 = __shfl_sync(FULL, iw - tw, wid), q0 = __shfl_sync(FULL, ir - tr, wid);
+                if (list) {
+                    const int q = q0 + __popc(bal & lanemask_lt());
+                    S.st[q] = r.x;
+                    S.len[q] = len;
+                    S.win[q] = w0 + incl - nwin;
+                    S.v[q] = v;
+                }
+                if (len > 0) any = true;
+                if (len > 0 && !list) {
+                    unsigned a = 0;
+                    for (int q = r.x; q < r.y; ++q) {
+                        const unsigned c = (unsigned)__ldg(enc + q);
+                        if (MID) a += S.get(c) - 1u; else S.add(c);
+                    }
+                    if (MID && a) {
+                        add64(&vacc[v].C4, a);
+                        su += a;
                     }
                 }
+                __syncthreads();
+                // the next batch's runs, in flight during this one
+                v = vn;
+                r = run(e + THREADS, v);
+                vn = vertex(e + 2 * THREADS);
+                // this warp's share of the windows, [x, y)
+                const int x = (int)((long long)total * wid / NW);
+                const int y = (int)((long long)total * (wid + 1) / NW);
+                if (x >= y) continue;
+                int q = 0, above = nlist;   // the run that holds window x
+                while (above - q > 1) {
+                    const int m = (q + above) >> 1;
+                    if (S.win[m] <= x) q = m; else above = m;
+                }
+                for (int x0 = x; x0 < y; x0 += 32) {   // 32 windows
+                    const int xl = x0 + lane;
+                    if (q + 1 < nlist && S.win[q + 1] <= x0) ++q;   // the run of window x0
+                    int j = q, ln = 0;   // the run of this lane's window: a run has at least one, so below q + 32
+#pragma unroll
+                    for (int step = 16; step > 0; step >>= 1)
+                        if (j + step < nlist && S.win[j + step] <= xl) j += step;
+                    if (xl < y) {
+                        const int o = (xl - S.win[j]) * 32;
+                        ln = min(32, S.len[j] - o);
+                        S.wnd[lane] = make_int2(S.st[j] + o, ln);
+                    } else {
+                        S.wnd[lane] = make_int2(0, 0);
+                    }
+                    __syncwarp();
+                    const int cnt = min(32, y - x0);
+                    unsigned sum = 0;   // of the lane's window
+                    for (int h0 = 0; h0 < cnt; h0 += U) {
+                        // lanes past a window's end hold `none`, the entry of a counter that stays 0
+                        unsigned c[U];
+#pragma unroll
+                        for (int h = 0; h < U; h += 2) {
+                            const int4 d = *reinterpret_cast<const int4 *>(S.wnd + h0 + h);
+                            c[h] = c[h + 1] = none;
+                            if (lane < d.y) c[h] = (unsigned)__ldg(encl + d.x);
+                            if (lane < d.w) c[h + 1] = (unsigned)__ldg(encl + d.z);
+                        }
+#pragma unroll
+                        for (int h = 0; h < U; ++h) {
+                            if (MID) {
+                                const unsigned t = __reduce_add_sync(FULL, S.get(c[h]));
+                                if (lane == h0 + h) sum = t;
+                            } else if (c[h] != none) {
+                                S.add(c[h]);
+                            }
+                        }
+                    }
+                    if (MID) {
+                        sum -= (unsigned)ln;   // (sums of c - 1 over a root's wedges are below W <= m)
+                        su += sum;
+                        run_add(&vacc[S.v[j]].C4, j, sum);
+                    }
+                    q = __shfl_sync(FULL, j, 31);
+                    __syncwarp();
+                }
             }
-        }
-        // 3. middle vertices: c - 1 per wedge, summed per in-neighbour
-        visit(e0, e1, total, c0, [&](bool ok, int q, int w) {
-            const bool in = ok && (unsigned)(w - lo) < (unsigned)nk;
-            add_middle(pv, q, in ? T.get(w - lo) : 0);
-        }, [&](int v) {
-            const long long x = pv[lane];
-            if (x) add64(&vacc[v].C4, x);
-            pv[lane] = 0;
-        });
-        if (threadIdx.x == 0) *s_next = CK_INF;
+            return any;
+        };
+        if (walk(std::false_type{})) *S.any = 1;   // 1. count
         __syncthreads();
-        // 4. cursors past the runs; the smallest next key starts the next
-        // tile; clear the tile
-        int tnext = CK_INF;
-        for (int p = wid * R + lane; p < min((wid + 1) * R, din); p += 32) {   // the warp's own range
-            const int4 s4 = st[p];
-            const int z = s4.z + woff[wid];
-            const int len = (p + 1 < din ? st[p + 1].z + woff[p + 1 == (wid + 1) * R ? wid + 1 : wid] : total) - z;
-            int nx = s4.w;
-            if (len > 0) {
-                const int cur = s4.x + min(len, s4.y - s4.x);   // never past the wedge prefix
-                nx = cur < s4.y ? g.ncol[cur] : CK_INF;
-                st[p].x = cur;
-                st[p].w = nx;
+        const bool live = *S.any != 0;
+        if (live) {
+            walk(std::true_type{});                // 2. middle vertices: c - 1 per wedge
+            __syncthreads();
+            if (threadIdx.x == 0) *S.any = 0;
+            // 3. C(c, 2) to every key with c >= 2; clear
+            const int gw0 = gi * words;
+            ck_sweep<THREADS, 0>(S, vacc, gw0, lim_word & ~3, gw0 + words);
+        }
+        __syncthreads();
+    }
+    su = warp_sum(su);   // of all warps: sum of c - 1 over the wedges = twice the sum of C(c, 2) over the keys
+    if (lane == 0 && su) add64(S.twice, su);
+    __syncthreads();
+    if (threadIdx.x == 0 && *S.twice) {
+        add64(&vacc[u].C4, *S.twice / 2);
+        *S.twice = 0;
+    }
+}
+
+// The keys of zone 0 (degree 1024 and more) for a root u with so many
+// in-neighbours that a count could pass 16 bits: 32-bit counters, `words` ids
+// at a time, runs found by search, one warp per run. Such a root has 65535
+// in-neighbours or more; a graph has few of them.
+template <int THREADS>
+__device__ __forceinline__ void c4_wide_top(const Graph &g, VAcc *vacc, int u, int words, const CkShared &S) {
+    constexpr int NW = THREADS / 32;
+    const int lane = lane_id(), wid = threadIdx.x >> 5;
+    const int *__restrict__ col = g.ncol;
+    const int4 ru = g.rinfo[u];
+    unsigned *const cnt = reinterpret_cast<unsigned *>(S.cnt);
+    long long su = 0;
+    for (int lo = S.z[0].lo; lo < u; lo += words) {
+        const int nk = min(words, u - lo);
+        auto walk = [&](auto mid) {
+            constexpr bool MID = decltype(mid)::value;
+            for (int p0 = ru.x + 32 * wid; p0 < ru.y; p0 += 32 * NW) {
+                const int v = p0 + lane < ru.y ? col[p0 + lane] : -1;
+                int st = 0, ln = 0;
+                if (v >= 0) {
+                    const int4 rv = g.rinfo[v];
+                    st = lower_bound(col, rv.x, rv.z, lo);
+                    ln = lower_bound(col, st, rv.z, lo + nk) - st;
+                }
+                unsigned acc = 0;   // below W <= m
+                for (unsigned m = __ballot_sync(FULL, ln > 0); m; m &= m - 1) {
+                    const int j = __ffs(m) - 1, js = __shfl_sync(FULL, st, j), jl = __shfl_sync(FULL, ln, j);
+                    unsigned a = 0;
+                    for (int o = lane; o < jl; o += 32) {
+                        const unsigned k = (unsigned)(__ldg(col + js + o) - lo);
+                        if (k >= (unsigned)nk) continue;   // never, for sorted rows
+                        if (MID) a += cnt[k] - 1u; else atomicAdd(&cnt[k], 1u);
+                    }
+                    if (MID) {
+                        a = __reduce_add_sync(FULL, a);
+                        if (lane == j) acc = a;
+                    }
+                }
+                if (MID && acc) add64(&vacc[v].C4, acc);
             }
-            tnext = min(tnext, nx);
+            __syncthreads();
+        };
+        walk(std::false_type{});
+        walk(std::true_type{});
+        for (int k = threadIdx.x; k < nk; k += THREADS) {
+            const long long cc = c2((long long)cnt[k]);
+            cnt[k] = 0;
+            if (cc) add64(&vacc[lo + k].C4, cc);
+            su += cc;
         }
-        tnext = -warp_max(-tnext);
-        if (lane == 0 && tnext < CK_INF) atomicMin(s_next, tnext);
-        for (int i = threadIdx.x; i < nw4; i += CK_THREADS) reinterpret_cast<uint4 *>(cnt)[i] = make_uint4(0, 0, 0, 0);
-        __syncthreads();
-        lo = *s_next;
         __syncthreads();
     }
     su = warp_sum(su);
     if (lane == 0 && su) add64(&vacc[u].C4, su);
-    __syncthreads();
 }
 
-// cursors: room for `cap` entries; a list of roots whose in-degrees sum to
-// more (only for a CSR that is not symmetric) stops with ENOTSIMPLE.
-__global__ void __launch_bounds__(CK_THREADS) k_c4_tiled(Graph g, VAcc *vacc, const int *lists, int *counters,
-                                                         int4 *cursors, long long cap, int *status) {
+// Roots from the work queue. The prefix sums of the roots' in-degrees pass
+// m / 2 only for a CSR that is not symmetric: such a root stops with
+// ENOTSIMPLE.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1)
+    k_c4_tiled(Graph g, VAcc *vacc, const int *lists, int *counters, const int *coff, int ntiles, int words, int *region,
+               int *status) {
     pdl_begin();
     extern __shared__ __align__(16) unsigned char dsm[];
-    unsigned *cnt = reinterpret_cast<unsigned *>(dsm);
-    SegTab *segs = reinterpret_cast<SegTab *>(cnt + CK_WORDS);
-    long long *pvs = reinterpret_cast<long long *>(segs + CK_NW);
-    int *ssm = reinterpret_cast<int *>(pvs + CK_NW * 32);   // scan partials, next key, run total
-    int *s_job = ssm + 40;
+    CkShared S;
+    S.cnt = dsm;
+    S.z = reinterpret_cast<CkZone *>(dsm + 4 * (size_t)words + 16);
+    S.st = reinterpret_cast<int *>(S.z + CK_ZONES + 1);   // (16-byte aligned, like S.wnd)
+    S.len = S.st + THREADS;
+    S.win = S.len + THREADS;
+    S.v = S.win + THREADS;
+    S.wnd = reinterpret_cast<int2 *>(S.v + THREADS) + (threadIdx.x & ~31u);
+    S.wwin = S.v + 3 * THREADS;
+    S.wrun = S.wwin + THREADS / 32;
+    S.any = S.wrun + THREADS / 32;
+    S.job = S.any + 1;
+    S.twice = reinterpret_cast<long long *>(S.any + 2);
     if (degree_overflow(counters)) return;
     const int nt = counters[CNT_C4_TEAM];
     if (nt == 0) return;
     const int *sorted = lists, *offs = lists + 2 * (size_t)g.n;
-    for (int i = threadIdx.x; i < CK_WORDS / 4; i += CK_THREADS)
-        reinterpret_cast<uint4 *>(cnt)[i] = make_uint4(0, 0, 0, 0);
+    for (int i = threadIdx.x; i <= words / 4; i += THREADS) reinterpret_cast<uint4 *>(S.cnt)[i] = make_uint4(0, 0, 0, 0);
+    if (threadIdx.x == 0) {
+        ck_zones(coff, ntiles, g.n, S.z);
+        *S.any = 0;
+        *S.twice = 0;
+    }
+    __syncthreads();
+    const CkPlan P = ck_plan(region, S.z, words, g.n, g.m);
     for (;;) {
         __syncthreads();
-        if (threadIdx.x == 0) *s_job = atomicAdd(&counters[CNT_C4_TILED_NEXT], 1);
+        if (threadIdx.x == 0) *S.job = atomicAdd(&counters[CNT_C4_TILED_NEXT], 1);
         __syncthreads();
-        const int j = *s_job;
+        const int j = *S.job;
         if (j >= nt) break;
         const int u = sorted[j];
         const int4 ru = g.rinfo[u];
-        if ((long long)offs[j] + (ru.y - ru.x) > cap || offs[j] < 0) {
+        if ((long long)offs[j] + (ru.y - ru.x) > g.m / 2 || offs[j] < 0) {
             if (threadIdx.x == 0) set_status(status, ST_ENOTSIMPLE);
             continue;
         }
-        int4 *st = cursors + offs[j];
-        if (ru.y - ru.x <= CK_NARROW_MAXD) c4_tiled_root<false>(g, vacc, u, st, cnt, segs, pvs, ssm);
-        else c4_tiled_root<true>(g, vacc, u, st, cnt, segs, pvs, ssm);
+        const bool wide = ru.y - ru.x > CK_NARROW_MAXD;
+        if (wide) c4_wide_top<THREADS>(g, vacc, u, words, S);
+        c4_tiled_root<THREADS>(g, vacc, u, wide ? min(u, S.z[0].lo) : u, words, P, S);
     }
 }
 
@@ -1063,12 +1268,20 @@ void launch_cycle4(Work &w, cudaStream_t st) {
     after_launch(st, K_C4_MID);
     launch_pdl(k_c4_cta, w.num_sms * occ_c, CC_THREADS, CC_SMEM, st, g, w.vacc, w.lists, w.counters, cb);
     after_launch(st, K_C4_CTA);
-    launch_pdl(k_c4_tiled_plan, 1, 1024, 0, st, g, w.lists, w.counters);
+    const bool small = w.n <= CK_SMALL_N;
+    const int words = small ? (w.n / 2 + 4 * CK_ZONES + 4) & ~3 : CK_WORDS;
+    launch_pdl(k_c4_tiled_plan, 1 + min(2 * w.num_sms, w.m / 4096 + 1), 1024, 0, st, g, w.lists, w.counters, w.coff, w.ntiles, words,
+               w.tcnt);
     after_launch(st, K_C4_PLAN);
-    static const int occ_t = resident_ctas((const void *)k_c4_tiled, CK_THREADS, CK_SMEM);
-    launch_pdl(k_c4_tiled, w.num_sms * occ_t, CK_THREADS, CK_SMEM, st, g, w.vacc, w.lists, w.counters,
-                                                      reinterpret_cast<int4 *>(w.tcnt), (long long)w.m / 2,
-                                                      w.status);
+    if (small) {
+        const size_t smem = ck_smem(256, words);
+        const int occ = (int)min((size_t)4, (size_t)(227 * 1024) / (smem + 1024));
+        launch_pdl(k_c4_tiled<256>, w.num_sms * occ, 256, smem, st, g, w.vacc, w.lists, w.counters, w.coff, w.ntiles, words,
+                   w.tcnt, w.status);
+    } else {
+        launch_pdl(k_c4_tiled<1024>, w.num_sms, 1024, ck_smem(1024, words), st, g, w.vacc, w.lists, w.counters, w.coff,
+                   w.ntiles, words, w.tcnt, w.status);
+    }
     after_launch(st, K_C4_TILED);
 }
 
@@ -1080,7 +1293,10 @@ void configure_cycle4() {
     cudaFuncSetAttribute(k_c4_warp_big_split, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     cudaFuncSetAttribute(k_c4_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CM_SMEM);
     cudaFuncSetAttribute(k_c4_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CC_SMEM);
-    cudaFuncSetAttribute(k_c4_tiled, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CK_SMEM);
+    cudaFuncSetAttribute(k_c4_tiled<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ck_smem(256, CK_SMALL_N / 2 + 64));
+    cudaFuncSetAttribute(k_c4_tiled<256>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    cudaFuncSetAttribute(k_c4_tiled<1024>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    cudaFuncSetAttribute(k_c4_tiled<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ck_smem(1024, CK_WORDS));
 }
 
 }  // namespace niorca
