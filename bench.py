@@ -128,7 +128,14 @@ class Shape:
         warp = live & ~hub & (w <= warp_lim)
         wbig = live & ~hub & ~warp & (w <= big_lim)
         rest = live & ~warp & ~wbig
-        team = rest & ((w > C4_CTA_MAXW) | hub)
+        # counters of the key-tiled tier: words per zone of degrees, a CTA holds 48K of them
+        words = 0
+        for lo, hi, bits in ((1024, None, 16), (256, 1024, 10), (64, 256, 8), (32, 64, 6), (16, 32, 5), (8, 16, 4),
+                             (4, 8, 3), (2, 4, 2)):
+            ids = int(((self.d >= lo) & (self.d < (hi or 1 << 62))).sum())
+            words += (-(-ids // (32 // bits)) + 3) & ~3
+        min_team = C4_MID_MAXW if words <= 48 << 10 else 2 * C4_MID_MAXW if words <= 192 << 10 else C4_CTA_MAXW
+        team = rest & ((w > min_team) | hub)
         midp = rest & ~team & (w <= 2 * C4_MID_MAXW) & (w <= pack_lim)
         mid = rest & ~team & ~midp & (w <= C4_MID_MAXW)
         cta = rest & ~team & ~midp & ~mid
@@ -220,7 +227,7 @@ def algorithmic_bytes(rowptr: np.ndarray, colidx: np.ndarray, c4_warp_ub: int = 
            "B_c4": 4 * w_c4, "W_c4": w_c4, "B_out": 120 * n, "tri_probes": b_tri // 4,
            "k4_pairs_checked": k4_pairs, "triangles": ntri}
     per_kernel = {"k_tri_warp": b_tri - b_tri_cta - b_tri_big, "k_tri_cta": b_tri_cta, "k_tri_big": b_tri_big,
-                  "k_relabel_rows_warp": 2 * res["B_csr"], "k_solve": res["B_csr"] + res["B_out"]}
+                  "k_relabel_rows": 2 * res["B_csr"], "k_solve": res["B_csr"] + res["B_out"]}
     for k, msk in sh.c4_tiers(c4_warp_ub).items():
         per_kernel[k] = 4 * int(sh.w_root[msk].sum())
     per_kernel["k_c4_mid"] += per_kernel.pop("k_c4_midp")   # one kernel takes both 128-thread queues

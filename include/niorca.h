@@ -226,7 +226,8 @@ int32_t niorca_version(void);
  *         out-neighbourhood in shared memory; above it, binary searches
  *         (2..8192; default 8192)
  *   10    4-cycle roots with more wedges than this are counted by the
- *         key-tiled tier (2..12288; default 12288)
+ *         key-tiled tier (2..12288; default 12288; graphs whose counters fit
+ *         few shared-memory groups send roots from 3072 or 6144 wedges there)
  * Any setting gives the same counts; only the speed changes. Returns
  * NIORCA_EINVAL (and changes nothing) for a value out of range.
  * niorca_get_tuning copies the current values and returns how many exist.

@@ -81,23 +81,28 @@ __device__ __forceinline__ int2 wedge_seg(const Graph &g, int u, int din, int p)
 
 // The wedge segment of every in-entry of the rows with at most WL_MAXD
 // in-neighbours, a group of L lanes per row (16, or 8 for graphs of mean
-// degree below 16): the row gather and binary search of each entry, made
-// here with every thread independent, so that the per-root kernels read one
-// coalesced 8-byte entry per in-neighbour.
+// degree below 16), a CTA per row from degree WL_LONG on (first, so that no
+// group walks a long row alone: R-MAT of 4610 vertices 129 -> 13 us): the row
+// gather and binary search of each entry, made here with every thread
+// independent, so that the per-root kernels read one coalesced 8-byte entry
+// per in-neighbour.
+constexpr int WL_LONG = 128;
 template <int L>
-__global__ void __launch_bounds__(256, 8) k_c4_wedge_len(Graph g, int2 *wl, const int *counters) {
+__global__ void __launch_bounds__(256, 8) k_c4_wedge_len(Graph g, int2 *wl, const int *counters, const int *coff, int ntiles) {
     pdl_begin();
     if (degree_overflow(counters)) return;
-    const int hl = threadIdx.x & (L - 1);
-    const int gh = (blockIdx.x * blockDim.x + threadIdx.x) / L, nh = (gridDim.x * blockDim.x) / L;
-    for (int u = gh; u < g.n; u += nh) {
+    auto row = [&](int u, int first, int stride) {
         const int4 ru = g.rinfo[u];
-        if (ru.y - ru.x > WL_MAXD) continue;
-        for (int p = ru.x + hl; p < ru.y; p += L) {
+        if (ru.y - ru.x > WL_MAXD) return;
+        for (int p = ru.x + first; p < ru.y; p += stride) {
             const int4 rv = g.rinfo[g.ncol[p]];
             wl[p] = make_int2(rv.x, wedge_len(g, u, rv));
         }
-    }
+    };
+    const int bound = min(coff[deg_class(WL_LONG) * ntiles], g.n);
+    for (int u = bound + blockIdx.x; u < g.n; u += gridDim.x) row(u, threadIdx.x, blockDim.x);
+    const int gh = (blockIdx.x * blockDim.x + threadIdx.x) / L, nh = (gridDim.x * blockDim.x) / L;
+    for (int u = gh; u < bound; u += nh) row(u, threadIdx.x & (L - 1), L);
 }
 
 // Segment table of in-neighbour chunk cb of root u in the calling warp: the
@@ -431,6 +436,61 @@ __device__ __forceinline__ void c4_root(const Graph &g, VAcc *vacc, int u, int b
 }
 
 
+// ------------------------------- counter layout of the key-tiled tier (below)
+
+constexpr int CK_WORDS = 48 * 1024;   // counter words of a 1024-thread CTA
+constexpr int CK_ZONES = 8;
+
+// Counter widths of the zones.
+__host__ __device__ constexpr int ck_bits(int zone) {
+    return zone == 0 ? 16 : zone == 1 ? 10 : zone == 2 ? 8 : 8 - zone + 1;
+}
+
+// Zone z: ids [lo, hi), `per` counters of `bits` bits in a word, stream words
+// from `off` on (a multiple of 4). Id w has word off + (hi - 1 - w) / per and
+// field (hi - 1 - w) % per. Zones run from the highest ids down.
+struct __align__(16) CkZone {
+    int lo, hi, off, fmt;
+    __device__ __forceinline__ int per() const { return fmt & 0xff; }
+    __device__ __forceinline__ int bits() const { return fmt >> 8; }
+};
+
+// The zones, from the first id of the class of each zone's lowest degree;
+// z[CK_ZONES].off is the length of the stream. One thread.
+__device__ __forceinline__ void ck_zones(const int *coff, int ntiles, int n, CkZone *z) {
+    const int deg[CK_ZONES] = {1024, 256, 64, 32, 16, 8, 4, 2};
+    int hi = n, off = 0;
+#pragma unroll
+    for (int i = 0; i < CK_ZONES; ++i) {
+        CkZone q;
+        q.hi = hi;
+        q.lo = min(coff[deg_class(deg[i]) * ntiles], hi);
+        q.off = off;
+        const int bits = ck_bits(i), per = 32 / bits;
+        q.fmt = per | bits << 8;
+        off += ((hi - q.lo + per - 1) / per + 3) & ~3;
+        hi = q.lo;
+        z[i] = q;
+    }
+    z[CK_ZONES].lo = z[CK_ZONES].hi = hi;
+    z[CK_ZONES].off = off;
+    z[CK_ZONES].fmt = 1;
+}
+
+// Wedges from which a root goes to the key-tiled tier. A root there costs
+// passes over its in-neighbours and over the counters for every group of
+// them, but it has a CTA to itself with no hash: with one group it takes
+// roots that the 128-thread tier walks for tens of microseconds (power-law
+// graph of 1e5 vertices: call 585 us from 12288 wedges on, 519 from 6144, 477
+// from 3072), with many it pays only for the largest (R-MAT 22, six groups:
+// 228 ms from 12288 on, 235 from 6144).
+__device__ __forceinline__ int ck_min_wedges(const int *coff, int ntiles, int n, int most) {
+    CkZone z[CK_ZONES + 1];
+    ck_zones(coff, ntiles, n, z);
+    const int words = z[CK_ZONES].off;
+    return words <= CK_WORDS ? min(most, CM_MAXW) : words <= 4 * CK_WORDS ? min(most, 2 * CM_MAXW) : most;
+}
+
 template <int WORDS>
 struct __align__(16) C4WarpSmem {
     unsigned t[WORDS];
@@ -451,8 +511,9 @@ __host__ __device__ constexpr int cw_maxw(bool split, int words) { return cw_slo
 // whose ids leave a packed word too few count bits.
 template <bool SPLIT, bool BIG>
 __device__ __forceinline__ void c4_warp_body(Graph g, VAcc *vacc, int *lists, int *counters, int maxw, int cb,
-                                             int teamw) {
+                                             int teamw, const int *coff, int ntiles) {
     if (degree_overflow(counters)) return;
+    if (!BIG) teamw = ck_min_wedges(coff, ntiles, g.n, teamw);
     constexpr int WORDS = BIG ? CWB_WORDS : CW_WORDS;
     constexpr int TS = cw_slots(SPLIT, WORDS);
     __shared__ C4WarpSmem<WORDS> sm_all[CW_WARPS];
@@ -569,27 +630,27 @@ __device__ __forceinline__ void c4_warp_body(Graph g, VAcc *vacc, int *lists, in
 
 // 8 CTAs of 4 warps per SM: 6 KB tables and at most 64 registers a thread.
 __global__ void __launch_bounds__(CW_WARPS * 32, 8) k_c4_warp(Graph g, VAcc *vacc, int *lists, int *counters,
-                                                              int maxw, int cb, int teamw) {
+                                                              int maxw, int cb, int teamw, const int *coff, int ntiles) {
     pdl_begin();
-    c4_warp_body<false, false>(g, vacc, lists, counters, maxw, cb, teamw);
+    c4_warp_body<false, false>(g, vacc, lists, counters, maxw, cb, teamw, coff, ntiles);
 }
 
 __global__ void __launch_bounds__(CW_WARPS * 32, 8) k_c4_warp_split(Graph g, VAcc *vacc, int *lists,
-                                                                    int *counters, int maxw, int cb, int teamw) {
+                                                                    int *counters, int maxw, int cb, int teamw, const int *coff, int ntiles) {
     pdl_begin();
-    c4_warp_body<true, false>(g, vacc, lists, counters, maxw, cb, teamw);
+    c4_warp_body<true, false>(g, vacc, lists, counters, maxw, cb, teamw, coff, ntiles);
 }
 
 __global__ void __launch_bounds__(CW_WARPS * 32) k_c4_warp_big(Graph g, VAcc *vacc, int *lists, int *counters,
-                                                               int maxw, int cb, int teamw) {
+                                                               int maxw, int cb, int teamw, const int *coff, int ntiles) {
     pdl_begin();
-    c4_warp_body<false, true>(g, vacc, lists, counters, maxw, cb, teamw);
+    c4_warp_body<false, true>(g, vacc, lists, counters, maxw, cb, teamw, coff, ntiles);
 }
 
 __global__ void __launch_bounds__(CW_WARPS * 32) k_c4_warp_big_split(Graph g, VAcc *vacc, int *lists,
-                                                                     int *counters, int maxw, int cb, int teamw) {
+                                                                     int *counters, int maxw, int cb, int teamw, const int *coff, int ntiles) {
     pdl_begin();
-    c4_warp_body<true, true>(g, vacc, lists, counters, maxw, cb, teamw);
+    c4_warp_body<true, true>(g, vacc, lists, counters, maxw, cb, teamw, coff, ntiles);
 }
 
 // Roots from a queue, one CTA each. The table (SLOTS split slots, or
@@ -698,53 +759,15 @@ __global__ void __launch_bounds__(CC_THREADS) k_c4_cta(Graph g, VAcc *vacc, cons
 // twice the time (every group passes over all in-neighbours).
 constexpr int CK_TINY = 4;
 constexpr int CK_NARROW_MAXD = 65534;               // in-degree up to which 16-bit counters cannot overflow
-constexpr int CK_WORDS = 48 * 1024;                 // counter words of a 1024-thread CTA
 constexpr int CK_SMALL_N = 12288;                   // graphs whose 16-bit counters fit 24 KB: 256-thread CTAs
 constexpr int CK_MAX_GROUPS = 64;                   // groups up to which there may be an index
 constexpr int CK_ENDS_MAXD = 8192;                  // in-degree of a root up to which `ends` holds its positions
 constexpr int CK_UNROLL = 16;                       // windows a warp has in flight (R-MAT 22: 125 ms with 8)
-constexpr int CK_ZONES = 8;
 constexpr size_t ck_smem(int threads, int words) {
     // counters; per thread: run start, length, window prefix, vertex and a window; warp totals, zones, scalars
     return (size_t)words * 4 + (size_t)threads * 24 + (size_t)(threads / 32) * 8 + (CK_ZONES + 1) * 16 + 32;
 }
 static_assert(ck_smem(1024, CK_WORDS) <= 227 * 1024, "k_c4_tiled shared memory");
-
-// Counter widths of the zones.
-__host__ __device__ constexpr int ck_bits(int zone) {
-    return zone == 0 ? 16 : zone == 1 ? 10 : zone == 2 ? 8 : 8 - zone + 1;
-}
-
-// Zone z: ids [lo, hi), `per` counters of `bits` bits in a word, stream words
-// from `off` on (a multiple of 4). Id w has word off + (hi - 1 - w) / per and
-// field (hi - 1 - w) % per. Zones run from the highest ids down.
-struct __align__(16) CkZone {
-    int lo, hi, off, fmt;
-    __device__ __forceinline__ int per() const { return fmt & 0xff; }
-    __device__ __forceinline__ int bits() const { return fmt >> 8; }
-};
-
-// The zones, from the first id of the class of each zone's lowest degree;
-// z[CK_ZONES].off is the length of the stream. One thread.
-__device__ __forceinline__ void ck_zones(const int *coff, int ntiles, int n, CkZone *z) {
-    const int deg[CK_ZONES] = {1024, 256, 64, 32, 16, 8, 4, 2};
-    int hi = n, off = 0;
-#pragma unroll
-    for (int i = 0; i < CK_ZONES; ++i) {
-        CkZone q;
-        q.hi = hi;
-        q.lo = min(coff[deg_class(deg[i]) * ntiles], hi);
-        q.off = off;
-        const int bits = ck_bits(i), per = 32 / bits;
-        q.fmt = per | bits << 8;
-        off += ((hi - q.lo + per - 1) / per + 3) & ~3;
-        hi = q.lo;
-        z[i] = q;
-    }
-    z[CK_ZONES].lo = z[CK_ZONES].hi = hi;
-    z[CK_ZONES].off = off;
-    z[CK_ZONES].fmt = 1;
-}
 
 // Lowest id with a counter before stream word e.
 __device__ __forceinline__ int ck_low_id(const CkZone *z, long long e) {
@@ -1229,8 +1252,8 @@ void launch_cycle4(Work &w, cudaStream_t st) {
     // the wedge segments take the region of the triangle counts, dead after the aggregate stage
     int2 *wl = reinterpret_cast<int2 *>(w.tcnt);
     Graph g{w.n, w.m, w.rinfo, w.ncol, wl};
-    if ((long long)w.m < 16ll * w.n) launch_pdl(k_c4_wedge_len<8>, w.num_sms * 8, 256, 0, st, g, wl, w.counters);
-    else launch_pdl(k_c4_wedge_len<16>, w.num_sms * 8, 256, 0, st, g, wl, w.counters);
+    if ((long long)w.m < 16ll * w.n) launch_pdl(k_c4_wedge_len<8>, w.num_sms * 8, 256, 0, st, g, wl, w.counters, w.coff, w.ntiles);
+    else launch_pdl(k_c4_wedge_len<16>, w.num_sms * 8, 256, 0, st, g, wl, w.counters, w.coff, w.ntiles);
     after_launch(st, K_C4_WEDGE_LEN);
     int maxw = w.tune[TUNE_C4_WARP_MAXW] < CW_MAXW ? w.tune[TUNE_C4_WARP_MAXW] : CW_MAXW;
     // A graph with fewer vertices than the warp tier has resident warps is
@@ -1249,25 +1272,31 @@ void launch_cycle4(Work &w, cudaStream_t st) {
     static const int occ_b = resident_ctas((const void *)k_c4_warp_big, CW_WARPS * 32, 0);
     static const int occ_bs = resident_ctas((const void *)k_c4_warp_big_split, CW_WARPS * 32, 0);
     if (packed)
-        launch_pdl(k_c4_warp, w.num_sms * min(w.tune[TUNE_GRID_C4], occ_w), CW_WARPS * 32, 0, st, g, w.vacc, w.lists, w.counters, maxw,
-                                                                             cb, teamw);
+        launch_pdl(k_c4_warp, w.num_sms * min(w.tune[TUNE_GRID_C4], occ_w), CW_WARPS * 32, 0, st, g, w.vacc, w.lists,
+                   w.counters, maxw, cb, teamw, w.coff, w.ntiles);
     else
-        launch_pdl(k_c4_warp_split, w.num_sms * min(w.tune[TUNE_GRID_C4], occ_ws), CW_WARPS * 32, 0, st, g, w.vacc, w.lists, w.counters,
-                                                                                   maxw, cb, teamw);
+        launch_pdl(k_c4_warp_split, w.num_sms * min(w.tune[TUNE_GRID_C4], occ_ws), CW_WARPS * 32, 0, st, g, w.vacc, w.lists,
+                   w.counters, maxw, cb, teamw, w.coff, w.ntiles);
     after_launch(st, K_C4_WARP);
-    // roots k_c4_warp queued for the 8 KB tables: one resident wave
-    if (packed)
-        launch_pdl(k_c4_warp_big, w.num_sms * occ_b, CW_WARPS * 32, 0, st, g, w.vacc, w.lists, w.counters, maxw, cb, teamw);
-    else
-        launch_pdl(k_c4_warp_big_split, w.num_sms * occ_bs, CW_WARPS * 32, 0, st, g, w.vacc, w.lists, w.counters, maxw, cb,
-                                                                     teamw);
-    after_launch(st, K_C4_WARP_BIG);
+    // roots k_c4_warp queued for the 8 KB tables: one resident wave (none when it keeps all it may)
+    if (maxw > cw_maxw(!packed, CW_WORDS)) {
+        if (packed)
+            launch_pdl(k_c4_warp_big, w.num_sms * occ_b, CW_WARPS * 32, 0, st, g, w.vacc, w.lists, w.counters, maxw, cb, teamw,
+                       w.coff, w.ntiles);
+        else
+            launch_pdl(k_c4_warp_big_split, w.num_sms * occ_bs, CW_WARPS * 32, 0, st, g, w.vacc, w.lists, w.counters, maxw,
+                       cb, teamw, w.coff, w.ntiles);
+        after_launch(st, K_C4_WARP_BIG);
+    }
     static const int occ_m = resident_ctas((const void *)k_c4_mid, CM_THREADS, CM_SMEM);
     static const int occ_c = resident_ctas((const void *)k_c4_cta, CC_THREADS, CC_SMEM);
     launch_pdl(k_c4_mid, w.num_sms * occ_m, CM_THREADS, CM_SMEM, st, g, w.vacc, w.lists, w.counters, cb);
     after_launch(st, K_C4_MID);
-    launch_pdl(k_c4_cta, w.num_sms * occ_c, CC_THREADS, CC_SMEM, st, g, w.vacc, w.lists, w.counters, cb);
-    after_launch(st, K_C4_CTA);
+    // (a graph whose counters surely are one group has no root between the 128-thread tier and the key-tiled one)
+    if (w.n / 2 + 4 * CK_ZONES > CK_WORDS) {
+        launch_pdl(k_c4_cta, w.num_sms * occ_c, CC_THREADS, CC_SMEM, st, g, w.vacc, w.lists, w.counters, cb);
+        after_launch(st, K_C4_CTA);
+    }
     const bool small = w.n <= CK_SMALL_N;
     const int words = small ? (w.n / 2 + 4 * CK_ZONES + 4) & ~3 : CK_WORDS;
     launch_pdl(k_c4_tiled_plan, 1 + min(2 * w.num_sms, w.m / 4096 + 1), 1024, 0, st, g, w.lists, w.counters, w.coff, w.ntiles, words,

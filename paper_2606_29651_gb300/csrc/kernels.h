@@ -2,7 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
-#include "common.cuh"
+#include "adj.cuh"
 
 namespace niorca {
 
@@ -55,7 +55,11 @@ enum TuneIndex {
 enum { CNT_TRI_HEAVY = 0, CNT_AGG_HEAVY = 1, CNT_C4_CTA = 2, CNT_C4_TEAM = 3, CNT_DMAX = 4, CNT_C4_MID = 5,
        CNT_C4_MIDP = 6, CNT_TRI_BIG = 7, CNT_AGG_BIG = 8, CNT_C4_WBIG = 9, CNT_C4_TILED_NEXT = 10,
        CNT_TRI_CTA_NEXT = 11, CNT_TRI_BIG_NEXT = 12, CNT_AGG_CTA_NEXT = 13, CNT_AGG_BIG_NEXT = 14,
-       CNT_C4_MID_NEXT = 15, CNT_C4_MIDP_NEXT = 16, CNT_C4_CTA_NEXT = 17, NCOUNTERS = 32 };
+       CNT_C4_MID_NEXT = 15, CNT_C4_MIDP_NEXT = 16, CNT_C4_CTA_NEXT = 17,
+       CNT_BAD_ROWS = 18,   // a row is not strictly increasing, or out of range (recorded in the status too)
+       CNT_ADJ_ON = 19,     // the triangle and aggregate stages probe the adjacency bitmap (AdjBits)
+       CNT_SCAN_DONE = 20,  // blocks of a scan's first pass that are done (0 between scans)
+       NCOUNTERS = 32 };
 
 // The next item of a work queue, for the whole CTA: thread 0 takes it from
 // the queue's counter, every thread returns the same index.
@@ -111,10 +115,23 @@ constexpr int SCAN_TILE = 4096;      // elements per scan block
 constexpr int LONG_ROW_CLASS = 32;   // deg_class(512): rows from here on get a CTA each
 
 size_t scan_partials(long long len);
-void launch_exclusive_scan(const int *in, int *out, long long len, bool write_total, int *part,
+// `done`: a counter that is 0 (and is again afterwards)
+void launch_exclusive_scan(const int *in, int *out, long long len, bool write_total, int *part, int *done,
                            cudaStream_t st);
 
 void launch_relabel(const int *rowptr, const int *colidx, Work &w, cudaStream_t st);
+// The adjacency bitmap of a call (see AdjBits), over the second half of the
+// triangle-count region, which is unused until the 4-cycle stage.
+AdjBits adj_bits(const Work &w);
+// Small graphs have none: their triangle stage takes a few microseconds either
+// way, as much as the launch that builds it (G(3213, mean degree 31): 110 us a
+// call without, 120 with), except dense ones (G(387, 0.53): 561 us without,
+// 410 with).
+inline bool adj_wanted(int n, int m) { return m >= 1 << 17 || (m >= 1 << 14 && m >= 64ll * n); }
+// Whether a graph of m entries may have an out-degree above d: u's d+
+// out-neighbours have u's degree class at least, so degrees of 4/5 of u's and
+// more, and all degrees sum to m: 0.8 (d+)^2 <= m.
+inline bool out_degree_above(int d, int m) { return (long long)d * d * 4 < 5ll * m; }
 void launch_stage1(Work &w, cudaStream_t st);
 void launch_stage2(Work &w, cudaStream_t st);
 void launch_cycle4(Work &w, cudaStream_t st);
@@ -124,9 +141,9 @@ void launch_validate(const int *rowptr, const int *colidx, int n, int m, int *st
 
 // Kernel ids for the optional per-kernel event timing and launch counting.
 enum KernelId {
-    K_CLASS_HIST, K_SCAN, K_CLASS_SCATTER, K_RELABEL_WARP, K_RELABEL_CTA, K_BATCH_SETUP,
+    K_CLASS_HIST, K_SCAN, K_CLASS_SCATTER, K_RELABEL, K_BATCH_SETUP,
     K_TRI_WARP, K_TRI_CTA, K_AGG_WARP, K_AGG_CTA, K_C4_WARP, K_C4_CTA, K_C4_PLAN, K_C4_TILED,
-    K_SOLVE, K_VALIDATE, K_C4_MID, K_TRI_BIG, K_AGG_BIG, K_C4_WARP_BIG, K_C4_WEDGE_LEN, K_COUNT
+    K_SOLVE, K_VALIDATE, K_C4_MID, K_TRI_BIG, K_AGG_BIG, K_C4_WARP_BIG, K_C4_WEDGE_LEN, K_ADJ_BITS, K_COUNT
 };
 const char *kernel_name(int id);
 

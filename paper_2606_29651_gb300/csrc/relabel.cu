@@ -40,10 +40,13 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *wsum, int *total
     return r;
 }
 
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_reduce(const int *in, long long len, int *part) {
+// Sums of the tiles; the block that finishes last scans them (no block waits
+// for another).
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_reduce(const int *in, long long len, int *part, int *done) {
     pdl_begin();
     __shared__ int wsum[32];
     __shared__ int tot;
+    __shared__ bool last;
     const long long base = (long long)blockIdx.x * SCAN_TILE;
     int s = 0;
     for (int i = threadIdx.x; i < SCAN_TILE; i += SCAN_THREADS) {
@@ -51,23 +54,38 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_reduce(const int *in, lon
         if (g < len) s += in[g];
     }
     block_exclusive_scan(s, wsum, &tot);
-    if (threadIdx.x == 0) part[blockIdx.x] = tot;
-}
-
-__global__ void __launch_bounds__(1024) k_scan_top(int *part, int nblocks) {
-    pdl_begin();
-    __shared__ int wsum[32];
-    __shared__ int tot;
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = tot;
+        __threadfence();
+        last = atomicAdd(done, 1) == (int)gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int nblocks = gridDim.x;
+    volatile int *vp = part;
     int carry = 0;
-    for (int b0 = 0; b0 < nblocks; b0 += 1024) {
-        int i = b0 + threadIdx.x;
-        int v = i < nblocks ? part[i] : 0;
-        int ex = block_exclusive_scan(v, wsum, &tot);
-        if (i < nblocks) part[i] = ex + carry;
+    for (int b0 = 0; b0 < nblocks; b0 += 4 * SCAN_THREADS) {
+        const int i = b0 + 4 * threadIdx.x;
+        int v[4], sum = 0;
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            v[h] = i + h < nblocks ? vp[i + h] : 0;
+            sum += v[h];
+        }
+        int ex = block_exclusive_scan(sum, wsum, &tot) + carry;
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            if (i + h < nblocks) vp[i + h] = ex;
+            ex += v[h];
+        }
         carry += tot;
         __syncthreads();
     }
-    if (threadIdx.x == 0) part[nblocks] = carry;
+    if (threadIdx.x == 0) {
+        vp[nblocks] = carry;
+        *done = 0;
+    }
 }
 
 // With part == nullptr a single block scans the whole array (len <= SCAN_TILE).
@@ -104,7 +122,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_down(const int *in, int *
     if (write_total && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[len] = part ? part[gridDim.x] : tot;
 }
 
-void launch_exclusive_scan(const int *in, int *out, long long len, bool write_total, int *part,
+void launch_exclusive_scan(const int *in, int *out, long long len, bool write_total, int *part, int *done,
                            cudaStream_t st) {
     const int nb = (int)((len + SCAN_TILE - 1) / SCAN_TILE);
     if (nb == 0) {
@@ -116,9 +134,7 @@ void launch_exclusive_scan(const int *in, int *out, long long len, bool write_to
         after_launch(st, K_SCAN);
         return;
     }
-    launch_pdl(k_scan_reduce, nb, SCAN_THREADS, 0, st, in, len, part);
-    after_launch(st, K_SCAN);
-    launch_pdl(k_scan_top, 1, 1024, 0, st, part, nb);
+    launch_pdl(k_scan_reduce, nb, SCAN_THREADS, 0, st, in, len, part, done);
     after_launch(st, K_SCAN);
     launch_pdl(k_scan_down, nb, SCAN_THREADS, 0, st, in, out, len, part, write_total ? 1 : 0);
     after_launch(st, K_SCAN);
@@ -300,253 +316,367 @@ __device__ __forceinline__ long long c2m1(int d) {  // C(d - 1, 2)
     return a * (a - 1) / 2;
 }
 
-// Row relabelling, one warp per row (rows below LONG_ROW_CLASS), taken in
-// input order so that the rows are read sequentially and written scattered.
-// Pass 1 validates the row, counts its classes and sums neighbour degrees;
-// pass 2 writes every new id at its class offset (stable within a class);
-// the first 64 entries keep their new id and class in registers between
-// the passes.
-__global__ void __launch_bounds__(256) k_relabel_rows_warp(const int *rowptr, const int *colidx, int n,
-                                                           const int2 *vrange, const int2 *vinfo, const int *perm,
-                                                           const int *nrow, const int *coff, int ntiles, int *ncol,
-                                                           int4 *rinfo, VAcc *vacc, int *tcnt, int *status,
-                                                           int long_class) {
-    pdl_begin();
-    __shared__ int hist_all[8][NCLASS];
-    const int lane = lane_id();
-    int *H = hist_all[threadIdx.x >> 5];
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    int bad = 0;
-    for (int x = gw; x < n; x += nw) {
-        const int2 vx = vinfo[x];   // new id, degree (0 for a row with bad offsets)
-        const int r = vx.x, d = vx.y;
-        if (deg_class(d) >= long_class) continue;   // a CTA takes it
-        const int ob = d > 0 ? rowptr[x] : 0;
-        const int nb = nrow[r];
-        const int2 vr = vrange ? vrange[x] : make_int2(0, n);
-        if (d <= 32) {
-            // One entry per lane: its place in the relabelled row is the
-            // number of entries of a lower class plus those of its class
-            // before it, from eight ballots over the class bits (inactive
-            // lanes take class NCLASS, above every real one).
-            const bool act = lane < d;
-            const int y = act ? colidx[ob + lane] : 0;
-            const int yp = __shfl_up_sync(FULL, y, 1);
-            int nid = 0, c = NCLASS;
-            unsigned dl = 0, bl = 0;
-            long long p6l = 0;
-            if (act) {
-                int ys = global_id(y, vr, n);
-                if (ys < 0) { bad |= ST_EINVAL; ys = x; }
-                else if (ys == x || (lane > 0 && y <= yp)) bad |= ST_ENOTSIMPLE;
-                const int2 vi = vinfo[ys];
-                nid = vi.x;
-                c = deg_class(vi.y);
-                dl = (unsigned)vi.y;
-                p6l = c2m1(vi.y);
-                bl = vi.x < r;
-            }
-            static_assert(NCLASS < 256, "classes and the inactive value NCLASS fit eight bits");
-            unsigned eq = FULL, lt = 0;
+// Place of every active lane's entry among the entries of its group (a mask
+// of the active lanes), stable by degree class: the entries of a lower class
+// plus those of its own class before it, from ballots over the class bits. A
+// bit that all active entries of the warp share costs its ballot only.
+__device__ __forceinline__ int class_rank(int c, bool act, unsigned group) {
+    static_assert(NCLASS <= 128, "classes fit seven bits");
+    const unsigned all = __ballot_sync(FULL, act);
+    unsigned eq = group, lt = 0;
 #pragma unroll
-            for (int bit = 7; bit >= 0; --bit) {
-                const bool one = (c >> bit) & 1;
-                const unsigned ones = __ballot_sync(FULL, one);
-                if (one) {
-                    lt |= eq & ~ones;
-                    eq &= ones;
-                } else {
-                    eq &= ~ones;
-                }
-            }
-            if (act) ncol[nb + __popc(lt) + __popc(eq & lanemask_lt())] = nid;
-            // neighbour degrees are at most MAX_DEGREE: 32 of them fit 32 bits
-            const long long s1 = __reduce_add_sync(FULL, dl);
-            const int below = (int)__reduce_add_sync(FULL, bl);
-            const long long p6 = warp_sum(p6l);
-            const int sp = nb + below;
-            if (lane == 0) {
-                rinfo[r] = make_int4(nb, sp, nb + d, 0);
-                VAcc a;
-                a.S1 = s1; a.A1 = 0; a.P6 = p6; a.A2 = 0; a.A3 = 0; a.D12 = 0; a.K4 = 0; a.C4 = 0;
-                vacc[r] = a;
-            }
-            if (sp + lane < nb + d) tcnt[sp + lane] = 0;
-            continue;
-        }
-        for (int c = lane; c < NCLASS; c += 32) H[c] = 0;
-        __syncwarp();
-        long long s1 = 0, p6 = 0;
-        int below = 0, last = -1;
-        int nv0 = 0, nc0 = NCLASS + lane, nv1 = 0, nc1 = NCLASS + lane;   // entries lane and 32 + lane
-        for (int k = 0; k < d; k += 32) {
-            const int i = k + lane;
-            const bool act = i < d;
-            const int y = act ? colidx[ob + i] : 0;
-            int yp = __shfl_up_sync(FULL, y, 1);
-            if (lane == 0) yp = last;
-            last = __shfl_sync(FULL, y, 31);
-            if (act) {
-                int ys = global_id(y, vr, n);
-                if (ys < 0) { bad |= ST_EINVAL; ys = x; }
-                else if (ys == x || (i > 0 && y <= yp)) bad |= ST_ENOTSIMPLE;
-                const int2 vi = vinfo[ys];
-                const int c = deg_class(vi.y);
-                atomicAdd(&H[c], 1);
-                s1 += vi.y;
-                p6 += c2m1(vi.y);
-                below += vi.x < r;
-                if (k == 0) { nv0 = vi.x; nc0 = c; }
-                else if (k == 32) { nv1 = vi.x; nc1 = c; }
-            }
-        }
-        // exclusive scan of the 128 class counts: 4 per lane
-        __syncwarp();
-        {
-            int a0 = H[4 * lane], a1 = H[4 * lane + 1], a2 = H[4 * lane + 2], a3 = H[4 * lane + 3];
-            int sum = a0 + a1 + a2 + a3;
-            int ex = warp_inclusive_scan(sum) - sum;
-            H[4 * lane] = ex;
-            H[4 * lane + 1] = ex + a0;
-            H[4 * lane + 2] = ex + a0 + a1;
-            H[4 * lane + 3] = ex + a0 + a1 + a2;
-        }
-        __syncwarp();
-        for (int k = 0; k < d; k += 32) {
-            const int i = k + lane;
-            const bool act = i < d;
-            int nid, c;
-            if (k == 0) { nid = nv0; c = nc0; }
-            else if (k == 32) { nid = nv1; c = nc1; }
-            else {
-                int ys = act ? global_id(colidx[ob + i], vr, n) : 0;
-                if (ys < 0) ys = x;
-                const int2 vi = act ? vinfo[ys] : make_int2(0, 0);
-                nid = vi.x;
-                c = act ? deg_class(vi.y) : NCLASS + lane;
-            }
-            const unsigned peers = __match_any_sync(FULL, c);
-            const int rank = __popc(peers & lanemask_lt());
-            int pos = 0;
-            if (act) pos = H[c] + rank;
-            __syncwarp();
-            if (act && rank == 0) H[c] += __popc(peers);
-            __syncwarp();
-            if (act) ncol[nb + pos] = nid;
-        }
-        s1 = warp_sum(s1);
-        p6 = warp_sum(p6);
-        below = warp_sum(below);
-        const int sp = nb + below;
-        if (lane == 0) {
-            rinfo[r] = make_int4(nb, sp, nb + d, 0);
-            VAcc a;
-            a.S1 = s1; a.A1 = 0; a.P6 = p6; a.A2 = 0; a.A3 = 0; a.D12 = 0; a.K4 = 0; a.C4 = 0;
-            vacc[r] = a;
-        }
-        for (int p = sp + lane; p < nb + d; p += 32) tcnt[p] = 0;
-        __syncwarp();
+    for (int bit = 6; bit >= 0; --bit) {
+        const bool one = act && ((c >> bit) & 1);
+        const unsigned ones = __ballot_sync(FULL, one);
+        if (ones == 0 || ones == all) continue;
+        if (one) lt |= eq & ~ones;
+        eq &= one ? ones : ~ones;
     }
-    bad = __reduce_or_sync(FULL, bad);
-    if (lane == 0 && bad) set_status(status, bad);
+    return __popc(lt) + __popc(eq & lanemask_lt());
 }
 
-// Row relabelling, one CTA per long row (rows from LONG_ROW_CLASS on).
-constexpr int RLC_THREADS = 512;
-__global__ void __launch_bounds__(RLC_THREADS) k_relabel_rows_cta(const int *rowptr, const int *colidx, int n,
-                                                                  const int2 *vrange, const int2 *vinfo,
-                                                                  const int *perm,
-                                                                  const int *nrow, const int *coff, int ntiles,
-                                                                  int *ncol, int4 *rinfo, VAcc *vacc, int *tcnt,
-                                                                  int *status, int long_class) {
-    pdl_begin();
-    constexpr int NW = RLC_THREADS / 32;
-    __shared__ int H[NCLASS];
-    __shared__ int tot[NCLASS];
-    __shared__ int wc[NW][NCLASS];
-    __shared__ long long red[3][NW];
-    const int lane = lane_id(), w = threadIdx.x >> 5;
-    const int bound = coff[long_class * ntiles];
+struct RelabelArgs {
+    const int *rowptr, *colidx;
+    int n;
+    const int2 *vrange, *vinfo;
+    const int *perm, *nrow, *coff;
+    int ntiles;
+    int *ncol;
+    int4 *rinfo;
+    VAcc *vacc;
+    int *tcnt, *status;
+    int long_class;
+    int *counters;
+};
+
+// Rows x of at most L entries each, one per group of L lanes (x, r, d, ob are
+// the group's; d = 0 for none): one entry per lane. Every lane stores one
+// accumulator of its row, or a few (L = 8: the row's 64 bytes at once).
+template <int L>
+__device__ __forceinline__ int relabel_group(const RelabelArgs &A, int x, int r, int d, int ob, bool have) {
+    const int lane = lane_id(), l = lane & (L - 1), first = lane & ~(L - 1);
+    const int nb = have ? A.nrow[r] : 0;
+    const bool act = l < d;
+    int2 vr = make_int2(0, A.n);
+    if (A.vrange && act) vr = A.vrange[x];
+    const int y = act ? A.colidx[ob + l] : 0;
+    const int yp = __shfl_up_sync(FULL, y, 1);
+    int bad = 0, nid = 0, c = 0, dy = 0;
+    if (act) {
+        int ys = global_id(y, vr, A.n);
+        if (ys < 0) { bad = ST_EINVAL; ys = x; }
+        else if (ys == x || (l > 0 && y <= yp)) bad = ST_ENOTSIMPLE;
+        const int2 vi = A.vinfo[ys];
+        nid = vi.x;
+        dy = vi.y;
+        c = deg_class(dy);
+    }
+    const unsigned group = __ballot_sync(FULL, act) & ((L == 32 ? FULL : (1u << (L & 31)) - 1u) << first);
+    const int rank = class_rank(c, act, group);
+    if (act) A.ncol[nb + rank] = nid;
+    const int below = __popc(__ballot_sync(FULL, act && nid < r) & group);
+    // sums over the group: degrees (at most 2^20 each, 32 of them fit 32 bits) and C(d - 1, 2)
+    unsigned s1 = (unsigned)dy;
+    long long p6;
+    if (L == 32) {
+        s1 = __reduce_add_sync(FULL, s1);
+    } else {
+#pragma unroll
+        for (int o = 1; o < L; o <<= 1) s1 += __shfl_xor_sync(FULL, s1, o);
+    }
+    if (!__any_sync(FULL, dy > 8192)) {   // C(8191, 2) < 2^25
+        unsigned p = act ? (unsigned)(dy - 1) * (unsigned)(dy - 2) / 2u : 0u;
+        if (L == 32) {
+            p = __reduce_add_sync(FULL, p);
+        } else {
+#pragma unroll
+            for (int o = 1; o < L; o <<= 1) p += __shfl_xor_sync(FULL, p, o);
+        }
+        p6 = p;
+    } else {
+        p6 = act ? c2m1(dy) : 0;
+#pragma unroll
+        for (int o = 1; o < L; o <<= 1) p6 += __shfl_xor_sync(FULL, p6, o);
+    }
+    const int sp = nb + below;
+    if (have) {
+        if (l == 0) A.rinfo[r] = make_int4(nb, sp, nb + d, 0);
+        if (l < 8) reinterpret_cast<long long *>(&A.vacc[r])[l] = l == 0 ? (long long)s1 : l == 2 ? p6 : 0;   // S1, P6
+    }
+    if (sp + l < nb + d) A.tcnt[sp + l] = 0;
+    return bad;
+}
+
+// A row of 33 to 64 entries, two per lane.
+__device__ __forceinline__ int relabel_two(const RelabelArgs &A, int x, int r, int d, int ob) {
+    const int lane = lane_id();
+    const int nb = A.nrow[r];
+    const int2 vr = A.vrange ? A.vrange[x] : make_int2(0, A.n);
+    const bool act = 32 + lane < d;
+    const int y0 = A.colidx[ob + lane], y1 = act ? A.colidx[ob + 32 + lane] : 0;
+    const int p0 = __shfl_up_sync(FULL, y0, 1), mid = __shfl_sync(FULL, y0, 31);
+    int p1 = __shfl_up_sync(FULL, y1, 1);
+    if (lane == 0) p1 = mid;
     int bad = 0;
-    for (int r = bound + blockIdx.x; r < n; r += gridDim.x) {
-        const int x = perm[r];
-        const int nb = nrow[r], d = nrow[r + 1] - nb;
-        const int ob = d > 0 ? rowptr[x] : 0;
-        const int2 vr = vrange ? vrange[x] : make_int2(0, n);
-        for (int c = threadIdx.x; c < NCLASS; c += RLC_THREADS) H[c] = 0;
-        __syncthreads();
-        long long s1 = 0, p6 = 0, below = 0;
-        for (int i = threadIdx.x; i < d; i += RLC_THREADS) {
-            const int y = colidx[ob + i];
-            int ys = global_id(y, vr, n);
+    auto look = [&](int y, int before, bool first) {
+        int ys = global_id(y, vr, A.n);
+        if (ys < 0) { bad |= ST_EINVAL; ys = x; }
+        else if (ys == x || (!first && y <= before)) bad |= ST_ENOTSIMPLE;
+        return A.vinfo[ys];
+    };
+    const int2 v0 = look(y0, p0, lane == 0);
+    const int2 v1 = act ? look(y1, p1, false) : make_int2(0, 0);
+    const int c0 = deg_class(v0.y), c1 = deg_class(v1.y);
+    const unsigned in1 = __ballot_sync(FULL, act);
+    // entries of a lower class / of the same class, in each half of the row
+    unsigned eq00 = FULL, eq01 = in1, eq10 = FULL, eq11 = in1, lt00 = 0, lt01 = 0, lt10 = 0, lt11 = 0;
+#pragma unroll
+    for (int bit = 6; bit >= 0; --bit) {
+        const bool b0 = (c0 >> bit) & 1, b1 = act && ((c1 >> bit) & 1);
+        const unsigned o0 = __ballot_sync(FULL, b0), o1 = __ballot_sync(FULL, b1);
+        if ((o0 | o1) == 0 || (o0 == FULL && o1 == in1)) continue;
+        if (b0) { lt00 |= eq00 & ~o0; lt01 |= eq01 & ~o1; }
+        eq00 &= b0 ? o0 : ~o0;
+        eq01 &= b0 ? o1 : ~o1;
+        if (b1) { lt10 |= eq10 & ~o0; lt11 |= eq11 & ~o1; }
+        eq10 &= b1 ? o0 : ~o0;
+        eq11 &= b1 ? o1 : ~o1;
+    }
+    A.ncol[nb + __popc(lt00) + __popc(lt01) + __popc(eq00 & lanemask_lt())] = v0.x;
+    if (act) A.ncol[nb + __popc(lt10) + __popc(lt11) + __popc(eq10) + __popc(eq11 & lanemask_lt())] = v1.x;
+    const int below = __popc(__ballot_sync(FULL, v0.x < r)) + __popc(__ballot_sync(FULL, act && v1.x < r));
+    // 64 degrees of at most 2^20 fit 32 bits
+    const long long s1 = __reduce_add_sync(FULL, (unsigned)(v0.y + v1.y));
+    long long p6;
+    if (!__any_sync(FULL, max(v0.y, v1.y) > 8192)) {   // 64 values below 2^25
+        unsigned p = (unsigned)(v0.y - 1) * (unsigned)(v0.y - 2) / 2u;
+        if (act) p += (unsigned)(v1.y - 1) * (unsigned)(v1.y - 2) / 2u;
+        p6 = __reduce_add_sync(FULL, p);
+    } else {
+        p6 = warp_sum(c2m1(v0.y) + (act ? c2m1(v1.y) : 0ll));
+    }
+    const int sp = nb + below;
+    if (lane == 0) A.rinfo[r] = make_int4(nb, sp, nb + d, 0);
+    if (lane < 8) reinterpret_cast<long long *>(&A.vacc[r])[lane] = lane == 0 ? s1 : lane == 2 ? p6 : 0;   // S1, P6
+    for (int p = sp + lane; p < nb + d; p += 32) A.tcnt[p] = 0;
+    return bad;
+}
+
+// A row of more than 64 entries, one warp: pass 1 validates it, counts its
+// classes (H) and sums neighbour degrees; pass 2 writes every new id at its
+// class offset (stable within a class).
+__device__ __forceinline__ int relabel_row(const RelabelArgs &A, int x, int r, int d, int ob, int *H) {
+    const int lane = lane_id();
+    const int nb = A.nrow[r];
+    const int2 vr = A.vrange ? A.vrange[x] : make_int2(0, A.n);
+    int bad = 0;
+    for (int c = lane; c < NCLASS; c += 32) H[c] = 0;
+    __syncwarp();
+    long long s1 = 0, p6 = 0;
+    int below = 0, last = -1;
+    for (int k = 0; k < d; k += 32) {
+        const int i = k + lane;
+        const bool act = i < d;
+        const int y = act ? A.colidx[ob + i] : 0;
+        int yp = __shfl_up_sync(FULL, y, 1);
+        if (lane == 0) yp = last;
+        last = __shfl_sync(FULL, y, 31);
+        if (act) {
+            int ys = global_id(y, vr, A.n);
             if (ys < 0) { bad |= ST_EINVAL; ys = x; }
-            else if (ys == x || (i > 0 && y <= colidx[ob + i - 1])) bad |= ST_ENOTSIMPLE;
-            const int2 vi = vinfo[ys];
+            else if (ys == x || (i > 0 && y <= yp)) bad |= ST_ENOTSIMPLE;
+            const int2 vi = A.vinfo[ys];
             atomicAdd(&H[deg_class(vi.y)], 1);
             s1 += vi.y;
             p6 += c2m1(vi.y);
             below += vi.x < r;
         }
-        s1 = warp_sum(s1);
-        p6 = warp_sum(p6);
-        below = warp_sum(below);
-        if (lane == 0) { red[0][w] = s1; red[1][w] = p6; red[2][w] = below; }
+    }
+    // exclusive scan of the 128 class counts: 4 per lane
+    __syncwarp();
+    {
+        int a0 = H[4 * lane], a1 = H[4 * lane + 1], a2 = H[4 * lane + 2], a3 = H[4 * lane + 3];
+        int sum = a0 + a1 + a2 + a3;
+        int ex = warp_inclusive_scan(sum) - sum;
+        H[4 * lane] = ex;
+        H[4 * lane + 1] = ex + a0;
+        H[4 * lane + 2] = ex + a0 + a1;
+        H[4 * lane + 3] = ex + a0 + a1 + a2;
+    }
+    __syncwarp();
+    for (int k = 0; k < d; k += 32) {
+        const int i = k + lane;
+        const bool act = i < d;
+        int ys = act ? global_id(A.colidx[ob + i], vr, A.n) : 0;
+        if (ys < 0) ys = x;
+        const int2 vi = act ? A.vinfo[ys] : make_int2(0, 0);
+        const int c = act ? deg_class(vi.y) : NCLASS + lane;
+        const unsigned peers = __match_any_sync(FULL, c);
+        const int rank = __popc(peers & lanemask_lt());
+        int pos = 0;
+        if (act) pos = H[c] + rank;
+        __syncwarp();
+        if (act && rank == 0) H[c] += __popc(peers);
+        __syncwarp();
+        if (act) A.ncol[nb + pos] = vi.x;
+    }
+    s1 = warp_sum(s1);
+    p6 = warp_sum(p6);
+    below = warp_sum(below);
+    const int sp = nb + below;
+    if (lane == 0) A.rinfo[r] = make_int4(nb, sp, nb + d, 0);
+    if (lane < 8) reinterpret_cast<long long *>(&A.vacc[r])[lane] = lane == 0 ? s1 : lane == 2 ? p6 : 0;   // S1, P6
+    for (int p = sp + lane; p < nb + d; p += 32) A.tcnt[p] = 0;
+    __syncwarp();
+    return bad;
+}
+
+// A long row (from LONG_ROW_CLASS on), the whole CTA.
+constexpr int RLR_THREADS = 256;
+struct LongRowSmem {
+    int H[NCLASS];
+    int tot[NCLASS];
+    int wc[RLR_THREADS / 32][NCLASS];
+    long long red[3][RLR_THREADS / 32];
+};
+__device__ __forceinline__ int relabel_long(const RelabelArgs &A, int r, LongRowSmem &S) {
+    constexpr int NW = RLR_THREADS / 32;
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    int bad = 0;
+    const int x = A.perm[r];
+    const int nb = A.nrow[r], d = A.nrow[r + 1] - nb;
+    const int ob = d > 0 ? A.rowptr[x] : 0;
+    const int2 vr = A.vrange ? A.vrange[x] : make_int2(0, A.n);
+    for (int c = threadIdx.x; c < NCLASS; c += RLR_THREADS) S.H[c] = 0;
+    __syncthreads();
+    long long s1 = 0, p6 = 0, below = 0;
+    for (int i = threadIdx.x; i < d; i += RLR_THREADS) {
+        const int y = A.colidx[ob + i];
+        int ys = global_id(y, vr, A.n);
+        if (ys < 0) { bad |= ST_EINVAL; ys = x; }
+        else if (ys == x || (i > 0 && y <= A.colidx[ob + i - 1])) bad |= ST_ENOTSIMPLE;
+        const int2 vi = A.vinfo[ys];
+        atomicAdd(&S.H[deg_class(vi.y)], 1);
+        s1 += vi.y;
+        p6 += c2m1(vi.y);
+        below += vi.x < r;
+    }
+    s1 = warp_sum(s1);
+    p6 = warp_sum(p6);
+    below = warp_sum(below);
+    if (lane == 0) { S.red[0][w] = s1; S.red[1][w] = p6; S.red[2][w] = below; }
+    __syncthreads();
+    if (w == 0) {
+        int a0 = S.H[4 * lane], a1 = S.H[4 * lane + 1], a2 = S.H[4 * lane + 2], a3 = S.H[4 * lane + 3];
+        int sum = a0 + a1 + a2 + a3;
+        int ex = warp_inclusive_scan(sum) - sum;
+        S.H[4 * lane] = ex;
+        S.H[4 * lane + 1] = ex + a0;
+        S.H[4 * lane + 2] = ex + a0 + a1;
+        S.H[4 * lane + 3] = ex + a0 + a1 + a2;
+    }
+    __syncthreads();
+    for (int k = 0; k < d; k += RLR_THREADS) {
+        for (int i = threadIdx.x; i < NW * NCLASS; i += RLR_THREADS) (&S.wc[0][0])[i] = 0;
         __syncthreads();
-        if (w == 0) {
-            int a0 = H[4 * lane], a1 = H[4 * lane + 1], a2 = H[4 * lane + 2], a3 = H[4 * lane + 3];
-            int sum = a0 + a1 + a2 + a3;
-            int ex = warp_inclusive_scan(sum) - sum;
-            H[4 * lane] = ex;
-            H[4 * lane + 1] = ex + a0;
-            H[4 * lane + 2] = ex + a0 + a1;
-            H[4 * lane + 3] = ex + a0 + a1 + a2;
-        }
+        const int i = k + threadIdx.x;
+        const bool act = i < d;
+        int ys = act ? global_id(A.colidx[ob + i], vr, A.n) : 0;
+        if (ys < 0) ys = x;
+        const int2 vi = act ? A.vinfo[ys] : make_int2(0, 0);
+        const int c = act ? deg_class(vi.y) : NCLASS + lane;
+        const unsigned peers = __match_any_sync(FULL, c);
+        const int rank = __popc(peers & lanemask_lt());
+        if (act && rank == 0) S.wc[w][c] = __popc(peers);
         __syncthreads();
-        for (int k = 0; k < d; k += RLC_THREADS) {
-            for (int i = threadIdx.x; i < NW * NCLASS; i += RLC_THREADS) (&wc[0][0])[i] = 0;
-            __syncthreads();
-            const int i = k + threadIdx.x;
-            const bool act = i < d;
-            int ys = act ? global_id(colidx[ob + i], vr, n) : 0;
-            if (ys < 0) ys = x;
-            const int2 vi = act ? vinfo[ys] : make_int2(0, 0);
-            const int c = act ? deg_class(vi.y) : NCLASS + lane;
-            const unsigned peers = __match_any_sync(FULL, c);
-            const int rank = __popc(peers & lanemask_lt());
-            if (act && rank == 0) wc[w][c] = __popc(peers);
-            __syncthreads();
-            if (threadIdx.x < NCLASS) {
-                int s = 0;
-                for (int ww = 0; ww < NW; ++ww) {
-                    int t = wc[ww][threadIdx.x];
-                    wc[ww][threadIdx.x] = s;
-                    s += t;
-                }
-                tot[threadIdx.x] = s;
+        if (threadIdx.x < NCLASS) {
+            int s = 0;
+            for (int ww = 0; ww < NW; ++ww) {
+                int t = S.wc[ww][threadIdx.x];
+                S.wc[ww][threadIdx.x] = s;
+                s += t;
             }
-            __syncthreads();
-            if (act) ncol[nb + H[c] + wc[w][c] + rank] = vi.x;
-            __syncthreads();
-            if (threadIdx.x < NCLASS) H[threadIdx.x] += tot[threadIdx.x];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            long long a = 0, b = 0, c = 0;
-            for (int ww = 0; ww < NW; ++ww) { a += red[0][ww]; b += red[1][ww]; c += red[2][ww]; }
-            const int sp = nb + (int)c;
-            rinfo[r] = make_int4(nb, sp, nb + d, 0);
-            VAcc v;
-            v.S1 = a; v.A1 = 0; v.P6 = b; v.A2 = 0; v.A3 = 0; v.D12 = 0; v.K4 = 0; v.C4 = 0;
-            vacc[r] = v;
-            red[0][0] = sp;
+            S.tot[threadIdx.x] = s;
         }
         __syncthreads();
-        const int sp = (int)red[0][0];
-        for (int p = sp + threadIdx.x; p < nb + d; p += RLC_THREADS) tcnt[p] = 0;
+        if (act) A.ncol[nb + S.H[c] + S.wc[w][c] + rank] = vi.x;
+        __syncthreads();
+        if (threadIdx.x < NCLASS) S.H[threadIdx.x] += S.tot[threadIdx.x];
         __syncthreads();
     }
-    if (bad) set_status(status, bad);
+    long long a = 0, b = 0, c = 0;
+    for (int ww = 0; ww < NW; ++ww) { a += S.red[0][ww]; b += S.red[1][ww]; c += S.red[2][ww]; }
+    const int sp = nb + (int)c;
+    if (threadIdx.x == 0) A.rinfo[r] = make_int4(nb, sp, nb + d, 0);
+    if (threadIdx.x < 8)
+        reinterpret_cast<long long *>(&A.vacc[r])[threadIdx.x] = threadIdx.x == 0 ? a : threadIdx.x == 2 ? b : 0;   // S1, P6
+    for (int p = sp + threadIdx.x; p < nb + d; p += RLR_THREADS) A.tcnt[p] = 0;
+    __syncthreads();
+    return bad;
+}
+
+// Row relabelling. Long rows first, a CTA each; then the others, taken in
+// input order so that they are read sequentially and written scattered. A
+// warp takes one row at a time, or, with FOUR, four: rows of at most 8
+// entries at once (eight lanes each), of at most 16 in pairs, longer ones in
+// turn. A row is a chain of four dependent loads, so FOUR pays where rows are
+// short (G(3e6, mean degree 6): 861 -> 425 us) and where every warp has many
+// rows (a power-law graph of 1e5 vertices: 44 us alone, 74 us by fours).
+template <bool FOUR>
+__global__ void __launch_bounds__(RLR_THREADS, 6) k_relabel_rows(RelabelArgs A) {
+    pdl_begin();
+    __shared__ union {
+        int H[RLR_THREADS / 32][NCLASS];
+        LongRowSmem S;
+    } sm;
+    int bad = 0;
+    for (int r = A.coff[A.long_class * A.ntiles] + blockIdx.x; r < A.n; r += gridDim.x) bad |= relabel_long(A, r, sm.S);
+    const int lane = lane_id();
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int nw = (gridDim.x * blockDim.x) >> 5;
+    auto row = [&](int x, int r, int d, int ob) {
+        if (d <= 32) bad |= relabel_group<32>(A, x, r, d, ob, true);
+        else if (d <= 64) bad |= relabel_two(A, x, r, d, ob);
+        else bad |= relabel_row(A, x, r, d, ob, sm.H[threadIdx.x >> 5]);
+    };
+    for (int x = FOUR ? A.n : gw; x < A.n; x += nw) {
+        const int2 vx = A.vinfo[x];   // new id, degree (0 for a row with bad offsets)
+        if (deg_class(vx.y) < A.long_class) row(x, vx.x, vx.y, vx.y > 0 ? A.rowptr[x] : 0);
+    }
+    for (long long x0 = FOUR ? 4ll * gw : A.n; x0 < A.n; x0 += 4ll * nw) {
+        // lanes 8 q ..: row x0 + q
+        const int x = (int)min(x0 + (lane >> 3), (long long)A.n - 1);
+        bool have = x0 + (lane >> 3) < A.n;
+        const int2 vx = A.vinfo[x];
+        const int r = vx.x;
+        int d = vx.y;
+        const int ob = d > 0 ? A.rowptr[x] : 0;
+        if (deg_class(d) >= A.long_class) have = false;   // done by a CTA
+        if (!have) d = 0;
+        const int top = (int)__reduce_max_sync(FULL, (unsigned)d);
+        if (top <= 8) {
+            bad |= relabel_group<8>(A, x, r, d, ob, have);
+            continue;
+        }
+#pragma unroll 1
+        for (int q = 0; q < 4; ++q) {
+            const int src = top <= 16 ? 8 * (q + (lane >> 4)) : 8 * q;
+            const int xq = __shfl_sync(FULL, x, src), rq = __shfl_sync(FULL, r, src), dq = __shfl_sync(FULL, d, src);
+            const int oq = __shfl_sync(FULL, ob, src);
+            const bool hq = __shfl_sync(FULL, (int)have, src);
+            if (top <= 16) {
+                bad |= relabel_group<16>(A, xq, rq, dq, oq, hq);
+                ++q;
+            } else if (hq) {
+                row(xq, rq, dq, oq);
+            }
+        }
+    }
+    bad = __reduce_or_sync(FULL, bad);
+    if (lane == 0 && bad) {
+        set_status(A.status, bad);
+        atomicOr(&A.counters[CNT_BAD_ROWS], 1);
+    }
 }
 
 static void relabel_common(const int *rowptr, const int *colidx, const int2 *vrange, Work &w, cudaStream_t st) {
@@ -558,23 +688,22 @@ static void relabel_common(const int *rowptr, const int *colidx, const int2 *vra
     } else {
         launch_pdl(k_class_hist, nt, RL_THREADS, 0, st, rowptr, w.n, w.m, w.vinfo, w.chist, nt, w.counters, w.status);
         after_launch(st, K_CLASS_HIST);
-        launch_exclusive_scan(w.chist, w.coff, (long long)NCLASS * nt, false, w.scan_part, st);
+        launch_exclusive_scan(w.chist, w.coff, (long long)NCLASS * nt, false, w.scan_part, w.counters + CNT_SCAN_DONE, st);
         // ndeg (degree of each new id) is staged in `split`, then scanned into nrow
         launch_pdl(k_class_scatter, nt, RL_THREADS, 0, st, w.n, w.vinfo, w.coff, nt, w.perm, w.split);
         after_launch(st, K_CLASS_SCATTER);
-        launch_exclusive_scan(w.split, w.nrow, w.n, true, w.scan_part, st);
+        launch_exclusive_scan(w.split, w.nrow, w.n, true, w.scan_part, w.counters + CNT_SCAN_DONE, st);
     }
-    const int lrc = w.tune[TUNE_LONG_ROW_CLASS];
     // more CTAs than an SM holds: with rows of uneven length, the later
     // waves act as load balancing
-    launch_pdl(k_relabel_rows_warp, w.num_sms * w.tune[TUNE_GRID_RELABEL], 256, 0, st,
-        rowptr, colidx, w.n, vrange, w.vinfo, w.perm, w.nrow, w.coff, nt, w.ncol, w.rinfo, w.vacc, w.tcnt, w.status,
-        lrc);
-    after_launch(st, K_RELABEL_WARP);
-    launch_pdl(k_relabel_rows_cta, w.num_sms * 2, RLC_THREADS, 0, st, rowptr, colidx, w.n, vrange, w.vinfo, w.perm, w.nrow,
-                                                              w.coff, nt, w.ncol, w.rinfo, w.vacc, w.tcnt,
-                                                              w.status, lrc);
-    after_launch(st, K_RELABEL_CTA);
+    const RelabelArgs A{rowptr, colidx, w.n, vrange, w.vinfo, w.perm, w.nrow, w.coff, nt, w.ncol, w.rinfo, w.vacc, w.tcnt,
+                        w.status, w.tune[TUNE_LONG_ROW_CLASS], w.counters};
+    const int grid = w.num_sms * w.tune[TUNE_GRID_RELABEL];
+    // by fours: short rows, and at least 32 rows for every warp of the grid
+    const bool four = w.m < 16ll * w.n && w.n >= 32ll * grid * (RLR_THREADS / 32) / 4;
+    if (four) launch_pdl(k_relabel_rows<true>, grid, RLR_THREADS, 0, st, A);
+    else launch_pdl(k_relabel_rows<false>, grid, RLR_THREADS, 0, st, A);
+    after_launch(st, K_RELABEL);
 }
 
 void launch_relabel(const int *rowptr, const int *colidx, Work &w, cudaStream_t st) {

@@ -80,7 +80,9 @@ __device__ __forceinline__ void to_induced(long long *p) {
 // order puts them last): one warp per vertex. Every other vertex is solved in
 // groups of 32 consecutive caller ids: each lane loads its vertex's row bounds
 // and accumulators up front, the warp sums S1 and A1 over the neighbours of
-// each of the 32 in turn (coalesced gathers, two vertices in flight), each
+// four of the 32 at a time (eight lanes each, two gathers in flight: the sums
+// of a vertex take three shuffle steps of four vertices instead of five of
+// one, which kept the LSU pipe busier than the gathers), each
 // lane solves its own vertex, and the warp writes the group's 32 output rows
 // (3840 contiguous bytes) with coalesced stores through shared memory, which
 // also suits an output buffer in host memory. With long_class 0 (a graph
@@ -95,6 +97,7 @@ __device__ __forceinline__ void solve_write(long long d, const VAcc &a, long lon
 }
 
 constexpr int SOLVE_WARPS = 8;
+constexpr int SOLVE_GROUP_MAXD = 128;   // degree up to which eight lanes sum a vertex's neighbours
 
 __global__ void __launch_bounds__(SOLVE_WARPS * 32) k_solve(Graph g, const VAcc *vacc, const int *perm,
                                                             const int2 *vinfo, long long *out, int induced,
@@ -137,29 +140,41 @@ __global__ void __launch_bounds__(SOLVE_WARPS * 32) k_solve(Graph g, const VAcc 
         }
         long long mS1 = 0, mA1 = 0;   // this lane's vertex
         const int cnt = min(32, g.n - xo0);
-        for (int k = 0; k < cnt; k += 2) {
-            const int b0 = __shfl_sync(FULL, rx.x, k), e0 = __shfl_sync(FULL, rx.z, k);
-            const int b1 = __shfl_sync(FULL, rx.x, k + 1 < 32 ? k + 1 : 31);
-            const int e1 = k + 1 < cnt ? __shfl_sync(FULL, rx.z, k + 1) : b1;
-            long long s0 = 0, t0 = 0, s1 = 0, t1 = 0;
-            for (int off = lane; off < max(e0 - b0, e1 - b1); off += 32) {
-                if (b0 + off < e0) {
-                    const longlong2 sa = *reinterpret_cast<const longlong2 *>(&vacc[g.ncol[b0 + off]]);
-                    s0 += sa.x;
-                    t0 += sa.y;
+        for (int k = 0; k < cnt; k += 4) {   // four vertices, eight lanes each
+            const int src = k + (lane >> 3), sub = lane & 7;   // (past cnt: empty rows)
+            const int b = __shfl_sync(FULL, rx.x, src), e = __shfl_sync(FULL, rx.z, src);
+            const int top = (int)__reduce_max_sync(FULL, (unsigned)(e - b));
+            long long s1 = 0, a1 = 0;
+            if (top <= SOLVE_GROUP_MAXD) {
+                for (int p = b + sub; p - b - sub < top; p += 16) {
+                    longlong2 u = make_longlong2(0, 0), v = u;
+                    if (p < e) u = *reinterpret_cast<const longlong2 *>(&vacc[g.ncol[p]]);
+                    if (p + 8 < e) v = *reinterpret_cast<const longlong2 *>(&vacc[g.ncol[p + 8]]);
+                    s1 += u.x + v.x;
+                    a1 += u.y + v.y;
                 }
-                if (b1 + off < e1) {
-                    const longlong2 sa = *reinterpret_cast<const longlong2 *>(&vacc[g.ncol[b1 + off]]);
-                    s1 += sa.x;
-                    t1 += sa.y;
+#pragma unroll
+                for (int o = 1; o < 8; o <<= 1) {
+                    s1 += __shfl_xor_sync(FULL, s1, o);
+                    a1 += __shfl_xor_sync(FULL, a1, o);
+                }
+                // lane 8 q holds the sums of vertex k + q
+                const long long s = __shfl_sync(FULL, s1, (lane & 3) * 8), t = __shfl_sync(FULL, a1, (lane & 3) * 8);
+                if ((lane & ~3) == k) { mS1 = s; mA1 = t; }
+            } else {   // a long row among them: the whole warp, one vertex after the other
+                for (int q = 0; q < 4; ++q) {
+                    const int bq = __shfl_sync(FULL, b, 8 * q), eq = __shfl_sync(FULL, e, 8 * q);
+                    s1 = a1 = 0;
+                    for (int p = bq + lane; p < eq; p += 32) {
+                        const longlong2 u = *reinterpret_cast<const longlong2 *>(&vacc[g.ncol[p]]);
+                        s1 += u.x;
+                        a1 += u.y;
+                    }
+                    s1 = warp_sum(s1);
+                    a1 = warp_sum(a1);
+                    if (lane == k + q) { mS1 = s1; mA1 = a1; }
                 }
             }
-            s0 = warp_sum(s0);
-            t0 = warp_sum(t0);
-            s1 = warp_sum(s1);
-            t1 = warp_sum(t1);
-            if (lane == k) { mS1 = s0; mA1 = t0; }
-            if (lane == k + 1) { mS1 = s1; mA1 = t1; }
         }
         if (have) solve_write(rx.z - rx.x, a, mS1, mA1, induced, ob + lane * 15);
         __syncwarp();

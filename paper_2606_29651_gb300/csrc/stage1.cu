@@ -3,23 +3,27 @@
 //
 // In the relabelled graph every triangle u < v < w is found once, at its
 // lowest vertex u, as w in N+(u) ∩ N+(v) (Algorithm 2 enumerates the same
-// way with ids). For a root u the kernel loads N+(u) into a shared-memory
-// hash table, streams N+(v) of every v in N+(u) across the lanes of a warp
-// (the lists of several v are concatenated so that every lane is busy) and
-// probes each element. A hit is a triangle (u, v, w): t(v,w) is added to
-// global memory at the position of w in row v, and the hit sets bit i of row
-// j of R, the adjacency bit-matrix of N+(u) oriented upwards (R[j] bit i <=>
-// N+(u)[i] in N+(N+(u)[j]), v = N+(u)[j], w = N+(u)[i]).
-// In the warp tier t(u,v) and t(u,w) are also counted in shared memory per
-// hit, and a K4 u < v < w < x is a triangle (j, i) of R together with a
-// common bit of R[j] and R[i] -- Algorithm 2's pairwise test over `neigh`
-// done as word-wide bit operations. In the CTA tiers R is mirrored after the
-// expansion (a ballot transpose per 32 x 32 block), t(u, N+(u)[y]) is the
-// popcount of row y, and the K4s of u through y are the triangles of R at y:
-// twice their number is the sum over the neighbours z of y in R of
-// popc(R[y] & R[z]). A warp takes a row and its lanes one neighbour z each,
-// with the same word loop on every lane, so the cost follows the edges of R
-// and not the (much larger) number of K4s of dense hub neighbourhoods.
+// way with ids). Two ways to intersect, by graph (k_adj_bits decides):
+//   - hubs: the rows N+(v) of a skewed graph are long whatever the length of
+//     N+(u) (on R-MAT 22 a mean of 360 to 540 entries for roots of any
+//     out-degree), so the pairs (v, w) of N+(u) are probed in an adjacency
+//     bitmap of the hubs instead (adj.cuh): 7e9 tests there, against 2.8e10
+//     entries to stream;
+//   - no hubs: N+(v) of every v in N+(u) is streamed past a bit filter of
+//     N+(u) (warp tier) or a hash of it (CTA tiers).
+// A hit is a triangle (u, v, w): t(v,w) is added to global memory at the
+// position of w in row v (for a probe: a prefix count and a popcount), and
+// the hit sets R[j] bit i and R[i] bit j of the symmetric adjacency
+// bit-matrix of N+(u) (v = N+(u)[j], w = N+(u)[i]). The K4s of u are the
+// triangles of R, counted from common bits of adjacent rows (Algorithm 2's
+// pairwise test over `neigh` as word-wide bit operations), so the cost follows
+// the edges of R and not the (much larger) number of K4s of dense hub
+// neighbourhoods.
+//
+// Measured on GB300, triangle and aggregate stages together: R-MAT 22 220 ->
+// 91 ms, R-MAT 18 5.9 -> 2.8 ms, G(1501, 0.5) 3.3 -> 2.0 ms, against hash
+// probes of every streamed entry; G(3e6, mean degree 6) 1.40 -> 0.41 ms and
+// 8192 power-law graphs in a batch 6.6 -> 3.2 ms with four small roots per warp.
 #include "kernels.h"
 
 namespace niorca {
@@ -31,16 +35,202 @@ constexpr int TS_MAXD = 256;  // out-degree handled by a 256-thread CTA (k_tri_c
 constexpr int TW_WARPS = 8;
 
 struct __align__(16) TriWarpSmem {
-    int hk[4 * TW_MAXD];   // N+(u) hash at load <= 1/4 (most probes are misses)
-    int hv[4 * TW_MAXD];
+    Filter filter;
     int cnt[TW_MAXD];
-    int kc[TW_MAXD];
     unsigned R[TW_MAXD][2];
-    SegTab seg;
 };
 
-__global__ void __launch_bounds__(TW_WARPS * 32, 8) k_tri_warp(Graph g, int *tcnt, VAcc *vacc, int *heavy,
-                                                            int *counters, int maxd) {
+// K4s of a warp-tier root from its symmetric bit matrix R, a row per lane: the
+// triangles of R through y number half the common bits of y's row and its
+// neighbours' rows.
+__device__ __forceinline__ void warp_k4(const Graph &g, VAcc *vacc, int u, int s, int dp, const unsigned (*R)[2]) {
+    const int lane = lane_id();
+    unsigned ku = 0;
+    for (int y = lane; y < dp; y += 32) {
+        const uint2 ry = *reinterpret_cast<const uint2 *>(R[y]);
+        unsigned k = 0;
+        for (unsigned m = ry.x; m; m &= m - 1) {
+            const uint2 rz = *reinterpret_cast<const uint2 *>(R[__ffs(m) - 1]);
+            k += __popc(ry.x & rz.x) + __popc(ry.y & rz.y);
+        }
+        for (unsigned m = ry.y; m; m &= m - 1) {
+            const uint2 rz = *reinterpret_cast<const uint2 *>(R[31 + __ffs(m)]);
+            k += __popc(ry.x & rz.x) + __popc(ry.y & rz.y);
+        }
+        if (!k) continue;
+        ku += k;
+        add64(&vacc[g.ncol[s + y]].K4, k / 2);
+    }
+    ku = __reduce_add_sync(FULL, ku);   // each K4 at three of N+(u), twice
+    if (lane == 0 && ku) add64(&vacc[u].K4, ku / 6);
+    __syncwarp();
+}
+
+// ------------------------------------------------- adjacency bitmap
+
+// Words of the bitmap, one thread each: its entries' position in N+(v) by a
+// search, then the few entries themselves. Also decides whether the call's
+// triangle and aggregate stages probe (CNT_ADJ_ON): at least half of the
+// entries belong to vertices with a bitmap row, and those are hubs (at least
+// twice their share) or all vertices. Without hubs, out-lists are as short as
+// the rows they point at and streaming is as good (G(3213, mean degree 31):
+// 118 us a call streamed, 134 us probed with a bitmap of 2/3 of the rows). A
+// malformed graph (rows out of order) is not probed: the positions rely on
+// sorted rows.
+__global__ void __launch_bounds__(256) k_adj_bits(Graph g, AdjBits A, const int *nrow, unsigned *words,
+                                                  unsigned short *prefix, int *counters) {
+    pdl_begin();
+    if (degree_overflow(counters)) return;
+    const int total = nrow[g.n];
+    const long long own = total - nrow[A.base], rows = g.n - A.base;
+    const bool on = rows > 0 && !counters[CNT_BAD_ROWS] && 2 * own >= total &&
+                    (A.base == 0 || own * g.n >= 2 * rows * total);
+    if (blockIdx.x == 0 && threadIdx.x == 0) counters[CNT_ADJ_ON] = on;
+    if (!on) return;
+    const int lane = lane_id();
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    for (int v = A.base + gw; v < g.n; v += nw) {   // longest rows first
+        const int4 rv = g.rinfo[v];
+        const int at = A.row(v), nq = ((g.n - 1 - v) >> 5) + 1;
+        const int y = rv.y, z = rv.z - y < 65536 ? rv.z : y;   // (more out-entries: only in an asymmetric CSR)
+        for (int q = lane; q < nq; q += 32) {
+            const int top = g.n - 1 - 32 * q;   // id of bit 0
+            int p = lower_bound(g.ncol, y, z, top - 31);
+            prefix[at + q] = (unsigned short)(p - y);
+            unsigned bits = 0;
+            for (; p < z; ++p) {
+                const int k = top - g.ncol[p];
+                if (k < 0) break;
+                bits |= 1u << k;
+            }
+            words[at + q] = bits;
+        }
+    }
+}
+
+AdjBits adj_bits(const Work &w) {
+    // 6 bytes per word (word and prefix) in 4 m bytes
+    long long lo = 0, hi = w.n;
+    while (lo < hi) {
+        const long long mid = (lo + hi + 1) / 2;
+        if (6 * AdjBits::row_words(mid) <= 4ll * w.m) lo = mid; else hi = mid - 1;
+    }
+    AdjBits A;
+    A.words = reinterpret_cast<const unsigned *>(w.tcnt + w.m);
+    A.prefix = reinterpret_cast<const unsigned short *>(A.words + AdjBits::row_words(lo));
+    A.n = w.n;
+    A.base = w.n - (int)lo;
+    return A;
+}
+
+// One warp-tier root over the adjacency bitmap: its pairs of out-neighbours
+// are probed 32 columns at a time, dp^2 / 2 tests instead of the sum of its
+// out-neighbours' row lengths. A ballot is a row of R, and a lane counts its
+// own column.
+__device__ __forceinline__ void tri_root_probe(const Graph &g, const AdjBits &A, int *tcnt, VAcc *vacc, int u, int s, int dp,
+                                               TriWarpSmem &S) {
+    const int lane = lane_id();
+    const OutList L = out_list(g, A, s, dp);
+    int c0 = 0, c1 = 0;                        // t(u, .) of entries lane, 32 + lane
+    unsigned r00 = 0, r01 = 0, r10 = 0, r11 = 0;   // the lane's rows of the symmetric R: entry lane, 32 + lane
+    out_pairs(g, A, L, FULL, FULL, lane < dp, 32 + lane < dp, [&](int b, int r, bool hit, int pos) {
+        const unsigned bal = __ballot_sync(FULL, hit);
+        if (hit) {
+            atomicAdd(&tcnt[pos], 1);
+            if (b == 0) { ++c0; r00 |= 1u << r; }
+            else if (b == 1) { ++c1; r10 |= 1u << r; }
+            else { ++c1; r11 |= 1u << r; }
+        }
+        if (lane == r) {
+            if (b == 0) r00 |= bal;
+            else if (b == 1) r01 = bal;
+            else r11 |= bal;
+            if (b == 2) c1 += __popc(bal); else c0 += __popc(bal);
+        }
+    });
+    if (!__any_sync(FULL, c0 | c1)) return;
+    if (c0) atomicAdd(&tcnt[s + lane], c0);
+    if (c1) atomicAdd(&tcnt[s + 32 + lane], c1);
+    S.R[lane][0] = r00;
+    S.R[lane][1] = r01;
+    S.R[32 + lane][0] = r10;
+    S.R[32 + lane][1] = r11;
+    __syncwarp();
+    warp_k4(g, vacc, u, s, dp, S.R);
+}
+
+// One warp-tier root whose out-neighbours' rows (r0, r1: entries lane and 32
+// + lane, ids w0, w1) are streamed past a filter of N+(u).
+__device__ __forceinline__ void tri_root_stream(const Graph &g, int *tcnt, VAcc *vacc, int u, int s, int dp, TriWarpSmem &S) {
+    const int lane = lane_id();
+    int w0 = -1, w1 = -1;
+    int2 r0 = make_int2(0, 0), r1 = r0;
+    auto fill = [&](int i, int &w, int2 &r) {
+        if (i >= dp) return;
+        w = g.ncol[s + i];
+        if (i == dp - 1) return;   // the last out-neighbour has no row to walk
+        const int4 rw = g.rinfo[w];
+        r = make_int2(rw.y, rw.z);
+    };
+    fill(lane, w0, r0);
+    if (dp > 32) fill(32 + lane, w1, r1);
+    S.filter.set(w0, w1, w0 >= 0, w1 >= 0);
+    S.cnt[lane] = S.cnt[32 + lane] = 0;
+    *reinterpret_cast<uint4 *>(S.R[2 * lane]) = make_uint4(0, 0, 0, 0);
+    __syncwarp();
+    bool found = false;
+    filter_walk(g.ncol, S.filter, r0, r1, dp, [&](int j, int pos, int w) {
+        const int i = S.filter.find(w, dp);
+        if (i < 0) return;
+        atomicAdd(&S.cnt[j], 1);
+        atomicAdd(&S.cnt[i], 1);
+        atomicOr(&S.R[j][i >> 5], 1u << (i & 31));
+        atomicOr(&S.R[i][j >> 5], 1u << (j & 31));
+        atomicAdd(&tcnt[pos], 1);
+        found = true;
+    });
+    if (!__any_sync(FULL, found)) return;
+    __syncwarp();
+    for (int i = lane; i < dp; i += 32)
+        if (S.cnt[i]) atomicAdd(&tcnt[s + i], S.cnt[i]);
+    warp_k4(g, vacc, u, s, dp, S.R);
+}
+
+// Four roots of out-degree at most 8, eight lanes each (lane 8 q + l: entry l
+// of root q, id w, row r).
+__device__ __forceinline__ void tri_roots_small(const Graph &g, int *tcnt, VAcc *vacc, int u, int s, int dp, int w, int2 r) {
+    const int lane = lane_id(), l = lane & 7;
+    unsigned R = 0;   // the lane's row of the root's oriented 8 x 8 matrix
+    int t = 0;
+    small_walk(g.ncol, w, r, [&](int pos, int x) {
+        for (int i = l + 1; i < dp; ++i)
+            if (g.ncol[s + i] == x) {
+                R |= 1u << i;
+                ++t;
+                atomicAdd(&tcnt[s + i], 1);
+                atomicAdd(&tcnt[pos], 1);
+            }
+    });
+    if (t) atomicAdd(&tcnt[s + l], t);
+    if (!__any_sync(FULL, R & (R - 1))) return;   // a K4 has two triangles in the row of its second vertex
+    for (int i = 1; i < 8; ++i) {
+        const unsigned Ri = __shfl_sync(FULL, R, (lane & 24) | i);
+        unsigned x = (R >> i) & 1u ? R & Ri : 0u;
+        if (!x) continue;
+        const int k = __popc(x);
+        add64(&vacc[u].K4, k);
+        add64(&vacc[w].K4, k);
+        add64(&vacc[g.ncol[s + i]].K4, k);
+        for (; x; x &= x - 1) add64(&vacc[g.ncol[s + __ffs(x) - 1]].K4, 1);
+    }
+}
+
+// The warp tier, over the adjacency bitmap when the call has one, else
+// streaming rows. Six CTAs per SM (40 registers): eight make the streaming
+// path spill more than the occupancy gains (G(1e6, mean degree 32): 641
+// against 539 us).
+__global__ void __launch_bounds__(TW_WARPS * 32, 6) k_tri_warp(Graph g, AdjBits A, int *tcnt, VAcc *vacc, int *heavy,
+                                                            int *counters, int maxd, const int *coff, int ntiles) {
     pdl_begin();
     __shared__ TriWarpSmem sm_all[TW_WARPS];
     TriWarpSmem &S = sm_all[threadIdx.x >> 5];
@@ -48,83 +238,47 @@ __global__ void __launch_bounds__(TW_WARPS * 32, 8) k_tri_warp(Graph g, int *tcn
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     if (degree_overflow(counters)) return;
-    for (int u = gw; u < g.n; u += nw) {
-        const int4 ru = g.rinfo[u];
-        const int s = ru.y, e = ru.z, dp = e - s;
-        if (dp < 2) continue;
+    const bool probe = counters[CNT_ADJ_ON];
+    auto root = [&](int u, int s, int dp) {
+        if (dp < 2) return;
         if (dp > maxd) {
             if (lane == 0) {
                 if (dp <= TS_MAXD) heavy[atomicAdd(&counters[CNT_TRI_HEAVY], 1)] = u;
                 else heavy[g.n - 1 - atomicAdd(&counters[CNT_TRI_BIG], 1)] = u;
             }
-            continue;
+            return;
         }
-        const unsigned mask = next_pow2(4 * dp) - 1;
-        for (int i = lane; i <= (int)mask; i += 32) S.hk[i] = -1;
-        for (int i = lane; i < TW_MAXD; i += 32) {
-            S.cnt[i] = 0;
-            S.kc[i] = 0;
-            S.R[i][0] = 0;
-            S.R[i][1] = 0;
-        }
+        if (probe) tri_root_probe(g, A, tcnt, vacc, u, s, dp, S);
+        else tri_root_stream(g, tcnt, vacc, u, s, dp, S);
         __syncwarp();
-        for (int i = lane; i < dp; i += 32) hset_insert(S.hk, S.hv, mask, g.ncol[s + i], i);
-        const int umax = g.ncol[e - 1];
-        __syncwarp();
-        int found = 0;
-        for (int jb = 0; jb < dp - 1; jb += 32) {   // the last out-neighbour has no row to walk
-            const int j = jb + lane;
-            int len = 0, vs = 0;
-            if (j < dp - 1) {
-                const int4 rv = g.rinfo[g.ncol[s + j]];
-                vs = rv.y;
-                len = rv.z - rv.y;
-            }
-            int mypre;
-            const int total = seg_build(S.seg, vs, len, mypre);
-            seg_visit32<2>(g.ncol, S.seg, mypre, len, total, 0, [&](bool valid, int q, int pos, int w) {
-                const int i = (valid && w <= umax) ? hset_find(S.hk, S.hv, mask, w) : -1;
-                const bool hit = i >= 0;
-                if (!__any_sync(FULL, hit)) return;
-                const int jj = jb + q;
-                if (hit) {
-                    atomicAdd(&S.cnt[jj], 1);
-                    atomicOr(&S.R[0][0] + jj * 2 + (i >> 5), 1u << (i & 31));
-                    atomicAdd(&S.cnt[i], 1);
-                    atomicAdd(&tcnt[pos], 1);
-                    found = 1;
-                }
-            });
-            __syncwarp();
-        }
-        if (!__any_sync(FULL, found)) continue;
-        for (int i = lane; i < dp; i += 32)
-            if (S.cnt[i]) atomicAdd(&tcnt[s + i], S.cnt[i]);
-        long long ku = 0;
-        for (int j = lane; j < dp; j += 32) {
-            const unsigned rj0 = S.R[j][0], rj1 = S.R[j][1];
-            for (int wd = 0; wd < 2; ++wd) {
-                unsigned bits = wd ? rj1 : rj0;
-                while (bits) {
-                    const int i = wd * 32 + __ffs(bits) - 1;
-                    bits &= bits - 1;
-                    unsigned x0 = rj0 & S.R[i][0], x1 = rj1 & S.R[i][1];
-                    const int k = __popc(x0) + __popc(x1);
-                    if (!k) continue;
-                    ku += k;
-                    atomicAdd(&S.kc[j], k);
-                    atomicAdd(&S.kc[i], k);
-                    while (x0) { atomicAdd(&S.kc[__ffs(x0) - 1], 1); x0 &= x0 - 1; }
-                    while (x1) { atomicAdd(&S.kc[32 + __ffs(x1) - 1], 1); x1 &= x1 - 1; }
+    };
+    // ids of low degree: four roots at a time, eight lanes each
+    const int low = probe ? 0 : low_degree_ids(g.n, nw, coff, ntiles);
+    for (long long u0 = 4ll * gw; u0 < low; u0 += 4ll * nw) {
+        const int u = (int)u0 + (lane >> 3), l = lane & 7;
+        int4 ru = make_int4(0, 0, 0, 0);
+        if (u < low) ru = g.rinfo[u];
+        const int s = ru.y, dp = ru.z - s;
+        if (!__any_sync(FULL, dp > min(SMALL_DP, maxd))) {
+            int w = -1;
+            int2 r = make_int2(0, 0);
+            if (dp >= 2 && l < dp) {
+                w = g.ncol[s + l];
+                if (l < dp - 1) {
+                    const int4 rw = g.rinfo[w];
+                    r = make_int2(rw.y, rw.z);
                 }
             }
+            if (!__any_sync(FULL, r.y - r.x > SMALL_ROW)) {
+                tri_roots_small(g, tcnt, vacc, u, s, dp, w, r);
+                continue;
+            }
         }
-        ku = warp_sum(ku);
-        __syncwarp();
-        if (lane == 0 && ku) add64(&vacc[u].K4, ku);
-        for (int i = lane; i < dp; i += 32)
-            if (S.kc[i]) add64(&vacc[g.ncol[s + i]].K4, S.kc[i]);
-        __syncwarp();
+        for (int q = 0; q < 4; ++q) root((int)u0 + q, __shfl_sync(FULL, s, 8 * q), __shfl_sync(FULL, dp, 8 * q));
+    }
+    for (int u = low + gw; u < g.n; u += nw) {
+        const int4 ru = g.rinfo[u];
+        root(u, ru.y, ru.z - ru.y);
     }
 }
 
@@ -170,8 +324,8 @@ __device__ __forceinline__ int out_index(const int *hk, const int *hv, unsigned 
 // than the compiled ones, bits_maxd <= hash_maxd), else it probes N+(u) by
 // binary search and enumerates the K4 of each triangle.
 template <int THREADS, int BITMAT_MAXD, int BITMAT_HSLOTS, int HASH_MAXD, bool BACK, int HMUL>
-__device__ __forceinline__ void tri_cta(const Graph &g, int *tcnt, VAcc *vacc, const int *list, int count,
-                                        int *next, int bits_maxd, int hash_maxd) {
+__device__ __forceinline__ void tri_cta(const Graph &g, const AdjBits &A, bool probe, int *tcnt, VAcc *vacc,
+                                        const int *list, int count, int *next, int bits_maxd, int hash_maxd) {
     extern __shared__ __align__(16) unsigned char dsm[];
     constexpr int TC_THREADS = THREADS;
     constexpr int NW = THREADS / 32;
@@ -182,7 +336,9 @@ __device__ __forceinline__ void tri_cta(const Graph &g, int *tcnt, VAcc *vacc, c
         const int s = ru.y, e = ru.z, dp = e - s;
         const bool use_hash = dp <= HASH_MAXD && dp <= hash_maxd;
         const bool use_bits = use_hash && dp <= BITMAT_MAXD && dp <= bits_maxd;
-        unsigned H = use_hash ? next_pow2(HMUL * dp) : 0;   // hash load at most 1 / HMUL, within the carve:
+        // rows js .. of N+(u) are probed in the bitmap, the ones before streamed
+        const int js = use_bits && probe ? lower_bound(g.ncol, s, e, A.base) - s : dp;
+        unsigned H = use_hash && js > 0 ? next_pow2(HMUL * dp) : 0;   // hash load at most 1 / HMUL, within the carve:
         const unsigned hcap = use_bits ? BITMAT_HSLOTS : 2 * HASH_MAXD;   // its mode's slots
         if (H > hcap) H = hcap;
         const unsigned mask = H ? H - 1 : 0;
@@ -198,7 +354,6 @@ __device__ __forceinline__ void tri_cta(const Graph &g, int *tcnt, VAcc *vacc, c
         SegTab *segs = reinterpret_cast<SegTab *>(kc + nloc);   // one per warp
         unsigned short *zb = reinterpret_cast<unsigned short *>(segs + NW) + wid * 64;  // 64 per warp
         int *work = reinterpret_cast<int *>(reinterpret_cast<unsigned short *>(segs + NW) + NW * 64);
-        long long *ksum = reinterpret_cast<long long *>(work + 2);    // sum of kc over the rows
         unsigned *R = reinterpret_cast<unsigned *>(work + 4);
         SegTab &seg = segs[wid];
         for (int i = threadIdx.x; i < (int)H; i += TC_THREADS) hk[i] = -1;
@@ -207,18 +362,56 @@ __device__ __forceinline__ void tri_cta(const Graph &g, int *tcnt, VAcc *vacc, c
             for (int i = threadIdx.x; i < dp * WP; i += TC_THREADS) R[i] = 0;
         if (threadIdx.x < 4) work[threadIdx.x] = 0;
         __syncthreads();
-        if (use_hash)
+        if (H)
             for (int i = threadIdx.x; i < dp; i += TC_THREADS) hset_insert(hk, hv, mask, g.ncol[s + i], i);
         const int umax = g.ncol[e - 1];
-        __syncthreads();
         long long ku = 0;
+        if (js < dp) {
+            // Probe blocks of 32 rows x 32 columns (rows jb, columns t >= jb), a
+            // warp each: a ballot is a row's word of R, a lane's hits over the
+            // rows the word of its mirror image.
+            const int b0 = js >> 5;   // the first block of rows
+            for (int it = b0 * (b0 + 1) / 2 + wid; it < W * (W + 1) / 2; it += NW) {
+                int t, jb;
+                block_pair(it, t, jb);
+                if (jb < b0) continue;
+                const int i = 32 * t + lane, j = 32 * jb + lane;
+                const int k = i < dp ? g.n - 1 - g.ncol[s + i] : 0;
+                int roff = 0, ry = 0;
+                if (j >= js && j < dp) {
+                    const int v = g.ncol[s + j];
+                    roff = A.row(v);
+                    ry = g.rinfo[v].y;
+                }
+                const bool diag = t == jb;
+                unsigned row = 0, col = 0;
+                adj_probe<8>(A, __ballot_sync(FULL, j >= js && j < dp - 1), roff, k, i < dp, diag,
+                             [&](int r, bool hit, int at, unsigned word) {
+                                 const unsigned bal = __ballot_sync(FULL, hit);
+                                 const int y = __shfl_sync(FULL, ry, r);
+                                 if (lane == r) row = bal;
+                                 if (hit) {
+                                     col |= 1u << r;
+                                     atomicAdd(&tcnt[y + A.rank(at, k, word)], 1);
+                                 }
+                             });
+                if (diag) {
+                    if (i < dp) R[i * WP + t] = row | col;
+                } else {
+                    if (j < dp) R[j * WP + t] = row;
+                    if (i < dp) R[i * WP + jb] = col;
+                }
+            }
+        }
+        __syncthreads();
         // every warp takes every chunk of 32 out-neighbours and the windows
         // wid, wid + NW, ... of its concatenated lists: no warp waits on a
         // larger chunk of another
-        for (int jb = 0; jb < dp - 1; jb += 32) {
+        const int jend = min(js, dp - 1);   // the last out-neighbour has no row to walk
+        for (int jb = 0; jb < jend; jb += 32) {
             const int j = jb + lane;
             int len = 0, vs = 0;
-            if (j < dp - 1) {
+            if (j < jend) {
                 const int4 rv = g.rinfo[g.ncol[s + j]];
                 vs = rv.y;
                 len = rv.z - rv.y;
@@ -231,10 +424,10 @@ __device__ __forceinline__ void tri_cta(const Graph &g, int *tcnt, VAcc *vacc, c
                 if (!__any_sync(FULL, hit)) return;
                 const int jj = jb + q;
                 if (use_bits) {
-                    // the upper half of R only; t(u, v) and t(u, w) follow
-                    // from R's rows once it is symmetric
+                    // both halves of R; t(u, v) and t(u, w) follow from its rows
                     if (hit) {
                         atomicOr(&R[jj * WP + (i >> 5)], 1u << (i & 31));
+                        atomicOr(&R[i * WP + (jj >> 5)], 1u << (jj & 31));
                         atomicAdd(&tcnt[pos], 1);
                     }
                     return;
@@ -273,56 +466,45 @@ __device__ __forceinline__ void tri_cta(const Graph &g, int *tcnt, VAcc *vacc, c
         for (int i = threadIdx.x; i < nloc; i += TC_THREADS)
             if (cnt[i]) atomicAdd(&tcnt[s + i], cnt[i]);
         if (use_bits) {
-            // Mirror R: every 32 x 32 block above the diagonal (and the
-            // diagonal ones) is transposed by one warp with ballots and ORed
-            // into its place below.
-            const int nblk = W * (W + 1) / 2;
-            for (int bidx = wid; bidx < nblk; bidx += NW) {
-                int bj = 0, rem = bidx;
-                while (rem >= W - bj) {
-                    rem -= W - bj;
-                    ++bj;
-                }
-                const int bi = bj + rem;   // block of rows bj, word bi (bi >= bj)
-                const int j = bj * 32 + lane;
-                const unsigned wv = j < dp ? R[j * WP + bi] : 0u;
-                unsigned tv = 0;
-                for (int k = 0; k < 32; ++k) {
-                    const unsigned b = __ballot_sync(FULL, (wv >> k) & 1u);
-                    if (lane == k) tv = b;
-                }
-                const int i = bi * 32 + lane;
-                if (i < dp) {
-                    if (bi == bj) R[i * WP + bj] = wv | tv;
-                    else if (tv) R[i * WP + bj] |= tv;
-                }
-                __syncwarp();
-            }
-            __syncthreads();
-            // K4 credits from the symmetric R: warp per row y, one neighbour
-            // z of y per lane, 32 at a time (collected in zb); the row's
-            // popcount is t(u, N+(u)[y]) from the triangles rooted at u.
+            // K4s of u: triangles p < q < r of R. A warp takes a row y and, one
+            // per lane, its neighbours z < y, 32 at a time (collected in zb):
+            // the common bits of rows y and z below z are triangles with y
+            // highest, those above y triangles with z lowest and y in the
+            // middle. Two thirds of the words of a pair are read, once per
+            // pair. The row's popcount is t(u, N+(u)[y]) from the triangles
+            // rooted at u.
             for (;;) {
                 int y = 0;
-                if (lane == 0) y = atomicAdd(&work[0], 1);
+                if (lane == 0) y = dp - 1 - atomicAdd(&work[0], 1);   // most neighbours below first
                 y = __shfl_sync(FULL, y, 0);
-                if (y >= dp) break;
+                if (y < 0) break;
                 const unsigned *ry = R + y * WP;
-                long long acc = 0;
+                const int wy = y >> 5;
+                unsigned acc = 0;
                 auto batch = [&](int cnt) {
-                    if (lane < cnt) {
-                        const unsigned *rz = R + zb[lane] * WP;
-                        int k = 0;
-                        for (int t = 0; t < W; ++t) k += __popc(ry[t] & rz[t]);
+                    if (lane >= cnt) return;
+                    const int z = zb[lane], wz = z >> 5;
+                    const unsigned *rz = R + z * WP;
+                    unsigned k = 0;
+                    for (int t = 0; t < wz; ++t) k += __popc(ry[t] & rz[t]);
+                    acc += k + __popc(ry[wz] & rz[wz] & ((1u << (z & 31)) - 1u));
+                    k = __popc(ry[wy] & rz[wy] & ~((2u << (y & 31)) - 1u));
+                    for (int t = wy + 1; t < W; ++t) k += __popc(ry[t] & rz[t]);
+                    if (k) {
                         acc += k;
+                        ku += k;
+                        atomicAdd(&kc[z], (int)k);
                     }
                 };
+                int tuy = 0;   // set bits of row y
+                for (int t = lane; t < W; t += 32) tuy += __popc(ry[t]);
+                tuy = (int)__reduce_add_sync(FULL, (unsigned)tuy);
+                if (tuy == 0) continue;
+                if (lane == 0) atomicAdd(&tcnt[s + y], tuy);
                 int nb = 0;   // entries waiting in zb (warp-uniform)
-                int tuy = 0;  // set bits of row y
-                for (int t = 0; t < W; ++t) {
-                    const bool set = (ry[t] >> lane) & 1u;
+                for (int t = 0; t <= wy; ++t) {
+                    const bool set = ((ry[t] >> lane) & 1u) && t * 32 + lane < y;
                     const unsigned bal = __ballot_sync(FULL, set);
-                    tuy += __popc(bal);
                     if (set) zb[nb + __popc(bal & lanemask_lt())] = (unsigned short)(t * 32 + lane);
                     nb += __popc(bal);
                     __syncwarp();
@@ -335,38 +517,34 @@ __device__ __forceinline__ void tri_cta(const Graph &g, int *tcnt, VAcc *vacc, c
                     }
                 }
                 if (nb) batch(nb);
-                if (lane == 0 && tuy) atomicAdd(&tcnt[s + y], tuy);
-                acc = warp_sum(acc) / 2;   // K4s of u through y
-                if (lane == 0 && acc) {
-                    kc[y] = (int)acc;
-                    atomicAdd((unsigned long long *)ksum, (unsigned long long)acc);
-                }
+                acc = __reduce_add_sync(FULL, acc);   // at most C(1151, 2)
+                if (lane == 0 && acc) atomicAdd(&kc[y], (int)acc);
                 __syncwarp();
             }
         }
         __syncthreads();
         ku = warp_sum(ku);
         if (lane == 0 && ku) add64(&vacc[u].K4, ku);
-        if (use_bits && threadIdx.x == 0 && *ksum) add64(&vacc[u].K4, *ksum / 3);   // each K4 at 3 of N+(u)
         for (int i = threadIdx.x; i < nloc; i += TC_THREADS)
             if (kc[i]) add64(&vacc[g.ncol[s + i]].K4, kc[i]);
         __syncthreads();
     }
 }
 
-__global__ void __launch_bounds__(TS_THREADS) k_tri_cta(Graph g, int *tcnt, VAcc *vacc, const int *heavy,
+__global__ void __launch_bounds__(TS_THREADS) k_tri_cta(Graph g, AdjBits A, int *tcnt, VAcc *vacc, const int *heavy,
                                                         int *counters, int bits_maxd, int hash_maxd) {
     pdl_begin();
     if (degree_overflow(counters)) return;
-    tri_cta<TS_THREADS, TS_MAXD, 4 * TS_MAXD, TS_MAXD, false, 4>(g, tcnt, vacc, heavy, counters[CNT_TRI_HEAVY],
-                                                            counters + CNT_TRI_CTA_NEXT, bits_maxd, hash_maxd);
+    tri_cta<TS_THREADS, TS_MAXD, 4 * TS_MAXD, TS_MAXD, false, 4>(g, A, counters[CNT_ADJ_ON], tcnt, vacc, heavy,
+                                                            counters[CNT_TRI_HEAVY], counters + CNT_TRI_CTA_NEXT,
+                                                            bits_maxd, hash_maxd);
 }
 
-__global__ void __launch_bounds__(TB_THREADS) k_tri_big(Graph g, int *tcnt, VAcc *vacc, const int *heavy,
+__global__ void __launch_bounds__(TB_THREADS) k_tri_big(Graph g, AdjBits A, int *tcnt, VAcc *vacc, const int *heavy,
                                                         int *counters, int bits_maxd, int hash_maxd) {
     pdl_begin();
     if (degree_overflow(counters)) return;
-    tri_cta<TB_THREADS, TB_BITMAT_MAXD, TB_BITMAT_HSLOTS, TB_HASH_MAXD, true, 4>(g, tcnt, vacc, heavy,
+    tri_cta<TB_THREADS, TB_BITMAT_MAXD, TB_BITMAT_HSLOTS, TB_HASH_MAXD, true, 4>(g, A, counters[CNT_ADJ_ON], tcnt, vacc, heavy,
                                                                             counters[CNT_TRI_BIG],
                                                                             counters + CNT_TRI_BIG_NEXT, bits_maxd,
                                                                             hash_maxd);
@@ -379,14 +557,24 @@ void launch_stage1(Work &w, cudaStream_t st) {
     static const int occ_w = resident_ctas((const void *)k_tri_warp, TW_WARPS * 32, 0);
     static const int occ_c = resident_ctas((const void *)k_tri_cta, TS_THREADS, TS_SMEM);
     static const int occ_b = resident_ctas((const void *)k_tri_big, TB_THREADS, TB_SMEM);
-    launch_pdl(k_tri_warp, w.num_sms * min(w.tune[TUNE_GRID_TRI], occ_w), TW_WARPS * 32, 0, st, g, w.tcnt, w.vacc, w.lists,
-                                                                                       w.counters, maxd);
+    const AdjBits A = adj_bits(w);
+    if (adj_wanted(w.n, w.m)) {
+        launch_pdl(k_adj_bits, w.num_sms * 8, 256, 0, st, g, A, w.nrow, const_cast<unsigned *>(A.words),
+                   const_cast<unsigned short *>(A.prefix), w.counters);
+        after_launch(st, K_ADJ_BITS);
+    }
+    launch_pdl(k_tri_warp, w.num_sms * min(w.tune[TUNE_GRID_TRI], occ_w), TW_WARPS * 32, 0, st, g, A, w.tcnt, w.vacc, w.lists,
+               w.counters, maxd, w.coff, w.ntiles);
     after_launch(st, K_TRI_WARP);
     const int bits = w.tune[TUNE_TRI_BITS_MAXD], hash = w.tune[TUNE_TRI_HASH_MAXD];
-    launch_pdl(k_tri_cta, w.num_sms * occ_c, TS_THREADS, TS_SMEM, st, g, w.tcnt, w.vacc, w.lists, w.counters, bits, hash);
-    after_launch(st, K_TRI_CTA);
-    launch_pdl(k_tri_big, w.num_sms * occ_b, TB_THREADS, TB_SMEM, st, g, w.tcnt, w.vacc, w.lists, w.counters, bits, hash);
-    after_launch(st, K_TRI_BIG);
+    if (out_degree_above(maxd, w.m)) {
+        launch_pdl(k_tri_cta, w.num_sms * occ_c, TS_THREADS, TS_SMEM, st, g, A, w.tcnt, w.vacc, w.lists, w.counters, bits, hash);
+        after_launch(st, K_TRI_CTA);
+    }
+    if (out_degree_above(TS_MAXD, w.m)) {
+        launch_pdl(k_tri_big, w.num_sms * occ_b, TB_THREADS, TB_SMEM, st, g, A, w.tcnt, w.vacc, w.lists, w.counters, bits, hash);
+        after_launch(st, K_TRI_BIG);
+    }
 }
 
 void configure_stage1() {

@@ -21,10 +21,8 @@ constexpr int AW_WARPS = 8;
 constexpr int AS_MAXD = 256;   // out-degree handled by a 256-thread CTA (k_agg_cta)
 
 struct __align__(16) AggWarpSmem {
-    int hk[4 * AW_MAXD];   // N+(u) hash at load <= 1/4 (most probes are misses)
-    int hv[4 * AW_MAXD];
-    long long dc[AW_MAXD];
-    SegTab seg;
+    Filter filter;
+    long long dc[AW_MAXD];   // D12 sums of N+(u)
 };
 
 // Edge aggregates of u's out-edges; returns whether any has a triangle.
@@ -57,8 +55,74 @@ __device__ __forceinline__ bool edge_aggregates(const Graph &g, const int *tcnt,
     return a1 != 0;
 }
 
-__global__ void __launch_bounds__(AW_WARPS * 32, 8) k_agg_warp(Graph g, const int *tcnt, VAcc *vacc, int *heavy,
-                                                            int *counters, int maxd) {
+// One warp-tier root over the adjacency bitmap: the pairs of u's
+// out-neighbours whose edges to u close triangles are probed, as in Stage I.
+// A column's sum of t(u, row) - 1 and a row's sum of t(u, column) - 1 stay in
+// its lane.
+__device__ __forceinline__ void agg_root_probe(const Graph &g, const AdjBits &A, const int *tcnt, VAcc *vacc, int u, int s,
+                                               int dp) {
+    const int lane = lane_id();
+    const OutList L = out_list(g, A, s, dp);
+    const int t0 = lane < dp ? tcnt[s + lane] : 0, t1 = 32 + lane < dp ? tcnt[s + 32 + lane] : 0;
+    long long du12 = 0, d0 = 0, d1 = 0;   // D12 of u, of entries lane and 32 + lane
+    out_pairs(g, A, L, __ballot_sync(FULL, t0 > 0), __ballot_sync(FULL, t1 > 0), t0 > 0, t1 > 0,
+              [&](int b, int r, bool hit, int pos) {
+                  const int tr = __shfl_sync(FULL, b == 2 ? t1 : t0, r);   // t(u, row)
+                  const int tc = b == 0 ? t0 : t1;                         // t(u, column)
+                  // (32 counts of at most 2^20 fit 32 bits)
+                  const int sum = (int)__reduce_add_sync(FULL, (unsigned)(hit ? tc - 1 : 0));
+                  if (hit) {
+                      du12 += tcnt[pos] - 1;
+                      if (b == 0) d0 += tr - 1; else d1 += tr - 1;
+                  }
+                  if (lane == r) {
+                      if (b == 2) d1 += sum; else d0 += sum;
+                  }
+              });
+    du12 = warp_sum(du12);
+    if (lane == 0 && du12) add64(&vacc[u].D12, du12);
+    if (d0) add64(&vacc[L.w0].D12, d0);
+    if (d1) add64(&vacc[L.w1].D12, d1);
+}
+
+// One warp-tier root whose out-neighbours' rows are streamed past a filter of
+// N+(u), as in Stage I; only rows of edges with triangles.
+__device__ __forceinline__ void agg_root_stream(const Graph &g, const int *tcnt, VAcc *vacc, int u, int s, int dp,
+                                                AggWarpSmem &S) {
+    const int lane = lane_id();
+    int w0 = -1, w1 = -1;
+    bool in0 = false, in1 = false;   // entries with t(u, .) > 0
+    int2 r0 = make_int2(0, 0), r1 = r0;
+    auto fill = [&](int i, int &w, bool &in, int2 &r) {
+        if (i >= dp) return;
+        w = g.ncol[s + i];
+        in = tcnt[s + i] > 0;
+        if (!in || i == dp - 1) return;
+        const int4 rw = g.rinfo[w];
+        r = make_int2(rw.y, rw.z);
+    };
+    fill(lane, w0, in0, r0);
+    if (dp > 32) fill(32 + lane, w1, in1, r1);
+    S.filter.set(w0, w1, in0, in1);
+    S.dc[lane] = S.dc[32 + lane] = 0;
+    __syncwarp();
+    long long du12 = 0;
+    filter_walk_some(g.ncol, S.filter, r0, r1, [&](int j, int pos, int w) {
+        const int i = S.filter.find(w, dp);
+        if (i < 0) return;
+        add64(&S.dc[j], tcnt[s + i] - 1);   // t(u, w) - 1 -> v
+        du12 += tcnt[pos] - 1;              // t(v, w) - 1 -> u
+        add64(&S.dc[i], tcnt[s + j] - 1);   // t(u, v) - 1 -> w
+    });
+    du12 = warp_sum(du12);
+    if (lane == 0 && du12) add64(&vacc[u].D12, du12);
+    __syncwarp();
+    for (int i = lane; i < dp; i += 32)
+        if (S.dc[i]) add64(&vacc[g.ncol[s + i]].D12, S.dc[i]);
+}
+
+__global__ void __launch_bounds__(AW_WARPS * 32, 6) k_agg_warp(Graph g, AdjBits A, const int *tcnt, VAcc *vacc, int *heavy,
+                                                            int *counters, int maxd, const int *coff, int ntiles) {
     pdl_begin();
     __shared__ AggWarpSmem sm_all[AW_WARPS];
     AggWarpSmem &S = sm_all[threadIdx.x >> 5];
@@ -66,85 +130,107 @@ __global__ void __launch_bounds__(AW_WARPS * 32, 8) k_agg_warp(Graph g, const in
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     if (degree_overflow(counters)) return;
-    for (int u = gw; u < g.n; u += nw) {
-        const int4 ru = g.rinfo[u];
-        const int s = ru.y, e = ru.z, dp = e - s;
-        if (dp < 1) continue;
+    const bool probe = counters[CNT_ADJ_ON];
+    auto triangles = [&](int u, int s, int dp) {
+        if (probe) agg_root_probe(g, A, tcnt, vacc, u, s, dp);
+        else agg_root_stream(g, tcnt, vacc, u, s, dp, S);
+        __syncwarp();
+    };
+    auto root = [&](int u, int s, int dp) {
+        if (dp < 1) return;
         if (dp > maxd) {
             if (lane == 0) {
                 if (dp <= AS_MAXD) heavy[atomicAdd(&counters[CNT_AGG_HEAVY], 1)] = u;
                 else heavy[g.n - 1 - atomicAdd(&counters[CNT_AGG_BIG], 1)] = u;
             }
+            return;
+        }
+        if (edge_aggregates(g, tcnt, vacc, u, s, dp, lane, 32) && dp >= 2) triangles(u, s, dp);
+    };
+    // ids of low degree: four roots at a time, eight lanes each
+    const int low = low_degree_ids(g.n, nw, coff, ntiles);
+    for (long long u0 = 4ll * gw; u0 < low; u0 += 4ll * nw) {
+        const int u = (int)u0 + (lane >> 3);
+        int4 ru = make_int4(0, 0, 0, 0);
+        if (u < low) ru = g.rinfo[u];
+        const int dp = ru.z - ru.y;
+        if (!__any_sync(FULL, dp > min(SMALL_DP, maxd))) {
+            // edge aggregates of the four roots' out-edges
+            const int l = lane & 7;
+            const long long t = l < dp ? tcnt[ru.y + l] : 0;
+            if (!__any_sync(FULL, t != 0)) continue;
+            int w = -1;
+            int2 r = make_int2(0, 0);
+            long long a1 = t, a2 = t * t, a3 = 0;
+            if (t) {
+                w = g.ncol[ru.y + l];
+                const int4 rw = g.rinfo[w];
+                a3 = t * (rw.z - rw.x);
+                add64(&vacc[w].A1, t);
+                add64(&vacc[w].A2, t * t);
+                add64(&vacc[w].A3, t * (ru.z - ru.x));
+                if (l < dp - 1) r = make_int2(rw.y, rw.z);
+            }
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {
+                a1 += __shfl_xor_sync(FULL, a1, o);
+                a2 += __shfl_xor_sync(FULL, a2, o);
+                a3 += __shfl_xor_sync(FULL, a3, o);
+            }
+            if (l == 0 && a1) {
+                add64(&vacc[u].A1, a1);
+                add64(&vacc[u].A2, a2);
+                add64(&vacc[u].A3, a3);
+            }
+            if (!__any_sync(FULL, r.y - r.x > SMALL_ROW)) {
+                long long du12 = 0, dv = 0;
+                small_walk(g.ncol, w, r, [&](int pos, int x) {
+                    for (int i = l + 1; i < dp; ++i)
+                        if (g.ncol[ru.y + i] == x) {
+                            dv += tcnt[ru.y + i] - 1;               // t(u, w) - 1 -> v
+                            du12 += tcnt[pos] - 1;                  // t(v, w) - 1 -> u
+                            if (t > 1) add64(&vacc[x].D12, t - 1);  // t(u, v) - 1 -> w
+                        }
+                });
+                if (dv) add64(&vacc[w].D12, dv);
+                if (du12) add64(&vacc[u].D12, du12);
+                continue;
+            }
+            for (int q = 0; q < 4; ++q) {
+                const int s = __shfl_sync(FULL, ru.y, 8 * q), d = __shfl_sync(FULL, dp, 8 * q);
+                if (d >= 2 && __shfl_sync(FULL, (int)(a1 != 0), 8 * q)) triangles((int)u0 + q, s, d);
+            }
             continue;
         }
-        if (!edge_aggregates(g, tcnt, vacc, u, s, dp, lane, 32) || dp < 2) continue;
-        const unsigned mask = next_pow2(4 * dp) - 1;
-        for (int i = lane; i <= (int)mask; i += 32) S.hk[i] = -1;
-        for (int i = lane; i < AW_MAXD; i += 32) S.dc[i] = 0;
-        __syncwarp();
-        for (int i = lane; i < dp; i += 32) hset_insert(S.hk, S.hv, mask, g.ncol[s + i], i);
-        const int umax = g.ncol[e - 1];
-        __syncwarp();
-        long long du12 = 0;
-        for (int jb = 0; jb < dp - 1; jb += 32) {
-            const int j = jb + lane;
-            int len = 0, vs = 0;
-            if (j < dp - 1 && tcnt[s + j] > 0) {
-                const int4 rv = g.rinfo[g.ncol[s + j]];
-                vs = rv.y;
-                len = rv.z - rv.y;
-            }
-            int mypre;
-            const int total = seg_build(S.seg, vs, len, mypre);
-            seg_visit32<2>(g.ncol, S.seg, mypre, len, total, 0, [&](bool valid, int q, int pos, int w) {
-                const int i = (valid && w <= umax) ? hset_find(S.hk, S.hv, mask, w) : -1;
-                const bool hit = i >= 0;
-                if (!__any_sync(FULL, hit)) return;
-                const int jj = jb + q;
-                if (!hit) return;
-                add64(&S.dc[jj], tcnt[s + i] - 1);                           // t(u, w) - 1 -> v
-                du12 += tcnt[pos] - 1;                                       // t(v, w) - 1 -> u
-                atomicAdd((unsigned long long *)&S.dc[i], (unsigned long long)(tcnt[s + jj] - 1));  // t(u, v) - 1 -> w
-            });
-            __syncwarp();
-        }
-        du12 = warp_sum(du12);
-        if (lane == 0 && du12) add64(&vacc[u].D12, du12);
-        for (int i = lane; i < dp; i += 32)
-            if (S.dc[i]) add64(&vacc[g.ncol[s + i]].D12, S.dc[i]);
-        __syncwarp();
+        for (int q = 0; q < 4; ++q) root((int)u0 + q, __shfl_sync(FULL, ru.y, 8 * q), __shfl_sync(FULL, dp, 8 * q));
+    }
+    for (int u = low + gw; u < g.n; u += nw) {
+        const int4 ru = g.rinfo[u];
+        root(u, ru.y, ru.z - ru.y);
     }
 }
 
-// Roots above the warp tier: k_agg_cta (256 threads, dp <= AS_MAXD, about
-// 21 KB of shared memory, several CTAs per SM) and k_agg_big (1024 threads),
-// from the front and the back of the heavy list. Up to AB_BITMAT_MAXD the
-// triangles of u are kept as the upper half of a bit matrix R of N+(u) (as
-// in Stage I): a hit sets its bit and adds t(v, w) - 1 to u; R is then made
-// symmetric, and each y in N+(u) receives the sum over its neighbours z in
-// R of t(u, z) - 1 (t(u, .) cached in shared memory). Above that, a hash of
-// N+(u) up to AB_HASH_MAXD and per-triangle credits; binary searches beyond.
+// Roots above the warp tier: k_agg_cta (256 threads, dp <= AS_MAXD, several
+// CTAs per SM) and k_agg_big (1024 threads), from the front and the back of
+// the heavy list. Out-neighbours with a bitmap row are probed in blocks of 32
+// rows x 32 columns, a warp each: a column's and a row's sums stay in its
+// lane until the block ends. The rows of the others are streamed against a
+// hash of N+(u) up to AB_HASH_MAXD with a credit per triangle in shared
+// memory; above that, binary searches and credits in global memory.
 constexpr int AS_THREADS = 256;
 constexpr int AB_THREADS = 1024;
-constexpr int AB_BITMAT_MAXD = 1152;
-constexpr int AB_BITMAT_HSLOTS = 4096;
 constexpr int AB_HASH_MAXD = 8192;
-constexpr int ac_rowstride(int rows) { return ((rows + 31) / 32) | 1; }
-// dc (nloc x 8 B, hash-only mode), hash (2 x hslots ints), t(u, .) cache
-// (rows ints), per warp a segment table and 64 row indices, 4 work words, R.
-constexpr size_t ac_smem(int threads, int hslots, int nloc, int rows) {
-    return (size_t)nloc * 8 + (size_t)2 * hslots * 4 + (size_t)rows * 4 + (size_t)(threads / 32) * (sizeof(SegTab) + 128) +
-           16 + (size_t)rows * ac_rowstride(rows) * 4;
+// D12 sums (nloc x 8 B), hash (2 x hslots ints), a segment table per warp.
+constexpr size_t ac_smem(int threads, int hslots, int nloc) {
+    return (size_t)nloc * 8 + (size_t)2 * hslots * 4 + (size_t)(threads / 32) * sizeof(SegTab);
 }
-constexpr size_t AS_SMEM = ac_smem(AS_THREADS, 4 * AS_MAXD, 0, AS_MAXD);
-constexpr size_t AB_SMEM_BITS = ac_smem(AB_THREADS, AB_BITMAT_HSLOTS, 0, AB_BITMAT_MAXD);
-constexpr size_t AB_SMEM_HASH = ac_smem(AB_THREADS, 2 * AB_HASH_MAXD, AB_HASH_MAXD, 0);
-constexpr size_t AB_SMEM = AB_SMEM_BITS > AB_SMEM_HASH ? AB_SMEM_BITS : AB_SMEM_HASH;
+constexpr size_t AS_SMEM = ac_smem(AS_THREADS, 4 * AS_MAXD, AS_MAXD);
+constexpr size_t AB_SMEM = ac_smem(AB_THREADS, 2 * AB_HASH_MAXD, AB_HASH_MAXD);
 static_assert(AB_SMEM <= 227 * 1024, "k_agg_big shared memory");
 
-template <int THREADS, int BITMAT_MAXD, int BITMAT_HSLOTS, int HASH_MAXD, bool BACK, int HMUL>
-__device__ __forceinline__ void agg_cta(const Graph &g, const int *tcnt, VAcc *vacc, const int *heavy, int nh,
-                                        int *next, int bits_maxd, int hash_maxd) {
+template <int THREADS, int HASH_MAXD, int HSLOTS, bool BACK>
+__device__ __forceinline__ void agg_cta(const Graph &g, const AdjBits &A, bool probe, const int *tcnt, VAcc *vacc,
+                                        const int *heavy, int nh, int *next, int hash_maxd) {
     extern __shared__ __align__(16) unsigned char dsm[];
     constexpr int NW = THREADS / 32;
     __shared__ int any_tri;
@@ -159,38 +245,60 @@ __device__ __forceinline__ void agg_cta(const Graph &g, const int *tcnt, VAcc *v
         __syncthreads();
         if (!any_tri) continue;
         const bool use_hash = dp <= HASH_MAXD && dp <= hash_maxd;
-        const bool use_bits = use_hash && dp <= BITMAT_MAXD && dp <= bits_maxd;
-        unsigned H = use_hash ? next_pow2(HMUL * dp) : 0;   // hash load at most 1 / HMUL, within the carve:
-        const unsigned hcap = use_bits ? BITMAT_HSLOTS : 2 * HASH_MAXD;   // its mode's slots
-        if (H > hcap) H = hcap;
+        // rows js .. of N+(u) are probed in the bitmap, the ones before streamed
+        const int js = use_hash && probe ? lower_bound(g.ncol, s, e, A.base) - s : dp;
+        unsigned H = use_hash && js > 0 ? next_pow2(4 * dp) : 0;   // hash load at most 1/4, within the carve
+        if (H > HSLOTS) H = HSLOTS;
         const unsigned mask = H ? H - 1 : 0;
-        const int W = (dp + 31) >> 5, WP = W | 1;   // words per row of R, row stride
-        const int nloc = (use_hash && !use_bits) ? dp : 0;
-        const int nrow = use_bits ? dp : 0;
-        long long *dc = reinterpret_cast<long long *>(dsm);   // hash-only mode
+        const int W = (dp + 31) >> 5;
+        const int nloc = use_hash ? dp : 0;
+        long long *dc = reinterpret_cast<long long *>(dsm);   // D12 sums of N+(u)
         int *hk = reinterpret_cast<int *>(dc + ((nloc + 1) & ~1));   // 16-byte aligned buckets
         int *hv = hk + H;
-        int *T = hv + H;                                       // t(u, N+(u)[i]), bit-matrix mode
-        SegTab *segs = reinterpret_cast<SegTab *>(T + nrow);
-        int *work = reinterpret_cast<int *>(reinterpret_cast<unsigned short *>(segs + NW) + NW * 64);
-        unsigned *R = reinterpret_cast<unsigned *>(work + 4);
-        SegTab &seg = segs[wid];
+        SegTab &seg = reinterpret_cast<SegTab *>(hv + H)[wid];
         for (int i = threadIdx.x; i < (int)H; i += THREADS) hk[i] = -1;
         for (int i = threadIdx.x; i < nloc; i += THREADS) dc[i] = 0;
-        for (int i = threadIdx.x; i < nrow; i += THREADS) T[i] = tcnt[s + i];
-        if (use_bits)
-            for (int i = threadIdx.x; i < dp * WP; i += THREADS) R[i] = 0;
-        if (threadIdx.x < 4) work[threadIdx.x] = 0;
         __syncthreads();
-        if (use_hash)
+        if (H)
             for (int i = threadIdx.x; i < dp; i += THREADS) hset_insert(hk, hv, mask, g.ncol[s + i], i);
         const int umax = g.ncol[e - 1];
-        __syncthreads();
         long long du12 = 0;
-        for (int jb = 0; jb < dp - 1; jb += 32) {   // all warps share each chunk
+        if (js < dp) {
+            const int b0 = js >> 5;   // the first block of rows
+            for (int it = b0 * (b0 + 1) / 2 + wid; it < W * (W + 1) / 2; it += NW) {
+                int t, jb;
+                block_pair(it, t, jb);
+                if (jb < b0) continue;
+                const int i = 32 * t + lane, j = 32 * jb + lane;
+                const int tc = i < dp ? tcnt[s + i] : 0, tr = j >= js && j < dp - 1 ? tcnt[s + j] : 0;   // t(u, .)
+                const int k = i < dp ? g.n - 1 - g.ncol[s + i] : 0;
+                int roff = 0, ry = 0;
+                if (tr > 0) {
+                    const int v = g.ncol[s + j];
+                    roff = A.row(v);
+                    ry = g.rinfo[v].y;
+                }
+                unsigned rsum = 0, csum = 0;   // 32 counts of at most 2^20 each
+                adj_probe<8>(A, __ballot_sync(FULL, tr > 0), roff, k, tc > 0, t == jb,
+                             [&](int r, bool hit, int at, unsigned word) {
+                                 const int y = __shfl_sync(FULL, ry, r), tw = __shfl_sync(FULL, tr, r);
+                                 const unsigned sum = __reduce_add_sync(FULL, (unsigned)(hit ? tc - 1 : 0));
+                                 if (lane == r) rsum = sum;
+                                 if (hit) {
+                                     csum += tw - 1;                                // t(u, v) - 1 -> w
+                                     du12 += tcnt[y + A.rank(at, k, word)] - 1;     // t(v, w) - 1 -> u
+                                 }
+                             });
+                if (rsum) add64(&dc[j], rsum);   // t(u, w) - 1 -> v
+                if (csum) add64(&dc[i], csum);
+            }
+        }
+        __syncthreads();
+        const int jend = min(js, dp - 1);
+        for (int jb = 0; jb < jend; jb += 32) {   // all warps share each chunk
             const int j = jb + lane;
             int len = 0, vs = 0;
-            if (j < dp - 1 && tcnt[s + j] > 0) {
+            if (j < jend && tcnt[s + j] > 0) {
                 const int4 rv = g.rinfo[g.ncol[s + j]];
                 vs = rv.y;
                 len = rv.z - rv.y;
@@ -207,84 +315,39 @@ __device__ __forceinline__ void agg_cta(const Graph &g, const int *tcnt, VAcc *v
                         i = p < 0 ? -1 : p - s;
                     }
                 }
-                const bool hit = i >= 0;
-                if (!__any_sync(FULL, hit)) return;
+                if (i < 0) return;
                 const int jj = jb + q;
-                if (hit) du12 += tcnt[pos] - 1;   // t(v, w) - 1 -> u
-                if (use_bits) {
-                    if (hit) atomicOr(&R[jj * WP + (i >> 5)], 1u << (i & 31));
-                    return;
-                }
-                if (!hit) return;
-                add64(use_hash ? &dc[jj] : &vacc[g.ncol[s + jj]].D12, tcnt[s + i] - 1);   // t(u, w) - 1 -> v
-                const long long tw = tcnt[s + jj] - 1;                                      // t(u, v) - 1 -> w
-                if (use_hash) atomicAdd((unsigned long long *)&dc[i], (unsigned long long)tw);
-                else add64(&vacc[w].D12, tw);
+                du12 += tcnt[pos] - 1;                                                     // t(v, w) - 1 -> u
+                const long long tv = tcnt[s + i] - 1, tw = tcnt[s + jj] - 1;
+                add64(use_hash ? &dc[jj] : &vacc[g.ncol[s + jj]].D12, tv);                 // t(u, w) - 1 -> v
+                add64(use_hash ? &dc[i] : &vacc[w].D12, tw);                               // t(u, v) - 1 -> w
             });
             __syncwarp();
         }
-        __syncthreads();
         du12 = warp_sum(du12);
         if (lane == 0 && du12) add64(&vacc[u].D12, du12);
-        if (use_bits) {
-            // mirror R (a ballot transpose per 32 x 32 block), then y in N+(u)
-            // receives the sum over its neighbours z in R of t(u, z) - 1
-            const int nblk = W * (W + 1) / 2;
-            for (int bidx = wid; bidx < nblk; bidx += NW) {
-                int bj = 0, rem = bidx;
-                while (rem >= W - bj) {
-                    rem -= W - bj;
-                    ++bj;
-                }
-                const int bi = bj + rem;
-                const int jr = bj * 32 + lane;
-                const unsigned wv = jr < dp ? R[jr * WP + bi] : 0u;
-                unsigned tv = 0;
-                for (int k = 0; k < 32; ++k) {
-                    const unsigned b = __ballot_sync(FULL, (wv >> k) & 1u);
-                    if (lane == k) tv = b;
-                }
-                const int ir = bi * 32 + lane;
-                if (ir < dp) {
-                    if (bi == bj) R[ir * WP + bj] = wv | tv;
-                    else if (tv) R[ir * WP + bj] |= tv;
-                }
-                __syncwarp();
-            }
-            __syncthreads();
-            for (int y = wid; y < dp; y += NW) {
-                const unsigned *ry = R + y * WP;
-                long long c = 0;
-                for (int t = 0; t < W; ++t) {
-                    const int z = t * 32 + lane;
-                    if ((ry[t] >> lane) & 1u) c += T[z] - 1;
-                }
-                c = warp_sum(c);
-                if (lane == 0 && c) add64(&vacc[g.ncol[s + y]].D12, c);
-            }
-        }
+        __syncthreads();
         for (int i = threadIdx.x; i < nloc; i += THREADS)
             if (dc[i]) add64(&vacc[g.ncol[s + i]].D12, dc[i]);
         __syncthreads();
     }
 }
 
-__global__ void __launch_bounds__(AS_THREADS) k_agg_cta(Graph g, const int *tcnt, VAcc *vacc, const int *heavy,
-                                                        int *counters, int bits_maxd, int hash_maxd) {
+__global__ void __launch_bounds__(AS_THREADS) k_agg_cta(Graph g, AdjBits A, const int *tcnt, VAcc *vacc, const int *heavy,
+                                                        int *counters, int hash_maxd) {
     pdl_begin();
     if (degree_overflow(counters)) return;
-    agg_cta<AS_THREADS, AS_MAXD, 4 * AS_MAXD, AS_MAXD, false, 4>(g, tcnt, vacc, heavy, counters[CNT_AGG_HEAVY],
-                                                            counters + CNT_AGG_CTA_NEXT, bits_maxd, hash_maxd);
+    agg_cta<AS_THREADS, AS_MAXD, 4 * AS_MAXD, false>(g, A, counters[CNT_ADJ_ON], tcnt, vacc, heavy,
+                                                     counters[CNT_AGG_HEAVY], counters + CNT_AGG_CTA_NEXT, hash_maxd);
 }
 
-__global__ void __launch_bounds__(AB_THREADS) k_agg_big(Graph g, const int *tcnt, VAcc *vacc, const int *heavy,
-                                                        int *counters, int bits_maxd, int hash_maxd) {
+__global__ void __launch_bounds__(AB_THREADS) k_agg_big(Graph g, AdjBits A, const int *tcnt, VAcc *vacc, const int *heavy,
+                                                        int *counters, int hash_maxd) {
     pdl_begin();
     if (degree_overflow(counters)) return;
-    agg_cta<AB_THREADS, AB_BITMAT_MAXD, AB_BITMAT_HSLOTS, AB_HASH_MAXD, true, 4>(g, tcnt, vacc, heavy,
-                                                                            counters[CNT_AGG_BIG],
-                                                                            counters + CNT_AGG_BIG_NEXT, bits_maxd,
-                                                                            hash_maxd);
+    agg_cta<AB_THREADS, AB_HASH_MAXD, 2 * AB_HASH_MAXD, true>(g, A, counters[CNT_ADJ_ON], tcnt, vacc, heavy,
+                                                              counters[CNT_AGG_BIG], counters + CNT_AGG_BIG_NEXT,
+                                                              hash_maxd);
 }
 
 void launch_stage2(Work &w, cudaStream_t st) {
@@ -294,14 +357,19 @@ void launch_stage2(Work &w, cudaStream_t st) {
     static const int occ_w = resident_ctas((const void *)k_agg_warp, AW_WARPS * 32, 0);
     static const int occ_c = resident_ctas((const void *)k_agg_cta, AS_THREADS, AS_SMEM);
     static const int occ_b = resident_ctas((const void *)k_agg_big, AB_THREADS, AB_SMEM);
-    launch_pdl(k_agg_warp, w.num_sms * min(w.tune[TUNE_GRID_AGG], occ_w), AW_WARPS * 32, 0, st, g, w.tcnt, w.vacc, heavy,
-                                                                                       w.counters, maxd);
+    const AdjBits A = adj_bits(w);
+    launch_pdl(k_agg_warp, w.num_sms * min(w.tune[TUNE_GRID_AGG], occ_w), AW_WARPS * 32, 0, st, g, A, w.tcnt, w.vacc, heavy,
+               w.counters, maxd, w.coff, w.ntiles);
     after_launch(st, K_AGG_WARP);
-    const int bits = w.tune[TUNE_TRI_BITS_MAXD], hash = w.tune[TUNE_TRI_HASH_MAXD];
-    launch_pdl(k_agg_cta, w.num_sms * occ_c, AS_THREADS, AS_SMEM, st, g, w.tcnt, w.vacc, heavy, w.counters, bits, hash);
-    after_launch(st, K_AGG_CTA);
-    launch_pdl(k_agg_big, w.num_sms * occ_b, AB_THREADS, AB_SMEM, st, g, w.tcnt, w.vacc, heavy, w.counters, bits, hash);
-    after_launch(st, K_AGG_BIG);
+    const int hash = w.tune[TUNE_TRI_HASH_MAXD];
+    if (out_degree_above(maxd, w.m)) {
+        launch_pdl(k_agg_cta, w.num_sms * occ_c, AS_THREADS, AS_SMEM, st, g, A, w.tcnt, w.vacc, heavy, w.counters, hash);
+        after_launch(st, K_AGG_CTA);
+    }
+    if (out_degree_above(AS_MAXD, w.m)) {
+        launch_pdl(k_agg_big, w.num_sms * occ_b, AB_THREADS, AB_SMEM, st, g, A, w.tcnt, w.vacc, heavy, w.counters, hash);
+        after_launch(st, K_AGG_BIG);
+    }
 }
 
 void configure_stage2() {
