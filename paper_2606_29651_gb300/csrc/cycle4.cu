@@ -11,13 +11,16 @@
 //   u gets sum_w C(c_w, 2), w gets C(c_w, 2),
 //   each middle vertex v gets sum over its wedges of (c_w - 1).
 // The wedges through v are the entries of row v below u: a prefix of row v
-// ending at the position of u, which a search of N+(v) finds. Roots are
-// routed by their wedge count W (a count is at most W too): one warp with a
-// 6 KB table (k_c4_warp) or an 8 KB one (k_c4_warp_big), four warps
-// (k_c4_mid, packed or split tables), a 512-thread CTA (k_c4_cta), or, for the largest
-// roots, and for every root with more than WL_MAXD in-neighbours, a CTA with
-// a directly indexed counter per key in shared memory (k_c4_tiled). The other tables are open-addressing hash
-// tables in shared memory, either split (key and count arrays) or packed
+// ending at the position of u, which a search of N+(v) finds. Roots with few
+// repeated keys need no counts: a Bloom filter finds the keys that may repeat
+// (k_c4_filter). The others are routed by their wedge count W (a count is at
+// most W too): one warp with a 6 or 8 KB table (k_c4_warp_left; k_c4_warp in
+// small graphs, which go without the filter), four warps (k_c4_mid, packed or
+// split tables), a 512-thread CTA (k_c4_cta), or, for the largest roots, and
+// for every root with more than WL_MAXD in-neighbours, a CTA with a directly
+// indexed counter per key in shared memory (k_c4_tiled). The other tables are
+// open-addressing hash tables in shared memory, either split (key and count
+// arrays) or packed
 // (key << cb | count in one 32-bit word, cb = 32 - bits(n - 1) count bits,
 // usable while W < 2^cb - 1), which holds twice the keys in the same space.
 // Each table is emptied once per CTA; afterwards a warp sweeps the region
@@ -31,11 +34,11 @@ namespace niorca {
 
 constexpr int CW_WARPS = 4;
 constexpr int CW_WORDS = 1536;      // table words per warp of k_c4_warp: 6 KB, 8 CTAs of 4 warps per SM
-constexpr int CWB_WORDS = 2048;     // k_c4_warp_big: 8 KB, 6 CTAs per SM
+constexpr int CWB_WORDS = 2048;     // split tables: 8 KB, 6 CTAs per SM
 constexpr int CW_MAXW = 1536;       // largest W of a root in the warp tiers
-constexpr int CW_SMALL_MAXW = 256;  // the same, for graphs with fewer vertices than resident warps
+constexpr int CW_SMALL_MAXW = 32;  // the same, for graphs with fewer vertices than resident warps
 constexpr int CW_DUPS = 32;         // repeated keys a warp credits by search at most
-constexpr int CW_BIG_LIST = 0;      // list slot of k_c4_warp_big's roots: the triangle stage's heavy list,
+constexpr int CW_LEFT_LIST = 0;     // list slot of the roots of k_c4_warp_left: the triangle heavy list,
                                     // which nothing reads after that stage
 constexpr int CM_THREADS = 128;
 constexpr int CM_SLOTS = 4096;      // split; 8192 when packed
@@ -504,122 +507,282 @@ struct __align__(16) C4WarpSmem {
 __host__ __device__ constexpr int cw_slots(bool split, int words) { return split ? words / 2 : words; }
 __host__ __device__ constexpr int cw_maxw(bool split, int words) { return cw_slots(split, words) / 4 * 3; }
 
-// One warp per root. k_c4_warp (BIG = false) takes every vertex as a root:
-// those with W up to 3/4 of its 6 KB table are counted there, those that
-// fit the 8 KB table of k_c4_warp_big (BIG = true) are queued for it, the
-// rest for the wider tiers. SPLIT: (key, count) pair tables, for graphs
-// whose ids leave a packed word too few count bits.
-template <bool SPLIT, bool BIG>
-__device__ __forceinline__ void c4_warp_body(Graph g, VAcc *vacc, int *lists, int *counters, int maxw, int cb,
-                                             int teamw, const int *coff, int ntiles) {
-    if (degree_overflow(counters)) return;
-    if (!BIG) teamw = ck_min_wedges(coff, ntiles, g.n, teamw);
-    constexpr int WORDS = BIG ? CWB_WORDS : CW_WORDS;
-    constexpr int TS = cw_slots(SPLIT, WORDS);
-    __shared__ C4WarpSmem<WORDS> sm_all[CW_WARPS];
-    C4WarpSmem<WORDS> &S = sm_all[threadIdx.x >> 5];
+// ---- roots with few repeated keys, without counting
+//
+// Most roots of a large sparse graph have no repeated key (G(1e6, mean degree
+// 32): 0.03 per root of 256 wedges), and to learn that a root needs no table
+// of counts: a blocked Bloom filter does, one atomic per wedge with no probe
+// loop (a key clears three bits of one word, and one that finds them clear
+// may be a repeat). Which in-neighbours have each of those, and with that the
+// exact counts and the middle vertices, then comes from searching their rows
+// (few pairs), or from a second walk past a table of the keys alone: a chain
+// of searches took 10 us for the largest roots of G(12000, mean degree 15). A
+// root with more than CW_DUPS of them goes to a table of counts. The filter
+// is all ones when empty, like a table's keys.
+// One root of W wedges in a random graph repeats W^2 / 2n keys. Up to 24 of
+// them the filter is the better start: with the line at 4, 12, 24 calls on
+// G(80000, 40) took 786, 685, 529 us, G(30000, 30) 301, 280, 273, power-law
+// graphs of 17000 vertices, whose keys repeat more, 321, 332, 338 (before the
+// filter: 849, 324, 500).
+__device__ __forceinline__ bool c4_few_repeats(long long W, int n) { return W * W <= 48ll * n; }
+
+// (key, in-neighbour) pairs up to which they are searched, four rounds: G(1e6,
+// mean degree 32), whose roots have few, 2820 us a call at 32, 2790 at 64,
+// 2754 at 128, 2744 at 256; 8192 small graphs, with many, 12234, 12242, 12269,
+// 12335.
+constexpr int C4_SEARCH = 128;
+
+template <int LOG>
+__device__ __forceinline__ unsigned hash_top(int w) { return (unsigned)w * 0x9E3779B1u >> (32 - LOG); }
+
+__device__ __forceinline__ bool bloom_add(unsigned *t, int log_words, int w) {
+    const unsigned h = (unsigned)w * 0x9E3779B1u, b = h << 10;
+    const unsigned mask = __funnelshift_l(0u, 1u, b >> 27) | __funnelshift_l(0u, 1u, b >> 22) | __funnelshift_l(0u, 1u, b >> 17);
+    return (atomicAnd(&t[h >> (32 - log_words)], ~mask) & mask) == 0;
+}
+
+// The wedges of a root of at most 64 in-neighbours (lane: the segments s0 and
+// s1 of in-neighbours lane and 32 + lane): eight rows at a time, eight lanes
+// and two rows each, f(w[4], pa, pc) with the keys of in-neighbour pa in
+// w[0..1] and of pc in w[2..3] (-1: none), by the whole warp.
+template <class F>
+__device__ __forceinline__ void c4_rows(const int *__restrict__ col, int din, int2 s0, int2 s1, F f) {
+    const int sub = lane_id() & 7, q = lane_id() >> 3;
+    for (int jb = 0; jb < din; jb += 8) {
+        const int2 s = jb < 32 ? s0 : s1;
+        const int ja = (jb + q) & 31, jc = (jb + 4 + q) & 31;
+        const int xa = __shfl_sync(FULL, s.x, ja), na = __shfl_sync(FULL, s.y, ja);
+        const int xc = __shfl_sync(FULL, s.x, jc), nc = __shfl_sync(FULL, s.y, jc);
+        const int longest = (int)__reduce_max_sync(FULL, (unsigned)max(na, nc));
+        for (int o = sub; o - sub < longest; o += 16) {
+            int w[4];
+            w[0] = o < na ? __ldg(col + xa + o) : -1;
+            w[1] = o + 8 < na ? __ldg(col + xa + o + 8) : -1;
+            w[2] = o < nc ? __ldg(col + xc + o) : -1;
+            w[3] = o + 8 < nc ? __ldg(col + xc + o + 8) : -1;
+            f(w, jb + q, jb + 4 + q);
+        }
+    }
+}
+
+// One root of at most 64 in-neighbours, the warp (segments as in c4_rows).
+// False if too many keys may repeat (nothing is credited then).
+template <int LOG, class Smem>
+__device__ __forceinline__ bool c4_bloom_root(const Graph &g, VAcc *vacc, int u, int b, int din, int2 s0, int2 s1, Smem &S) {
     const int lane = lane_id();
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    const long long pack_lim = (1ll << cb) - 2;   // largest W a packed count may reach
-    const long long warp_cap = SPLIT ? maxw : (maxw < pack_lim ? maxw : pack_lim);   // W the warp tiers take
-    const long long here_lim = warp_cap < cw_maxw(SPLIT, WORDS) ? warp_cap : cw_maxw(SPLIT, WORDS);
-    const long long big_lim = warp_cap < cw_maxw(SPLIT, CWB_WORDS) ? warp_cap : cw_maxw(SPLIT, CWB_WORDS);
-    int *const big_roots = lists + (size_t)CW_BIG_LIST * g.n;
-    const int count = BIG ? counters[CNT_C4_WBIG] : g.n;
-    auto root = [&](int i) { return BIG ? big_roots[i] : i; };
-    int *const sk = reinterpret_cast<int *>(S.t), *const sc = sk + TS;   // split keys, counts
-    if (SPLIT) SplitTab{sk, sc, (unsigned)TS, nullptr}.clear_all(lane, 32);
-    else PackedTab{S.t, (unsigned)TS, cb, nullptr}.clear_all(lane, 32);
+    const int *__restrict__ col = g.ncol;
+    int nd = 0;   // keys that may repeat (warp-uniform), the first CW_DUPS of them in S.dups
+    c4_rows(col, din, s0, s1, [&](const int (&w)[4], int, int) {
+        bool may[4], any = false;
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            may[h] = w[h] >= 0 && bloom_add(S.t, LOG, w[h]);
+            any |= may[h];
+        }
+        if (!__any_sync(FULL, any)) return;
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            const unsigned r = __ballot_sync(FULL, may[h]);
+            const int at = nd + __popc(r & lanemask_lt());
+            if (may[h] && at < CW_DUPS) S.dups[at] = w[h];
+            nd += __popc(r);
+        }
+    });
     __syncwarp();
-    // Software pipeline over the warp's roots i, i + nw, i + 2 nw: row bounds
-    // are loaded two roots ahead, the first 32 in-neighbours and their row
-    // bounds one root ahead, so that a root starts with its data in flight.
+#pragma unroll
+    for (int i = 0; i < (1 << LOG) / 128; ++i)
+        reinterpret_cast<uint4 *>(S.t)[32 * i + lane] = make_uint4(EMPTY, EMPTY, EMPTY, EMPTY);
+    if (nd > 0 && nd <= CW_DUPS) {
+        // the different ones among them
+        const int key = lane < nd ? S.dups[lane] : -1 - lane;
+        const unsigned same = __match_any_sync(FULL, key);
+        const bool first = lane < nd && lane == __ffs(same) - 1;
+        const unsigned firsts = __ballot_sync(FULL, first);
+        const int nk = __popc(firsts);
+        __syncwarp();
+        if (first) S.dups[__popc(firsts & lanemask_lt())] = key;
+        unsigned *const common = reinterpret_cast<unsigned *>(S.pv);   // per key, a bit per in-neighbour
+        S.pv[lane] = 0;
+        __syncwarp();
+        if (nk * din <= C4_SEARCH) {
+            // one (key, in-neighbour) pair per lane, all searches independent
+            for (int t = lane; t < nk * din; t += 32) {
+                const int k = t / din, p = t - k * din;
+                const int4 rw = g.rinfo[S.dups[k]];
+                if (find_sorted(col, rw.x, rw.z, col[b + p]) >= 0) atomicOr(&common[2 * k + (p >> 5)], 1u << (p & 31));
+            }
+        } else {
+            // the rows once more, past a table of the keys (at most 32 in 1 << LOG slots)
+            constexpr unsigned MASK = (1u << LOG) - 1;
+            unsigned at = 0;
+            if (lane < nk) {
+                at = hash_top<LOG>(S.dups[lane]);
+                while (atomicCAS(&S.t[at], EMPTY, (unsigned)lane) != EMPTY) at = (at + 1) & MASK;
+            }
+            __syncwarp();
+            c4_rows(col, din, s0, s1, [&](const int (&w)[4], int pa, int pc) {
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    const int p = h < 2 ? pa : pc;
+                    unsigned x = hash_top<LOG>(w[h]), k;
+                    if (w[h] >= 0)
+                        for (; (k = S.t[x]) != EMPTY; x = (x + 1) & MASK)
+                            if (S.dups[k] == w[h]) {
+                                atomicOr(&common[2 * k + (p >> 5)], 1u << (p & 31));
+                                break;
+                            }
+                }
+            });
+            __syncwarp();
+            if (lane < nk) S.t[at] = EMPTY;
+        }
+        __syncwarp();
+        const int c = lane < nk ? __popc(common[2 * lane]) + __popc(common[2 * lane + 1]) : 0;
+        if (__any_sync(FULL, c >= 2)) {
+            if (c >= 2) add64(&vacc[S.dups[lane]].C4, c2(c));
+            const long long su = warp_sum(c2(c));
+            if (lane == 0) add64(&vacc[u].C4, su);
+            for (int t = lane; t < nk * din; t += 32) {
+                const int k = t / din, p = t - k * din;
+                const int ck = __popc(common[2 * k]) + __popc(common[2 * k + 1]);
+                if (ck >= 2 && (common[2 * k + (p >> 5)] >> (p & 31)) & 1u) add64(&vacc[col[b + p]].C4, ck - 1);
+            }
+        }
+    }
+    __syncwarp();
+    return nd <= CW_DUPS;
+}
+
+// Four roots of at most 8 in-neighbours each (lane 8 q + l: wedge segment s of
+// in-neighbour l of root q; its row bounds ru): every lane walks its own
+// segment past a filter of 32 words per root. False if a root has too many
+// keys that may repeat (nothing is credited then).
+template <class Smem>
+__device__ __forceinline__ bool c4_bloom_small(const Graph &g, VAcc *vacc, int u, int4 ru, int2 s, Smem &S) {
+    const int lane = lane_id(), l = lane & 7, q = lane >> 3;
+    const unsigned group = 0xffu << (8 * q);
+    const int *__restrict__ col = g.ncol;
+    int *const list = S.dups + 16 * q;   // at most 16 keys per root
+    int nd = 0;
+    const int longest = (int)__reduce_max_sync(FULL, (unsigned)s.y);
+    int w = s.y > 0 ? __ldg(col + s.x) : -1;
+    for (int o = 0; o < longest; ++o) {
+        const int next = o + 1 < s.y ? __ldg(col + s.x + o + 1) : -1;
+        const bool may = w >= 0 && bloom_add(S.t + 32 * q, 5, w);
+        const unsigned r = __ballot_sync(FULL, may);
+        if (r) {
+            const int at = nd + __popc(r & group & lanemask_lt());
+            if (may && at < 16) list[at] = w;
+            nd += __popc(r & group);
+        }
+        w = next;
+    }
+    __syncwarp();
+    reinterpret_cast<uint4 *>(S.t)[lane] = make_uint4(EMPTY, EMPTY, EMPTY, EMPTY);
+    __syncwarp();
+    const int most = (int)__reduce_max_sync(FULL, (unsigned)nd);
+    if (most > 16) return false;
+    const int din = ru.y - ru.x;
+    const int v = most > 0 && l < din ? col[ru.x + l] : -1;
+    for (int k = 0; k < most; ++k) {   // key k of every root
+        const int key = k < nd ? list[k] : -1;
+        const bool seen = key >= 0 && ((l < k && list[l] == key) || (l + 8 < k && list[l + 8] == key));
+        const bool again = (__ballot_sync(FULL, seen) & group) != 0;
+        bool in = false;
+        if (key >= 0 && !again && v >= 0) {
+            const int4 rw = g.rinfo[key];
+            in = find_sorted(col, rw.x, rw.z, v) >= 0;
+        }
+        const int c = __popc(__ballot_sync(FULL, in) & group);
+        if (c < 2) continue;
+        if (in) add64(&vacc[v].C4, c - 1);
+        if (l < 2) add64(&vacc[l ? key : u].C4, c2(c));
+    }
+    __syncwarp();
+    return true;
+}
+
+// Limits of the tiers by wedge count W. A table takes W up to 3/4 of its slots
+// (SPLIT: (key, count) pairs, for graphs whose ids leave a packed word too
+// few count bits), and a packed count must not reach its field's end.
+template <bool SPLIT>
+struct C4Limits {
+    long long pack, warp, team;   // packed tables, a warp's table, key-tiled from here on
+    __device__ __forceinline__ C4Limits(int maxw, int cb, int teamw) {
+        pack = (1ll << cb) - 2;
+        const long long cap = SPLIT ? maxw : (maxw < pack ? maxw : pack);   // W the warp tiers take
+        constexpr int most = cw_maxw(SPLIT, SPLIT ? CWB_WORDS : CW_WORDS);
+        warp = cap < most ? cap : most;
+        team = teamw;
+    }
+};
+
+// The wedge segments of a root's in-neighbours lane and 32 + lane (din <= 64;
+// s0 is loaded) and its wedge count W, for any din.
+__device__ __forceinline__ long long c4_wedges(const Graph &g, int b, int din, int2 s0, int2 &s1) {
+    const int lane = lane_id();
+    s1 = make_int2(0, 0);
+    if (din <= 64) {
+        if (32 + lane < din) s1 = g.wl[b + 32 + lane];
+        return __reduce_add_sync(FULL, (unsigned)(s0.y + s1.y));   // W <= m < 2^31
+    }
+    long long W = 0;
+    if (din <= WL_MAXD) {
+        for (int p = lane; p < din; p += 32) W += g.wl[b + p].y;
+    } else {
+        // more in-neighbours than the wedge-segment table covers: the
+        // key-tiled tier, which takes any root, without searching every row
+        // for W here (one warp for a hub's rows would be the kernel's tail);
+        // its order takes the in-neighbours' degree sum, at least W, in W's
+        // place
+#pragma unroll 8
+        for (int p = lane; p < din; p += 32) {
+            const int4 rv = g.rinfo[g.ncol[b + p]];
+            W += rv.z - rv.x;
+        }
+    }
+    return warp_sum(W);
+}
+
+// Queues a root for another kernel: k_c4_warp_left (`warp`: that is the next
+// one), or a wider tier's.
+template <bool SPLIT>
+__device__ __forceinline__ void c4_queue_root(const Graph &g, int *lists, int *counters, int u, int din, long long W, bool warp,
+                                              const C4Limits<SPLIT> &lim) {
+    if (lane_id() != 0) return;
+    int which, list;   // queue counter and list slot (lists + list * n)
+    if (din > WL_MAXD) { which = CNT_C4_TEAM; list = 4; }
+    else if (warp && W <= lim.warp) { which = CNT_C4_LEFT; list = CW_LEFT_LIST; }
+    else if (W > lim.team) { which = CNT_C4_TEAM; list = 4; }
+    else if (W <= 2 * CM_MAXW && W <= lim.pack) { which = CNT_C4_MIDP; list = 5; }
+    else if (W <= CM_MAXW) { which = CNT_C4_MID; list = 2; }
+    else { which = CNT_C4_CTA; list = 3; }
+    const int at = atomicAdd(&counters[which], 1);
+    lists[(size_t)list * g.n + at] = u;
+    if (which == CNT_C4_TEAM)   // the order of the key-tiled tier
+        lists[(size_t)g.n + at] = (int)(W < 0x7fffffffll ? W : 0x7fffffffll);
+}
+
+// The roots i = first, first + nw, ... < count of a warp, f(u, row bounds,
+// wedge segment of in-neighbour `lane`), in a software pipeline: row bounds
+// are loaded two roots ahead, the first 32 segments one root ahead.
+template <class R, class F>
+__device__ __forceinline__ void c4_roots(const Graph &g, int first, int nw, int count, R root, F f) {
+    const int lane = lane_id();
     const int4 Z = make_int4(0, 0, 0, 0);
-    int i = gw;
+    const int2 Z2 = make_int2(0, 0);
+    int i = first;
     int u = i < count ? root(i) : 0;
     int un = i + nw < count ? root(i + nw) : 0;
     int4 ru = i < count ? g.rinfo[u] : Z;
     int4 ru1 = i + nw < count ? g.rinfo[un] : Z;
-    const int2 Z2 = make_int2(0, 0);
-    // wedge segment through in-neighbour `lane` of the current root
     int2 s0 = (i < count && lane < ru.y - ru.x && ru.y - ru.x <= 64) ? g.wl[ru.x + lane] : Z2;
     for (; i < count; i += nw) {
         const int i2 = i + 2 * nw;
         const int u2 = i2 < count ? root(i2) : 0;
         const int4 ru2 = i2 < count ? g.rinfo[u2] : Z;
         const int2 s1 = (i + nw < count && lane < ru1.y - ru1.x && ru1.y - ru1.x <= 64) ? g.wl[ru1.x + lane] : Z2;
-        [&] {
-            const int b = ru.x, din = ru.y - ru.x;
-            if (din < 2) return;
-            long long W = 0;   // exact wedge count W of root u
-            RootChunks rc;
-            if (din <= 64) {   // both chunks' segments stay in registers
-                rc.v0 = lane < din ? g.ncol[b + lane] : -1;   // for the middle walk's credits
-                rc.st0 = s0.x;
-                rc.len0 = s0.y;
-                if (din <= 32) {   // one chunk: its segment table gives W
-                    rc.have = 1;
-                    rc.total0 = seg_build(S.seg, rc.st0, rc.len0, rc.pre0);
-                    rc.built0 = true;
-                    W = rc.total0;
-                } else {
-                    rc.have = 2;
-                    if (32 + lane < din) {
-                        rc.v1 = g.ncol[b + 32 + lane];
-                        const int2 sl = g.wl[b + 32 + lane];
-                        rc.st1 = sl.x;
-                        rc.len1 = sl.y;
-                    }
-                    W = warp_sum(rc.len0 + rc.len1);
-                }
-            } else if (din <= WL_MAXD) {
-                for (int p = lane; p < din; p += 32) W += g.wl[b + p].y;
-                W = warp_sum(W);
-            } else {
-                // more in-neighbours than the wedge-segment table covers: the
-                // key-tiled tier, which takes any root, without searching every
-                // row for W here (one warp for a hub's rows would be the
-                // kernel's tail); its order takes the in-neighbours' degree
-                // sum, at least W, in W's place
-#pragma unroll 8
-                for (int p = lane; p < din; p += 32) {
-                    const int4 rv = g.rinfo[g.ncol[b + p]];
-                    W += rv.z - rv.x;
-                }
-                W = warp_sum(W);
-            }
-            const bool hub = din > WL_MAXD;
-            if (W < 2 && !hub) return;
-            if (W > here_lim || hub) {
-                if (lane == 0) {
-                    int which, list;   // queue counter and list slot (lists + list * n)
-                    if (hub) { which = CNT_C4_TEAM; list = 4; }
-                    else if (!BIG && W <= big_lim) { which = CNT_C4_WBIG; list = CW_BIG_LIST; }
-                    else if (W > teamw) { which = CNT_C4_TEAM; list = 4; }
-                    else if (W <= 2 * CM_MAXW && W <= pack_lim) { which = CNT_C4_MIDP; list = 5; }
-                    else if (W <= CM_MAXW) { which = CNT_C4_MID; list = 2; }
-                    else { which = CNT_C4_CTA; list = 3; }
-                    const int at = atomicAdd(&counters[which], 1);
-                    lists[(size_t)list * g.n + at] = u;
-                    if (which == CNT_C4_TEAM)   // the order of the key-tiled tier
-                        lists[(size_t)g.n + at] = (int)(W < 0x7fffffffll ? W : 0x7fffffffll);
-                }
-                return;
-            }
-            // every root takes the whole table: at the low load this leaves
-            // (W / 1536 on the 6 KB table, about 0.2 on ER n = 1e6) a warp's
-            // slowest insert needs fewer probes, which paid more (k_c4_warp
-            // 1.58 -> 1.35 ms there) than the larger clear and sweep cost
-            const unsigned slots = (unsigned)TS;
-            if constexpr (SPLIT) {
-                const SplitTab T{sk, sc, slots, nullptr};
-                c4_root<false>(g, vacc, u, b, din, T, 0, 1, lane, 32, S.seg, S.pv, S.dups, rc, W);
-            } else {
-                const PackedTab T{S.t, slots, cb, nullptr};
-                c4_root<false>(g, vacc, u, b, din, T, 0, 1, lane, 32, S.seg, S.pv, S.dups, rc, W);
-            }
-        }();
+        f(u, ru, s0);
         u = un;
         un = u2;
         ru = ru1;
@@ -628,29 +791,138 @@ __device__ __forceinline__ void c4_warp_body(Graph g, VAcc *vacc, int *lists, in
     }
 }
 
+// One warp per root, with a count table. In small graphs k_c4_warp takes
+// every vertex as a root and queues those above its limit for the wider
+// tiers; in others k_c4_filter is the first kernel, and k_c4_warp_left
+// (QUEUE) takes the smaller roots that it could not finish. Packed tables
+// have 6 KB (8 CTAs per SM); ids that need split tables have 8 KB, since those
+// take half the wedges in the same space, and the 4-warp tier the rest (8192
+// small graphs: 442 + 2607 us with 6 KB, 717 + 2157 with 8 KB).
+template <bool SPLIT, bool QUEUE>
+__device__ __forceinline__ void c4_warp_body(const Graph &g, VAcc *vacc, int *lists, int *counters, int maxw, int cb,
+                                             int teamw) {
+    constexpr int WORDS = SPLIT ? CWB_WORDS : CW_WORDS;
+    constexpr int TS = cw_slots(SPLIT, WORDS);
+    __shared__ C4WarpSmem<WORDS> sm_all[CW_WARPS];
+    C4WarpSmem<WORDS> &S = sm_all[threadIdx.x >> 5];
+    const int lane = lane_id();
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int nw = (gridDim.x * blockDim.x) >> 5;
+    const C4Limits<SPLIT> lim(maxw, cb, teamw);
+    int *const left = lists + (size_t)CW_LEFT_LIST * g.n;
+    int *const sk = reinterpret_cast<int *>(S.t), *const sc = sk + TS;   // split keys, counts
+    if (SPLIT) SplitTab{sk, sc, (unsigned)TS, nullptr}.clear_all(lane, 32);
+    else PackedTab{S.t, (unsigned)TS, cb, nullptr}.clear_all(lane, 32);
+    __syncwarp();
+    c4_roots(
+        g, gw, nw, QUEUE ? counters[CNT_C4_LEFT] : g.n, [&](int i) { return QUEUE ? left[i] : i; },
+        [&](int u, const int4 &ru, int2 s0) {
+            const int b = ru.x, din = ru.y - ru.x;
+            if (din < 2) return;
+            int2 s1;
+            const long long W = c4_wedges(g, b, din, s0, s1);
+            const bool hub = din > WL_MAXD;
+            if (W < 2 && !hub) return;
+            if (!QUEUE && (W > lim.warp || hub)) {
+                c4_queue_root(g, lists, counters, u, din, W, false, lim);
+                return;
+            }
+            RootChunks rc;
+            if (din <= 64) {   // both chunks' segments stay in registers
+                rc.have = din > 32 ? 2 : 1;
+                rc.st0 = s0.x, rc.len0 = s0.y, rc.st1 = s1.x, rc.len1 = s1.y;
+                rc.v0 = lane < din ? g.ncol[b + lane] : -1;   // for the middle walk's credits
+                rc.v1 = 32 + lane < din ? g.ncol[b + 32 + lane] : -1;
+            }
+            // every root takes the whole table: at the low load this leaves
+            // (W / 1536 on the 6 KB table) a warp's slowest insert needs fewer
+            // probes, which paid more than the larger clear and sweep cost
+            if constexpr (SPLIT) {
+                const SplitTab T{sk, sc, (unsigned)TS, nullptr};
+                c4_root<false>(g, vacc, u, b, din, T, 0, 1, lane, 32, S.seg, S.pv, S.dups, rc, W);
+            } else {
+                const PackedTab T{S.t, (unsigned)TS, cb, nullptr};
+                c4_root<false>(g, vacc, u, b, din, T, 0, 1, lane, 32, S.seg, S.pv, S.dups, rc, W);
+            }
+        });
+}
+
 // 8 CTAs of 4 warps per SM: 6 KB tables and at most 64 registers a thread.
-__global__ void __launch_bounds__(CW_WARPS * 32, 8) k_c4_warp(Graph g, VAcc *vacc, int *lists, int *counters,
-                                                              int maxw, int cb, int teamw, const int *coff, int ntiles) {
+template <bool SPLIT>
+__global__ void __launch_bounds__(CW_WARPS * 32, SPLIT ? 6 : 8) k_c4_warp(Graph g, VAcc *vacc, int *lists, int *counters,
+                                                                          int maxw, int cb, int teamw, const int *coff,
+                                                                          int ntiles) {
     pdl_begin();
-    c4_warp_body<false, false>(g, vacc, lists, counters, maxw, cb, teamw, coff, ntiles);
+    if (degree_overflow(counters)) return;
+    c4_warp_body<SPLIT, false>(g, vacc, lists, counters, maxw, cb, ck_min_wedges(coff, ntiles, g.n, teamw));
 }
 
-__global__ void __launch_bounds__(CW_WARPS * 32, 8) k_c4_warp_split(Graph g, VAcc *vacc, int *lists,
-                                                                    int *counters, int maxw, int cb, int teamw, const int *coff, int ntiles) {
+template <bool SPLIT>
+__global__ void __launch_bounds__(CW_WARPS * 32, SPLIT ? 6 : 8) k_c4_warp_left(Graph g, VAcc *vacc, int *lists,
+                                                                               int *counters, int maxw, int cb) {
     pdl_begin();
-    c4_warp_body<true, false>(g, vacc, lists, counters, maxw, cb, teamw, coff, ntiles);
+    if (degree_overflow(counters)) return;
+    c4_warp_body<SPLIT, true>(g, vacc, lists, counters, maxw, cb, 0);
 }
 
-__global__ void __launch_bounds__(CW_WARPS * 32) k_c4_warp_big(Graph g, VAcc *vacc, int *lists, int *counters,
-                                                               int maxw, int cb, int teamw, const int *coff, int ntiles) {
-    pdl_begin();
-    c4_warp_body<false, true>(g, vacc, lists, counters, maxw, cb, teamw, coff, ntiles);
-}
+// The first kernel of large graphs: every vertex as a root, the filter only.
+// Without the table's code it takes 48 registers and 4.5 KB a warp, 40 warps
+// per SM instead of 32 (40 registers and 48 warps spill: 1.33 ms against 1.04
+// on G(1e6, mean degree 32), where the tables of three kernels took 1.79 ms;
+// G(3e6, mean degree 6) 0.37 ms against 0.76).
+// It is bound by the latency of row bounds -> segments -> rows and by issue,
+// about 60 instructions per 32 wedges.
+constexpr int CF_WARPS = 8;
+constexpr int CF_LOG = 10;
+constexpr int CF_MAXW = 2048;   // two keys per word: about 8 of them may be falsely taken for repeats
 
-__global__ void __launch_bounds__(CW_WARPS * 32) k_c4_warp_big_split(Graph g, VAcc *vacc, int *lists,
-                                                                     int *counters, int maxw, int cb, int teamw, const int *coff, int ntiles) {
+struct __align__(16) C4FilterSmem {
+    unsigned t[1 << CF_LOG];
+    long long pv[32];
+    int dups[2 * CW_DUPS];
+};
+
+template <bool SPLIT>
+__global__ void __launch_bounds__(CF_WARPS * 32, 5) k_c4_filter(Graph g, VAcc *vacc, int *lists, int *counters, int maxw,
+                                                                int tablew, int cb, int teamw, const int *coff, int ntiles) {
     pdl_begin();
-    c4_warp_body<true, true>(g, vacc, lists, counters, maxw, cb, teamw, coff, ntiles);
+    if (degree_overflow(counters)) return;
+    extern __shared__ __align__(16) unsigned char dsm[];
+    C4FilterSmem &S = reinterpret_cast<C4FilterSmem *>(dsm)[threadIdx.x >> 5];
+    const int lane = lane_id();
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int nw = (gridDim.x * blockDim.x) >> 5;
+    const C4Limits<SPLIT> lim(tablew, cb, ck_min_wedges(coff, ntiles, g.n, teamw));
+    const long long most = min(maxw < CW_MAXW ? (long long)maxw : CF_MAXW, lim.team);   // (lowered knobs hold here too)
+    for (int i = lane; i < (1 << CF_LOG) / 4; i += 32) reinterpret_cast<uint4 *>(S.t)[i] = make_uint4(EMPTY, EMPTY, EMPTY, EMPTY);
+    __syncwarp();
+    auto do_root = [&](int u, const int4 &ru, int2 s0) {
+        const int b = ru.x, din = ru.y - ru.x;
+        if (din < 2) return;
+        int2 s1;
+        const long long W = c4_wedges(g, b, din, s0, s1);
+        if (W < 2 && din <= WL_MAXD) return;
+        if (din <= 64 && W <= most && c4_few_repeats(W, g.n) && c4_bloom_root<CF_LOG>(g, vacc, u, b, din, s0, s1, S)) return;
+        c4_queue_root(g, lists, counters, u, din, W, true, lim);
+    };
+    // ids of low degree: four roots at a time, eight lanes each
+    const int2 Z2 = make_int2(0, 0);
+    const int low = maxw >= 256 ? low_degree_ids(g.n, nw, coff, ntiles) : 0;
+    for (long long u0 = 4ll * gw; u0 < low; u0 += 4ll * nw) {
+        const int u = (int)u0 + (lane >> 3), l = lane & 7;
+        int4 ru = make_int4(0, 0, 0, 0);
+        if (u < low) ru = g.rinfo[u];
+        const int din = ru.y - ru.x;
+        if (!__any_sync(FULL, din > 8)) {
+            const int2 s = l < din ? g.wl[ru.x + l] : Z2;
+            if (!__any_sync(FULL, s.y > SMALL_ROW) && c4_bloom_small(g, vacc, u, ru, s, S)) continue;
+        }
+        for (int q = 0; q < 4; ++q) {
+            const int x = __shfl_sync(FULL, ru.x, 8 * q), y = __shfl_sync(FULL, ru.y, 8 * q);
+            do_root((int)u0 + q, make_int4(x, y, 0, 0), lane < y - x && y - x <= 64 ? g.wl[x + lane] : Z2);
+        }
+    }
+    c4_roots(g, low + gw, nw, g.n, [](int i) { return i; }, do_root);
 }
 
 // Roots from a queue, one CTA each. The table (SLOTS split slots, or
@@ -1256,37 +1528,47 @@ void launch_cycle4(Work &w, cudaStream_t st) {
     else launch_pdl(k_c4_wedge_len<16>, w.num_sms * 8, 256, 0, st, g, wl, w.counters, w.coff, w.ntiles);
     after_launch(st, K_C4_WEDGE_LEN);
     int maxw = w.tune[TUNE_C4_WARP_MAXW] < CW_MAXW ? w.tune[TUNE_C4_WARP_MAXW] : CW_MAXW;
-    // A graph with fewer vertices than the warp tier has resident warps is
-    // bound by its slowest root's walk, one warp each: roots above
-    // CW_SMALL_MAXW wedges go to the 4-warp tier there (G(2000, 0.01):
-    // 104 -> 94 us per call).
-    if (w.n <= w.num_sms * 32 && maxw > CW_SMALL_MAXW) maxw = CW_SMALL_MAXW;
+    // Batches of graphs of under 150 vertices on average: their roots have many
+    // repeated keys and short walks, so all go to a warp's table at once (1756
+    // graphs of 18 to 144 vertices: 315 us a call; 359 with the filter first,
+    // 320 with the limit below; 357 graphs of 18 to 180: 138, 160, 141).
+    const bool tiny = w.graphs > 1 && w.n / w.graphs < 150 && w.n > w.num_sms * 32;
+    // The largest root that one warp walks. In other graphs of up to 3e5
+    // vertices (2048 a multiprocessor) the slowest warp's walk is a large part
+    // of the stage: above CW_SMALL_MAXW wedges, 4 warps walk it (limit 1152,
+    // 256, 32: power-law graph of 1e5 vertices 434, 420, 378 us a call, G(6000,
+    // mean degree 30) 185, 146, 147, 71 graphs of 60 to 1060 vertices 185, 171,
+    // 156). Beyond, the warp tier has work for every warp and is the cheaper
+    // one: 8192 graphs 12054, with 256 12891.
+    const int tablew = !tiny && w.n <= w.num_sms * 2048 && maxw > CW_SMALL_MAXW ? CW_SMALL_MAXW : maxw;
     const int cb = packed_count_bits(w.n);
     // a packed word holds counts up to 2^cb - 2; with many vertices (large
     // graphs, batches) that is below what the warp tier takes, and the warp
     // tier counts in split tables instead
     const bool packed = (1ll << cb) - 2 >= maxw;
     const int teamw = w.tune[TUNE_C4_TEAM_MINW];
-    static const int occ_w = resident_ctas((const void *)k_c4_warp, CW_WARPS * 32, 0);
-    static const int occ_ws = resident_ctas((const void *)k_c4_warp_split, CW_WARPS * 32, 0);
-    static const int occ_b = resident_ctas((const void *)k_c4_warp_big, CW_WARPS * 32, 0);
-    static const int occ_bs = resident_ctas((const void *)k_c4_warp_big_split, CW_WARPS * 32, 0);
-    if (packed)
-        launch_pdl(k_c4_warp, w.num_sms * min(w.tune[TUNE_GRID_C4], occ_w), CW_WARPS * 32, 0, st, g, w.vacc, w.lists,
-                   w.counters, maxw, cb, teamw, w.coff, w.ntiles);
-    else
-        launch_pdl(k_c4_warp_split, w.num_sms * min(w.tune[TUNE_GRID_C4], occ_ws), CW_WARPS * 32, 0, st, g, w.vacc, w.lists,
-                   w.counters, maxw, cb, teamw, w.coff, w.ntiles);
-    after_launch(st, K_C4_WARP);
-    // roots k_c4_warp queued for the 8 KB tables: one resident wave (none when it keeps all it may)
-    if (maxw > cw_maxw(!packed, CW_WORDS)) {
-        if (packed)
-            launch_pdl(k_c4_warp_big, w.num_sms * occ_b, CW_WARPS * 32, 0, st, g, w.vacc, w.lists, w.counters, maxw, cb, teamw,
-                       w.coff, w.ntiles);
-        else
-            launch_pdl(k_c4_warp_big_split, w.num_sms * occ_bs, CW_WARPS * 32, 0, st, g, w.vacc, w.lists, w.counters, maxw,
-                       cb, teamw, w.coff, w.ntiles);
-        after_launch(st, K_C4_WARP_BIG);
+    static const int occ_w = resident_ctas((const void *)k_c4_warp<false>, CW_WARPS * 32, 0);
+    static const int occ_ws = resident_ctas((const void *)k_c4_warp<true>, CW_WARPS * 32, 0);
+    static const int occ_l = resident_ctas((const void *)k_c4_warp_left<false>, CW_WARPS * 32, 0);
+    static const int occ_ls = resident_ctas((const void *)k_c4_warp_left<true>, CW_WARPS * 32, 0);
+    constexpr size_t CF_SMEM = CF_WARPS * sizeof(C4FilterSmem);
+    static const int occ_f = resident_ctas((const void *)k_c4_filter<false>, CF_WARPS * 32, CF_SMEM);
+    // More roots than resident warps: the filter first, then the table for
+    // what it leaves. Below, every warp has one root, and nearly all go to the
+    // 4-warp tier at once: with the filter in front, G(400, mean degree 20)
+    // took 67 us a call instead of 63, G(2000, 20) 75 instead of 71.
+    if (w.n > w.num_sms * 32 && !tiny) {
+        launch_pdl(packed ? k_c4_filter<false> : k_c4_filter<true>, w.num_sms * min(w.tune[TUNE_GRID_C4], occ_f),
+                   CF_WARPS * 32, CF_SMEM, st, g, w.vacc, w.lists, w.counters, maxw, tablew, cb, teamw, w.coff, w.ntiles);
+        after_launch(st, K_C4_WARP);
+        launch_pdl(packed ? k_c4_warp_left<false> : k_c4_warp_left<true>, w.num_sms * (packed ? occ_l : occ_ls),
+                   CW_WARPS * 32, 0, st, g, w.vacc, w.lists, w.counters, tablew, cb);
+        after_launch(st, K_C4_WARP_LEFT);
+    } else {
+        launch_pdl(packed ? k_c4_warp<false> : k_c4_warp<true>,
+                   w.num_sms * min(w.tune[TUNE_GRID_C4], packed ? occ_w : occ_ws), CW_WARPS * 32, 0, st, g, w.vacc, w.lists,
+                   w.counters, tablew, cb, teamw, w.coff, w.ntiles);
+        after_launch(st, K_C4_WARP);
     }
     static const int occ_m = resident_ctas((const void *)k_c4_mid, CM_THREADS, CM_SMEM);
     static const int occ_c = resident_ctas((const void *)k_c4_cta, CC_THREADS, CC_SMEM);
@@ -1316,10 +1598,9 @@ void launch_cycle4(Work &w, cudaStream_t st) {
 
 void configure_cycle4() {
     // the warp tiers need nearly all of an SM's shared memory for full residency
-    cudaFuncSetAttribute(k_c4_warp, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    cudaFuncSetAttribute(k_c4_warp_split, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    cudaFuncSetAttribute(k_c4_warp_big, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    cudaFuncSetAttribute(k_c4_warp_big_split, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    for (auto k : {(const void *)k_c4_warp<false>, (const void *)k_c4_warp<true>, (const void *)k_c4_warp_left<false>, (const void *)k_c4_warp_left<true>,
+                   (const void *)k_c4_filter<false>, (const void *)k_c4_filter<true>})
+        cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     cudaFuncSetAttribute(k_c4_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CM_SMEM);
     cudaFuncSetAttribute(k_c4_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CC_SMEM);
     cudaFuncSetAttribute(k_c4_tiled<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ck_smem(256, CK_SMALL_N / 2 + 64));

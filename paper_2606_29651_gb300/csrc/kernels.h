@@ -9,6 +9,7 @@ namespace niorca {
 // Per-call work memory, carved from one pool allocation.
 struct Work {
     int n = 0, m = 0;
+    int graphs = 1;          // graphs of a batch (n and m are their sums)
     int ntiles = 0;          // relabel tiles of RL_TILE vertices
     int2 *vinfo = nullptr;   // old id -> (new id, degree)
     int *perm = nullptr;     // new id -> old id
@@ -53,7 +54,7 @@ enum TuneIndex {
 // its next root from the queue's counter, so a CTA that starts late (or a
 // root that takes long) leaves no other CTA idle.
 enum { CNT_TRI_HEAVY = 0, CNT_AGG_HEAVY = 1, CNT_C4_CTA = 2, CNT_C4_TEAM = 3, CNT_DMAX = 4, CNT_C4_MID = 5,
-       CNT_C4_MIDP = 6, CNT_TRI_BIG = 7, CNT_AGG_BIG = 8, CNT_C4_WBIG = 9, CNT_C4_TILED_NEXT = 10,
+       CNT_C4_MIDP = 6, CNT_TRI_BIG = 7, CNT_AGG_BIG = 8, CNT_C4_LEFT = 9, CNT_C4_TILED_NEXT = 10,
        CNT_TRI_CTA_NEXT = 11, CNT_TRI_BIG_NEXT = 12, CNT_AGG_CTA_NEXT = 13, CNT_AGG_BIG_NEXT = 14,
        CNT_C4_MID_NEXT = 15, CNT_C4_MIDP_NEXT = 16, CNT_C4_CTA_NEXT = 17,
        CNT_BAD_ROWS = 18,   // a row is not strictly increasing, or out of range (recorded in the status too)
@@ -143,7 +144,7 @@ void launch_validate(const int *rowptr, const int *colidx, int n, int m, int *st
 enum KernelId {
     K_CLASS_HIST, K_SCAN, K_CLASS_SCATTER, K_RELABEL, K_BATCH_SETUP,
     K_TRI_WARP, K_TRI_CTA, K_AGG_WARP, K_AGG_CTA, K_C4_WARP, K_C4_CTA, K_C4_PLAN, K_C4_TILED,
-    K_SOLVE, K_VALIDATE, K_C4_MID, K_TRI_BIG, K_AGG_BIG, K_C4_WARP_BIG, K_C4_WEDGE_LEN, K_ADJ_BITS, K_COUNT
+    K_SOLVE, K_VALIDATE, K_C4_MID, K_TRI_BIG, K_AGG_BIG, K_C4_WARP_LEFT, K_C4_WEDGE_LEN, K_ADJ_BITS, K_COUNT
 };
 const char *kernel_name(int id);
 
