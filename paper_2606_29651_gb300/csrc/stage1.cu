@@ -299,8 +299,9 @@ constexpr int TB_HASH_MAXD = 8192;
 
 // Dynamic shared memory of one CTA: hash keys + values (hslots), cnt + kc
 // (nloc), per warp a segment table and a 64-entry buffer of row indices,
-// 4 work words, and R (rows x an odd number of words, to spread the banks).
-constexpr int tc_rowstride(int rows) { return ((rows + 31) / 32) | 1; }
+// 4 work words, and R (rows of an odd number of 16-byte groups, to spread the
+// banks).
+__host__ __device__ constexpr int tc_rowstride(int rows) { return ((rows + 127) / 128 | 1) * 4; }
 constexpr size_t tc_smem(int threads, int hslots, int nloc, int rows) {
     return (size_t)2 * hslots * 4 + (size_t)2 * nloc * 4 + (size_t)(threads / 32) * (sizeof(SegTab) + 128) + 16 +
            (size_t)rows * tc_rowstride(rows) * 4;
@@ -329,6 +330,8 @@ __device__ __forceinline__ void tri_cta(const Graph &g, const AdjBits &A, bool p
     extern __shared__ __align__(16) unsigned char dsm[];
     constexpr int TC_THREADS = THREADS;
     constexpr int NW = THREADS / 32;
+    __shared__ long long s_ku;   // K4s of the root, three times each
+    if (threadIdx.x == 0) s_ku = 0;
     const int lane = lane_id(), wid = threadIdx.x >> 5;
     for (int h = cta_next(next); h < count; h = cta_next(next)) {
         const int u = BACK ? list[g.n - 1 - h] : list[h];
@@ -343,15 +346,15 @@ __device__ __forceinline__ void tri_cta(const Graph &g, const AdjBits &A, bool p
         if (H > hcap) H = hcap;
         const unsigned mask = H ? H - 1 : 0;
         const int W = (dp + 31) >> 5;  // bit-matrix words per row
-        const int WP = W | 1;          // row stride of R
+        const int WP = tc_rowstride(dp);   // row stride of R
         // carve shared memory
         // beyond HASH_MAXD the per-position counters live in global memory
         const int nloc = use_hash ? dp : 0;
         int *hk = reinterpret_cast<int *>(dsm);
         int *hv = hk + H;
         int *cnt = hv + H;
-        int *kc = cnt + nloc;
-        SegTab *segs = reinterpret_cast<SegTab *>(kc + nloc);   // one per warp
+        int *kc = cnt + ((nloc + 1) & ~1);
+        SegTab *segs = reinterpret_cast<SegTab *>(kc + ((nloc + 1) & ~1));   // one per warp
         unsigned short *zb = reinterpret_cast<unsigned short *>(segs + NW) + wid * 64;  // 64 per warp
         int *work = reinterpret_cast<int *>(reinterpret_cast<unsigned short *>(segs + NW) + NW * 64);
         unsigned *R = reinterpret_cast<unsigned *>(work + 4);
@@ -466,12 +469,18 @@ __device__ __forceinline__ void tri_cta(const Graph &g, const AdjBits &A, bool p
         for (int i = threadIdx.x; i < nloc; i += TC_THREADS)
             if (cnt[i]) atomicAdd(&tcnt[s + i], cnt[i]);
         if (use_bits) {
-            // K4s of u: triangles p < q < r of R. A warp takes a row y and, one
-            // per lane, its neighbours z < y, 32 at a time (collected in zb):
-            // the common bits of rows y and z below z are triangles with y
-            // highest, those above y triangles with z lowest and y in the
-            // middle. Two thirds of the words of a pair are read, once per
-            // pair. The row's popcount is t(u, N+(u)[y]) from the triangles
+            // K4s of u: the triangles of R. A warp takes a row y and, one per
+            // lane, its neighbours z < y, 32 at a time (collected in zb), and
+            // adds the common bits of rows y and z to both. Every triangle is
+            // counted by three pairs, and added twice to each of its corners.
+            // Whole rows in 16-byte groups: the words below z and above y
+            // alone, two thirds of them, which count each triangle where it
+            // is needed, took two masked words and loops of different length
+            // in every lane (R-MAT 18: k_tri_cta 912 -> 817 us, k_tri_big 545
+            // -> 504; G(1501, 1/2): 141 -> 121, 1068 -> 1045, where rows are
+            // longest; carry-save adders to save population counts: no
+            // faster). The loop is bound by shared memory and by latency.
+            // The row's popcount is t(u, N+(u)[y]) from the triangles
             // rooted at u.
             for (;;) {
                 int y = 0;
@@ -483,13 +492,14 @@ __device__ __forceinline__ void tri_cta(const Graph &g, const AdjBits &A, bool p
                 unsigned acc = 0;
                 auto batch = [&](int cnt) {
                     if (lane >= cnt) return;
-                    const int z = zb[lane], wz = z >> 5;
+                    const int z = zb[lane];
                     const unsigned *rz = R + z * WP;
                     unsigned k = 0;
-                    for (int t = 0; t < wz; ++t) k += __popc(ry[t] & rz[t]);
-                    acc += k + __popc(ry[wz] & rz[wz] & ((1u << (z & 31)) - 1u));
-                    k = __popc(ry[wy] & rz[wy] & ~((2u << (y & 31)) - 1u));
-                    for (int t = wy + 1; t < W; ++t) k += __popc(ry[t] & rz[t]);
+#pragma unroll 1
+                    for (int t = 0; t < W; t += 4) {   // (words past W are 0)
+                        const uint4 a = *reinterpret_cast<const uint4 *>(ry + t), b = *reinterpret_cast<const uint4 *>(rz + t);
+                        k += __popc(a.x & b.x) + __popc(a.y & b.y) + __popc(a.z & b.z) + __popc(a.w & b.w);
+                    }
                     if (k) {
                         acc += k;
                         ku += k;
@@ -517,16 +527,23 @@ __device__ __forceinline__ void tri_cta(const Graph &g, const AdjBits &A, bool p
                     }
                 }
                 if (nb) batch(nb);
-                acc = __reduce_add_sync(FULL, acc);   // at most C(1151, 2)
+                acc = __reduce_add_sync(FULL, acc);   // at most 1152^2
                 if (lane == 0 && acc) atomicAdd(&kc[y], (int)acc);
                 __syncwarp();
             }
         }
         __syncthreads();
         ku = warp_sum(ku);
-        if (lane == 0 && ku) add64(&vacc[u].K4, ku);
+        if (lane == 0 && ku) add64(use_bits ? &s_ku : &vacc[u].K4, ku);
         for (int i = threadIdx.x; i < nloc; i += TC_THREADS)
-            if (kc[i]) add64(&vacc[g.ncol[s + i]].K4, kc[i]);
+            if (kc[i]) add64(&vacc[g.ncol[s + i]].K4, use_bits ? kc[i] >> 1 : kc[i]);
+        if (use_bits) {
+            __syncthreads();
+            if (threadIdx.x == 0 && s_ku) {
+                add64(&vacc[u].K4, s_ku / 3);
+                s_ku = 0;
+            }
+        }
         __syncthreads();
     }
 }
