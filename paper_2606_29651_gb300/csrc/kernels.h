@@ -33,10 +33,10 @@ struct Work {
 // Runtime tuning knobs (niorca_set_tuning): CTAs per SM of the persistent
 // warp-tier kernels, and the thresholds that route vertices to a warp or a CTA.
 enum TuneIndex {
-    TUNE_GRID_RELABEL = 0,   // k_relabel_rows_warp CTAs per SM
+    TUNE_GRID_RELABEL = 0,   // k_relabel_rows CTAs per SM
     TUNE_GRID_TRI = 1,       // k_tri_warp
     TUNE_GRID_AGG = 2,       // k_agg_warp
-    TUNE_GRID_C4 = 3,        // k_c4_warp
+    TUNE_GRID_C4 = 3,        // k_c4_filter, k_c4_warp
     TUNE_GRID_SOLVE = 4,     // k_solve
     TUNE_LONG_ROW_CLASS = 5, // degree class from which a row is relabelled by a whole CTA
     TUNE_C4_WARP_MAXW = 6,   // largest wedge count W of a 4-cycle root kept in one warp (<= 1536)

@@ -388,16 +388,16 @@ __device__ __forceinline__ void tri_cta(const Graph &g, const AdjBits &A, bool p
                 }
                 const bool diag = t == jb;
                 unsigned row = 0, col = 0;
-                adj_probe<8>(A, __ballot_sync(FULL, j >= js && j < dp - 1), roff, k, i < dp, diag,
-                             [&](int r, bool hit, int at, unsigned word) {
-                                 const unsigned bal = __ballot_sync(FULL, hit);
-                                 const int y = __shfl_sync(FULL, ry, r);
-                                 if (lane == r) row = bal;
-                                 if (hit) {
-                                     col |= 1u << r;
-                                     atomicAdd(&tcnt[y + A.rank(at, k, word)], 1);
-                                 }
-                             });
+                const unsigned rows = __ballot_sync(FULL, j >= js && j < dp - 1);
+                adj_probe<(THREADS > 256 ? 8 : 4), false>(A, rows, roff, ry, k, i < dp, diag, nullptr,
+                                                          [&](int r, bool hit, int pos, int) {
+                    const unsigned bal = __ballot_sync(FULL, hit);
+                    if (lane == r) row = bal;
+                    if (hit) {
+                        col |= 1u << r;
+                        atomicAdd(&tcnt[pos], 1);
+                    }
+                });
                 if (diag) {
                     if (i < dp) R[i * WP + t] = row | col;
                 } else {
@@ -477,8 +477,8 @@ __device__ __forceinline__ void tri_cta(const Graph &g, const AdjBits &A, bool p
             // alone, two thirds of them, which count each triangle where it
             // is needed, took two masked words and loops of different length
             // in every lane (R-MAT 18: k_tri_cta 912 -> 817 us, k_tri_big 545
-            // -> 504; G(1501, 1/2): 141 -> 121, 1068 -> 1045, where rows are
-            // longest; carry-save adders to save population counts: no
+            // -> 504, both then less by the probes' loads ahead; G(1501, 1/2):
+            // 141 -> 121, 1068 -> 1045, where rows are longest; carry-save adders to save population counts: no
             // faster). The loop is bound by shared memory and by latency.
             // The row's popcount is t(u, N+(u)[y]) from the triangles
             // rooted at u.

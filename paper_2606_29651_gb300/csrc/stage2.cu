@@ -279,16 +279,16 @@ __device__ __forceinline__ void agg_cta(const Graph &g, const AdjBits &A, bool p
                     ry = g.rinfo[v].y;
                 }
                 unsigned rsum = 0, csum = 0;   // 32 counts of at most 2^20 each
-                adj_probe<8>(A, __ballot_sync(FULL, tr > 0), roff, k, tc > 0, t == jb,
-                             [&](int r, bool hit, int at, unsigned word) {
-                                 const int y = __shfl_sync(FULL, ry, r), tw = __shfl_sync(FULL, tr, r);
-                                 const unsigned sum = __reduce_add_sync(FULL, (unsigned)(hit ? tc - 1 : 0));
-                                 if (lane == r) rsum = sum;
-                                 if (hit) {
-                                     csum += tw - 1;                                // t(u, v) - 1 -> w
-                                     du12 += tcnt[y + A.rank(at, k, word)] - 1;     // t(v, w) - 1 -> u
-                                 }
-                             });
+                adj_probe<4, true>(A, __ballot_sync(FULL, tr > 0), roff, ry, k, tc > 0, t == jb, tcnt,
+                                   [&](int r, bool hit, int, int tvw) {
+                                       const int tw = __shfl_sync(FULL, tr, r);
+                                       const unsigned sum = __reduce_add_sync(FULL, (unsigned)(hit ? tc - 1 : 0));
+                                       if (lane == r) rsum = sum;
+                                       if (hit) {
+                                           csum += tw - 1;      // t(u, v) - 1 -> w
+                                           du12 += tvw - 1;     // t(v, w) - 1 -> u
+                                       }
+                                   });
                 if (rsum) add64(&dc[j], rsum);   // t(u, w) - 1 -> v
                 if (csum) add64(&dc[i], csum);
             }
