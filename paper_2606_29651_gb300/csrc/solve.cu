@@ -76,7 +76,7 @@ __device__ __forceinline__ void to_induced(long long *p) {
     p[10] = i10; p[11] = i11; p[12] = i12; p[13] = i13; p[14] = i14;
 }
 
-// Rows from the long-row class on (new ids from `bound`, the degree-class
+// Rows from a degree class on (new ids from `bound`, the degree-class
 // order puts them last): one warp per vertex. Every other vertex is solved in
 // groups of 32 consecutive caller ids: each lane loads its vertex's row bounds
 // and accumulators up front, the warp sums S1 and A1 over the neighbours of
@@ -97,7 +97,13 @@ __device__ __forceinline__ void solve_write(long long d, const VAcc &a, long lon
 }
 
 constexpr int SOLVE_WARPS = 8;
-constexpr int SOLVE_GROUP_MAXD = 128;   // degree up to which eight lanes sum a vertex's neighbours
+// Degree class (of degree 64) from which a vertex has a warp to itself.
+// Vertices of high degree are often neighbours in the caller's order too, and
+// a warp that sums 32 of them in turn is the kernel's tail: with the line at
+// degrees 512, 128, 64 it took 84, 37, 25 us on a power-law graph of 1e5
+// vertices, 41, 27, 20 on R-MAT 14 and 1321, 1233, 1137 on R-MAT 22 (R-MAT
+// 18, with one vertex of 25254 neighbours: 83, 110, 95).
+constexpr int SOLVE_WARP_CLASS = 20;
 
 __global__ void __launch_bounds__(SOLVE_WARPS * 32) k_solve(Graph g, const VAcc *vacc, const int *perm,
                                                             const int2 *vinfo, long long *out, int induced,
@@ -111,7 +117,9 @@ __global__ void __launch_bounds__(SOLVE_WARPS * 32) k_solve(Graph g, const VAcc 
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     const int bound = min(coff[long_class * ntiles], g.n);
-    for (int x = bound + gw; x < g.n; x += nw) {
+    // highest degrees first, on different CTAs
+    const int spread = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    for (int x = g.n - 1 - spread; x >= bound; x -= nw) {
         const int4 rx = g.rinfo[x];
         long long sS1 = 0, sA1 = 0;
         for (int p = rx.x + lane; p < rx.z; p += 32) {
@@ -145,36 +153,21 @@ __global__ void __launch_bounds__(SOLVE_WARPS * 32) k_solve(Graph g, const VAcc 
             const int b = __shfl_sync(FULL, rx.x, src), e = __shfl_sync(FULL, rx.z, src);
             const int top = (int)__reduce_max_sync(FULL, (unsigned)(e - b));
             long long s1 = 0, a1 = 0;
-            if (top <= SOLVE_GROUP_MAXD) {
-                for (int p = b + sub; p - b - sub < top; p += 16) {
-                    longlong2 u = make_longlong2(0, 0), v = u;
-                    if (p < e) u = *reinterpret_cast<const longlong2 *>(&vacc[g.ncol[p]]);
-                    if (p + 8 < e) v = *reinterpret_cast<const longlong2 *>(&vacc[g.ncol[p + 8]]);
-                    s1 += u.x + v.x;
-                    a1 += u.y + v.y;
-                }
-#pragma unroll
-                for (int o = 1; o < 8; o <<= 1) {
-                    s1 += __shfl_xor_sync(FULL, s1, o);
-                    a1 += __shfl_xor_sync(FULL, a1, o);
-                }
-                // lane 8 q holds the sums of vertex k + q
-                const long long s = __shfl_sync(FULL, s1, (lane & 3) * 8), t = __shfl_sync(FULL, a1, (lane & 3) * 8);
-                if ((lane & ~3) == k) { mS1 = s; mA1 = t; }
-            } else {   // a long row among them: the whole warp, one vertex after the other
-                for (int q = 0; q < 4; ++q) {
-                    const int bq = __shfl_sync(FULL, b, 8 * q), eq = __shfl_sync(FULL, e, 8 * q);
-                    s1 = a1 = 0;
-                    for (int p = bq + lane; p < eq; p += 32) {
-                        const longlong2 u = *reinterpret_cast<const longlong2 *>(&vacc[g.ncol[p]]);
-                        s1 += u.x;
-                        a1 += u.y;
-                    }
-                    s1 = warp_sum(s1);
-                    a1 = warp_sum(a1);
-                    if (lane == k + q) { mS1 = s1; mA1 = a1; }
-                }
+            for (int p = b + sub; p - b - sub < top; p += 16) {
+                longlong2 u = make_longlong2(0, 0), v = u;
+                if (p < e) u = *reinterpret_cast<const longlong2 *>(&vacc[g.ncol[p]]);
+                if (p + 8 < e) v = *reinterpret_cast<const longlong2 *>(&vacc[g.ncol[p + 8]]);
+                s1 += u.x + v.x;
+                a1 += u.y + v.y;
             }
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {
+                s1 += __shfl_xor_sync(FULL, s1, o);
+                a1 += __shfl_xor_sync(FULL, a1, o);
+            }
+            // lane 8 q holds the sums of vertex k + q
+            const long long s = __shfl_sync(FULL, s1, (lane & 3) * 8), t = __shfl_sync(FULL, a1, (lane & 3) * 8);
+            if ((lane & ~3) == k) { mS1 = s; mA1 = t; }
         }
         if (have) solve_write(rx.z - rx.x, a, mS1, mA1, induced, ob + lane * 15);
         __syncwarp();
@@ -190,7 +183,7 @@ void launch_solve(Work &w, long long *out, cudaStream_t st) {
     const int grid = w.num_sms * w.tune[TUNE_GRID_SOLVE];
     // a graph with no more vertices than the grid has warps: one warp per
     // vertex (long_class 0), so that no warp solves 32 vertices in turn
-    const int lc = (long long)w.n <= (long long)grid * SOLVE_WARPS ? 0 : w.tune[TUNE_LONG_ROW_CLASS];
+    const int lc = (long long)w.n <= (long long)grid * SOLVE_WARPS ? 0 : min(w.tune[TUNE_LONG_ROW_CLASS], SOLVE_WARP_CLASS);
     launch_pdl(k_solve, grid, SOLVE_WARPS * 32, 0, st,
         g, w.vacc, w.perm, w.vinfo, out, w.induced, w.coff, w.ntiles, lc, w.counters);
     after_launch(st, K_SOLVE);
