@@ -36,7 +36,9 @@
  *     recorded in the status word of the call's stream, read by
  *     niorca_last_status(stream); after such an error `out` is unspecified.
  *     Malformed input never makes a kernel access memory outside the given
- *     arrays: a degree above 2^20 stops every stage after the degree pass.
+ *     arrays or the work memory: offsets that fall, leave [0, m] or do not
+ *     span it stop the call after the degree pass (the rows are not looked
+ *     at then), a degree above 2^20 after the rows' own checks.
  *   - Work memory is taken from a library-owned, stream-ordered pool on the
  *     current device and returned to it when the stream reaches the end of
  *     the call; the pool keeps freed memory for reuse.

@@ -93,7 +93,7 @@ constexpr int WL_LONG = 128;
 template <int L>
 __global__ void __launch_bounds__(256, 8) k_c4_wedge_len(Graph g, int2 *wl, const int *counters, const int *coff, int ntiles) {
     pdl_begin();
-    if (degree_overflow(counters)) return;
+    if (call_stopped(counters)) return;
     auto row = [&](int u, int first, int stride) {
         const int4 ru = g.rinfo[u];
         if (ru.y - ru.x > WL_MAXD) return;
@@ -853,7 +853,7 @@ __global__ void __launch_bounds__(CW_WARPS * 32, SPLIT ? 6 : 8) k_c4_warp(Graph 
                                                                           int maxw, int cb, int teamw, const int *coff,
                                                                           int ntiles) {
     pdl_begin();
-    if (degree_overflow(counters)) return;
+    if (call_stopped(counters)) return;
     c4_warp_body<SPLIT, false>(g, vacc, lists, counters, maxw, cb, ck_min_wedges(coff, ntiles, g.n, teamw));
 }
 
@@ -861,7 +861,7 @@ template <bool SPLIT>
 __global__ void __launch_bounds__(CW_WARPS * 32, SPLIT ? 6 : 8) k_c4_warp_left(Graph g, VAcc *vacc, int *lists,
                                                                                int *counters, int maxw, int cb) {
     pdl_begin();
-    if (degree_overflow(counters)) return;
+    if (call_stopped(counters)) return;
     c4_warp_body<SPLIT, true>(g, vacc, lists, counters, maxw, cb, 0);
 }
 
@@ -886,7 +886,7 @@ template <bool SPLIT>
 __global__ void __launch_bounds__(CF_WARPS * 32, 5) k_c4_filter(Graph g, VAcc *vacc, int *lists, int *counters, int maxw,
                                                                 int tablew, int cb, int teamw, const int *coff, int ntiles) {
     pdl_begin();
-    if (degree_overflow(counters)) return;
+    if (call_stopped(counters)) return;
     extern __shared__ __align__(16) unsigned char dsm[];
     C4FilterSmem &S = reinterpret_cast<C4FilterSmem *>(dsm)[threadIdx.x >> 5];
     const int lane = lane_id();
@@ -973,7 +973,7 @@ constexpr size_t CC_SMEM = cq_smem(CC_THREADS, CC_SLOTS, CC_MAXW);
 __global__ void __launch_bounds__(CM_THREADS) k_c4_mid(Graph g, VAcc *vacc, const int *lists, int *counters,
                                                        int cb) {
     pdl_begin();
-    if (degree_overflow(counters)) return;
+    if (call_stopped(counters)) return;
     c4_queue<CM_THREADS, CM_SLOTS, CM_MAXW, true>(g, vacc, lists + 5 * (size_t)g.n, counters[CNT_C4_MIDP],
                                                   counters + CNT_C4_MIDP_NEXT, cb);
     c4_queue<CM_THREADS, CM_SLOTS, CM_MAXW, false>(g, vacc, lists + 2 * (size_t)g.n, counters[CNT_C4_MID],
@@ -983,7 +983,7 @@ __global__ void __launch_bounds__(CM_THREADS) k_c4_mid(Graph g, VAcc *vacc, cons
 __global__ void __launch_bounds__(CC_THREADS) k_c4_cta(Graph g, VAcc *vacc, const int *lists, int *counters,
                                                        int cb) {
     pdl_begin();
-    if (degree_overflow(counters)) return;
+    if (call_stopped(counters)) return;
     c4_queue<CC_THREADS, CC_SLOTS, CC_MAXW, false>(g, vacc, lists + 3 * (size_t)g.n, counters[CNT_C4_CTA],
                                                    counters + CNT_C4_CTA_NEXT, cb);
 }
@@ -1081,7 +1081,7 @@ __global__ void __launch_bounds__(1024) k_c4_tiled_plan(Graph g, int *lists, int
     __shared__ int wsum[32];
     __shared__ CkZone z[CK_ZONES + 1];
     __shared__ int glo[CK_MAX_GROUPS];
-    if (degree_overflow(counters)) return;
+    if (call_stopped(counters)) return;
     const int nt = counters[CNT_C4_TEAM];
     if (nt == 0) return;
     const int *roots = lists + 4 * (size_t)g.n, *wts = lists + (size_t)g.n;
@@ -1482,7 +1482,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1)
     S.any = S.wrun + THREADS / 32;
     S.job = S.any + 1;
     S.twice = reinterpret_cast<long long *>(S.any + 2);
-    if (degree_overflow(counters)) return;
+    if (call_stopped(counters)) return;
     const int nt = counters[CNT_C4_TEAM];
     if (nt == 0) return;
     const int *sorted = lists, *offs = lists + 2 * (size_t)g.n;

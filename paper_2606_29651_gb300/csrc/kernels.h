@@ -60,6 +60,7 @@ enum { CNT_TRI_HEAVY = 0, CNT_AGG_HEAVY = 1, CNT_C4_CTA = 2, CNT_C4_TEAM = 3, CN
        CNT_BAD_ROWS = 18,   // a row is not strictly increasing, or out of range (recorded in the status too)
        CNT_ADJ_ON = 19,     // the triangle and aggregate stages probe the adjacency bitmap (AdjBits)
        CNT_SCAN_DONE = 20,  // blocks of a scan's first pass that are done (0 between scans)
+       CNT_BAD_OFFSETS = 21,   // the CSR offsets fall, leave [0, m] or do not span it (recorded in the status too)
        NCOUNTERS = 32 };
 
 // The next item of a work queue, for the whole CTA: thread 0 takes it from
@@ -102,13 +103,19 @@ void launch_pdl(void (*kernel)(P...), unsigned grid, unsigned threads, size_t sm
 // persistent grid is SMs times this.
 int resident_ctas(const void *kernel, int threads, size_t smem);
 
-// Whether the degree pass found a degree above MAX_DEGREE. NIORCA_EOVERFLOW
-// is then recorded already, and every kernel after the relabelling returns
-// at once: their fixed-size shared buffers and 32-bit partial sums rely on
-// the bound (Sec. 3 bounds the work by the largest degree; the bound itself
-// is this library's choice, see MAX_DEGREE).
-__device__ __forceinline__ bool degree_overflow(const int *counters) {
-    return *reinterpret_cast<const volatile int *>(counters + CNT_DMAX) > MAX_DEGREE;
+// Whether the degree pass stopped the call; its error is recorded already, and
+// every kernel after the relabelling returns at once. A degree above MAX_DEGREE
+// (NIORCA_EOVERFLOW): the fixed-size shared buffers and 32-bit partial sums of
+// those kernels rely on the bound (Sec. 3 bounds the work by the largest
+// degree; the bound itself is this library's choice, see MAX_DEGREE). CSR
+// offsets that fall or leave [0, m] (NIORCA_EINVAL): the rows that remain may
+// overlap, so that their degrees sum to more than m and a copy of them has no
+// place in the work memory; the row relabelling returns too.
+__device__ __forceinline__ bool offsets_bad(const int *counters) {
+    return *reinterpret_cast<const volatile int *>(counters + CNT_BAD_OFFSETS) != 0;
+}
+__device__ __forceinline__ bool call_stopped(const int *counters) {
+    return *reinterpret_cast<const volatile int *>(counters + CNT_DMAX) > MAX_DEGREE || offsets_bad(counters);
 }
 
 constexpr int RL_TILE = 2048;        // vertices per class-histogram tile

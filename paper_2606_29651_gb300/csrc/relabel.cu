@@ -166,7 +166,10 @@ __global__ void __launch_bounds__(RL_THREADS) k_class_hist(const int *rowptr, in
         atomicAdd(&h[deg_class(d)], 1);
         lmax = max(lmax, d);
     }
-    if (bad) set_status(status, ST_EINVAL);
+    if (bad) {
+        set_status(status, ST_EINVAL);
+        atomicOr(&counters[CNT_BAD_OFFSETS], 1);
+    }
     lmax = warp_max(lmax);
     if (lane_id() == 0) atomicMax(&smax, lmax);
     __syncthreads();
@@ -249,7 +252,10 @@ __global__ void __launch_bounds__(RS_THREADS) k_class_small(const int *rowptr, i
         atomicAdd(&h[deg_class(d)], 1);
         lmax = max(lmax, d);
     }
-    if (bad) set_status(status, ST_EINVAL);
+    if (bad) {
+        set_status(status, ST_EINVAL);
+        atomicOr(&counters[CNT_BAD_OFFSETS], 1);
+    }
     lmax = warp_max(lmax);
     if (lane == 0) atomicMax(&smax, lmax);
     __syncthreads();
@@ -629,6 +635,7 @@ __global__ void __launch_bounds__(RLR_THREADS, 6) k_relabel_rows(RelabelArgs A) 
         int H[RLR_THREADS / 32][NCLASS];
         LongRowSmem S;
     } sm;
+    if (offsets_bad(A.counters)) return;
     int bad = 0;
     for (int r = A.coff[A.long_class * A.ntiles] + blockIdx.x; r < A.n; r += gridDim.x) bad |= relabel_long(A, r, sm.S);
     const int lane = lane_id();
@@ -640,7 +647,7 @@ __global__ void __launch_bounds__(RLR_THREADS, 6) k_relabel_rows(RelabelArgs A) 
         else bad |= relabel_row(A, x, r, d, ob, sm.H[threadIdx.x >> 5]);
     };
     for (int x = FOUR ? A.n : gw; x < A.n; x += nw) {
-        const int2 vx = A.vinfo[x];   // new id, degree (0 for a row with bad offsets)
+        const int2 vx = A.vinfo[x];   // new id, degree
         if (deg_class(vx.y) < A.long_class) row(x, vx.x, vx.y, vx.y > 0 ? A.rowptr[x] : 0);
     }
     for (long long x0 = FOUR ? 4ll * gw : A.n; x0 < A.n; x0 += 4ll * nw) {

@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(SOLVE_WARPS * 32) k_solve(Graph g, const VAcc 
                                                             const int *counters) {
     pdl_begin();
     __shared__ long long obuf[SOLVE_WARPS][32 * 15];
-    if (degree_overflow(counters)) return;
+    if (call_stopped(counters)) return;
     const int lane = lane_id();
     long long *ob = obuf[threadIdx.x >> 5];
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;

@@ -80,7 +80,7 @@ __device__ __forceinline__ void warp_k4(const Graph &g, VAcc *vacc, int u, int s
 __global__ void __launch_bounds__(256) k_adj_bits(Graph g, AdjBits A, const int *nrow, unsigned *words,
                                                   unsigned short *prefix, int *counters) {
     pdl_begin();
-    if (degree_overflow(counters)) return;
+    if (call_stopped(counters)) return;
     const int total = nrow[g.n];
     const long long own = total - nrow[A.base], rows = g.n - A.base;
     const bool on = rows > 0 && !counters[CNT_BAD_ROWS] && 2 * own >= total &&
@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(TW_WARPS * 32, 6) k_tri_warp(Graph g, AdjBits 
     const int lane = lane_id();
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
-    if (degree_overflow(counters)) return;
+    if (call_stopped(counters)) return;
     const bool probe = counters[CNT_ADJ_ON];
     auto root = [&](int u, int s, int dp) {
         if (dp < 2) return;
@@ -551,7 +551,7 @@ __device__ __forceinline__ void tri_cta(const Graph &g, const AdjBits &A, bool p
 __global__ void __launch_bounds__(TS_THREADS) k_tri_cta(Graph g, AdjBits A, int *tcnt, VAcc *vacc, const int *heavy,
                                                         int *counters, int bits_maxd, int hash_maxd) {
     pdl_begin();
-    if (degree_overflow(counters)) return;
+    if (call_stopped(counters)) return;
     tri_cta<TS_THREADS, TS_MAXD, 4 * TS_MAXD, TS_MAXD, false, 4>(g, A, counters[CNT_ADJ_ON], tcnt, vacc, heavy,
                                                             counters[CNT_TRI_HEAVY], counters + CNT_TRI_CTA_NEXT,
                                                             bits_maxd, hash_maxd);
@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(TS_THREADS) k_tri_cta(Graph g, AdjBits A, int 
 __global__ void __launch_bounds__(TB_THREADS) k_tri_big(Graph g, AdjBits A, int *tcnt, VAcc *vacc, const int *heavy,
                                                         int *counters, int bits_maxd, int hash_maxd) {
     pdl_begin();
-    if (degree_overflow(counters)) return;
+    if (call_stopped(counters)) return;
     tri_cta<TB_THREADS, TB_BITMAT_MAXD, TB_BITMAT_HSLOTS, TB_HASH_MAXD, true, 4>(g, A, counters[CNT_ADJ_ON], tcnt, vacc, heavy,
                                                                             counters[CNT_TRI_BIG],
                                                                             counters + CNT_TRI_BIG_NEXT, bits_maxd,

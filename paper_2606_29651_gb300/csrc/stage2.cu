@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(AW_WARPS * 32, 6) k_agg_warp(Graph g, AdjBits 
     const int lane = lane_id();
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
-    if (degree_overflow(counters)) return;
+    if (call_stopped(counters)) return;
     const bool probe = counters[CNT_ADJ_ON];
     auto triangles = [&](int u, int s, int dp) {
         if (probe) agg_root_probe(g, A, tcnt, vacc, u, s, dp);
@@ -336,7 +336,7 @@ __device__ __forceinline__ void agg_cta(const Graph &g, const AdjBits &A, bool p
 __global__ void __launch_bounds__(AS_THREADS) k_agg_cta(Graph g, AdjBits A, const int *tcnt, VAcc *vacc, const int *heavy,
                                                         int *counters, int hash_maxd) {
     pdl_begin();
-    if (degree_overflow(counters)) return;
+    if (call_stopped(counters)) return;
     agg_cta<AS_THREADS, AS_MAXD, 4 * AS_MAXD, false>(g, A, counters[CNT_ADJ_ON], tcnt, vacc, heavy,
                                                      counters[CNT_AGG_HEAVY], counters + CNT_AGG_CTA_NEXT, hash_maxd);
 }
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(AS_THREADS) k_agg_cta(Graph g, AdjBits A, cons
 __global__ void __launch_bounds__(AB_THREADS) k_agg_big(Graph g, AdjBits A, const int *tcnt, VAcc *vacc, const int *heavy,
                                                         int *counters, int hash_maxd) {
     pdl_begin();
-    if (degree_overflow(counters)) return;
+    if (call_stopped(counters)) return;
     agg_cta<AB_THREADS, AB_HASH_MAXD, 2 * AB_HASH_MAXD, true>(g, A, counters[CNT_ADJ_ON], tcnt, vacc, heavy,
                                                               counters[CNT_AGG_BIG], counters + CNT_AGG_BIG_NEXT,
                                                               hash_maxd);

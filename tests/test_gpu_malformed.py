@@ -1,0 +1,47 @@
+"""Malformed CSR input through the device entry points: the error is reported,
+nothing is touched out of range, and the next call on the stream is right."""
+import numpy as np
+import pytest
+
+import graphgen as gg
+import oracle
+from test_gpu_parity import assert_same, gpu_count, ni  # noqa: F401 (fixture)
+from test_zz_no_alloc import _run, lib  # noqa: F401 (fixture)
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def _rows_that_overlap(n, m):
+    """Offsets 0, m, 0, m, ...: every other row is in range and holds all m
+    entries, so that the degrees sum to about n m / 2."""
+    rp = np.zeros(n + 1, np.int32)
+    rp[1::2] = m
+    rp[n] = m
+    return rp, (np.arange(m) % n).astype(np.int32)
+
+
+@pytest.mark.parametrize("n,m", [(3, 2), (1501, 6000), (2048, 40000),   # one tile of vertices
+                                 (2049, 9000), (30000, 120000),        # several
+                                 (6000, 1 << 20)])                      # the sum passes 2^31
+def test_overlapping_rows_stop_the_call(ni, lib, n, m):  # noqa: F811
+    from paper_2606_29651_gb300 import Status
+    rp, ci = _rows_that_overlap(n, m)
+    dev = torch.device("cuda:0")
+    a, b = torch.from_numpy(rp).to(dev), torch.from_numpy(ci).to(dev)
+    ni.last_status()
+    for call in (ni.count, ni.count_induced):
+        call(a, b)
+        assert ni.last_status() == Status.EINVAL
+    ni.count_batch(a, b, torch.tensor([0, n], device=dev), torch.tensor([0, m], device=dev))
+    assert ni.last_status() == Status.EINVAL
+    ha, hb = a.cpu().pin_memory(), b.cpu().pin_memory()
+    hout = ni.count_host(ha, hb)
+    assert hout.shape == (n, 15)
+    assert ni.last_status() == Status.EINVAL
+    # the rows are not looked at: their loops and repeats are not reported
+    status = torch.full((1,), 7, dtype=torch.int32, device=dev)
+    _run(lib, "noalloc", rp, ci, status)
+    assert int(status.item()) == 1 << Status.EINVAL
+    good = gg.rmat(10, 8, seed=2)
+    assert_same(gpu_count(ni, *good), oracle.count(*good), "the next call")
