@@ -110,12 +110,15 @@ int resident_ctas(const void *kernel, int threads, size_t smem);
 // degree; the bound itself is this library's choice, see MAX_DEGREE). CSR
 // offsets that fall or leave [0, m] (NIORCA_EINVAL): the rows that remain may
 // overlap, so that their degrees sum to more than m and a copy of them has no
-// place in the work memory; the row relabelling returns too.
-__device__ __forceinline__ bool offsets_bad(const int *counters) {
-    return *reinterpret_cast<const volatile int *>(counters + CNT_BAD_OFFSETS) != 0;
+// place in the work memory; the row relabelling returns too. Bad offsets raise
+// CNT_DMAX as well, so that a kernel waits for one load here (a second flag
+// after it: about 1 us a kernel).
+__device__ __forceinline__ void stop_bad_offsets(int *counters) {
+    atomicOr(&counters[CNT_BAD_OFFSETS], 1);
+    atomicMax(&counters[CNT_DMAX], 0x7fffffff);
 }
 __device__ __forceinline__ bool call_stopped(const int *counters) {
-    return *reinterpret_cast<const volatile int *>(counters + CNT_DMAX) > MAX_DEGREE || offsets_bad(counters);
+    return *reinterpret_cast<const volatile int *>(counters + CNT_DMAX) > MAX_DEGREE;
 }
 
 constexpr int RL_TILE = 2048;        // vertices per class-histogram tile

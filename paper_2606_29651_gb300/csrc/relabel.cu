@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(RL_THREADS) k_class_hist(const int *rowptr, in
     }
     if (bad) {
         set_status(status, ST_EINVAL);
-        atomicOr(&counters[CNT_BAD_OFFSETS], 1);
+        stop_bad_offsets(counters);
     }
     lmax = warp_max(lmax);
     if (lane_id() == 0) atomicMax(&smax, lmax);
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(RS_THREADS) k_class_small(const int *rowptr, i
     }
     if (bad) {
         set_status(status, ST_EINVAL);
-        atomicOr(&counters[CNT_BAD_OFFSETS], 1);
+        stop_bad_offsets(counters);
     }
     lmax = warp_max(lmax);
     if (lane == 0) atomicMax(&smax, lmax);
@@ -635,7 +635,7 @@ __global__ void __launch_bounds__(RLR_THREADS, 6) k_relabel_rows(RelabelArgs A) 
         int H[RLR_THREADS / 32][NCLASS];
         LongRowSmem S;
     } sm;
-    if (offsets_bad(A.counters)) return;
+    if (A.counters[CNT_BAD_OFFSETS]) return;
     int bad = 0;
     for (int r = A.coff[A.long_class * A.ntiles] + blockIdx.x; r < A.n; r += gridDim.x) bad |= relabel_long(A, r, sm.S);
     const int lane = lane_id();
