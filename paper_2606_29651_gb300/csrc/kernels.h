@@ -60,7 +60,11 @@ enum { CNT_TRI_HEAVY = 0, CNT_AGG_HEAVY = 1, CNT_C4_CTA = 2, CNT_C4_TEAM = 3, CN
        CNT_BAD_ROWS = 18,   // a row is not strictly increasing, or out of range (recorded in the status too)
        CNT_ADJ_ON = 19,     // the triangle and aggregate stages probe the adjacency bitmap (AdjBits)
        CNT_SCAN_DONE = 20,  // blocks of a scan's first pass that are done (0 between scans)
-       CNT_BAD_OFFSETS = 21,   // the CSR offsets fall, leave [0, m] or do not span it (recorded in the status too)
+       CNT_C4_MIDP_LEFT = 21,   // roots that k_c4_warp_left appends to k_c4_mid's packed queue
+       CNT_C4_MODE = 22,    // of the first 4-cycle kernels, set by k_c4_wedge_len (0: the call is stopped)
+       CNT_SAMPLE_DONE = 23,   // warps of k_c4_wedge_len that are done with the sample below
+       CNT_CLUSTER = 24,    // two 64-bit sums over a sample of the vertices: 2 x triangles, ordered pairs of neighbours
+       CNT_BAD_OFFSETS = 28,   // the CSR offsets fall, leave [0, m] or do not span it (recorded in the status too)
        NCOUNTERS = 32 };
 
 // The next item of a work queue, for the whole CTA: thread 0 takes it from
