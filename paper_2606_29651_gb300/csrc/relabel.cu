@@ -470,9 +470,10 @@ __device__ __forceinline__ int relabel_two(const RelabelArgs &A, int x, int r, i
 
 // A row of more than 64 entries, one warp: pass 1 validates it, counts its
 // classes (H) and sums neighbour degrees; pass 2 writes every new id at its
-// class offset (stable within a class). The first 64 entries stay in registers
-// between the passes: read again, they cross the host link twice when the CSR
-// is in host memory (G(4e5, mean degree 80): 1528 us, 997 so).
+// class offset (stable within a class). With KEEP the first 64 entries stay in
+// registers between the passes: read again, they cross the host link twice when
+// the CSR is in host memory (G(4e5, mean degree 80): 1528 us, 997 so).
+template <bool KEEP>
 __device__ __forceinline__ int relabel_row(const RelabelArgs &A, int x, int r, int d, int ob, int *H) {
     const int lane = lane_id();
     const int nb = A.nrow[r];
@@ -500,8 +501,8 @@ __device__ __forceinline__ int relabel_row(const RelabelArgs &A, int x, int r, i
             s1 += vi.y;
             p6 += c2m1(vi.y);
             below += vi.x < r;
-            if (k == 0) { nid0 = vi.x; c0 = c; }
-            else if (k == 32) { nid1 = vi.x; c1 = c; }
+            if (KEEP && k == 0) { nid0 = vi.x; c0 = c; }
+            else if (KEEP && k == 32) { nid1 = vi.x; c1 = c; }
         }
     }
     // exclusive scan of the 128 class counts: 4 per lane
@@ -520,7 +521,7 @@ __device__ __forceinline__ int relabel_row(const RelabelArgs &A, int x, int r, i
         const int i = k + lane;
         const bool act = i < d;
         int nid = k == 0 ? nid0 : nid1, c = k == 0 ? c0 : c1;   // (the row has more than 64 entries)
-        if (k >= 64) {
+        if (!KEEP || k >= 64) {
             int ys = act ? global_id(A.colidx[ob + i], vr, A.n) : 0;
             if (ys < 0) ys = x;
             const int2 vi = act ? A.vinfo[ys] : make_int2(0, 0);
@@ -660,7 +661,8 @@ __device__ __forceinline__ int relabel_long(const RelabelArgs &A, int r, LongRow
 // warp takes one row at a time, or, with FOUR, four: rows of at most 8
 // entries at once (eight lanes each), of at most 16 in pairs, longer ones in
 // turn. A row is a chain of four dependent loads, so FOUR pays where rows are
-// short (G(3e6, mean degree 6): 861 -> 425 us) and where every warp has many
+// short (G(3e6, mean degree 6): 861 -> 410 us; 433 with KEEP, which needs
+// registers that its code for short rows misses) and where every warp has many
 // rows (a power-law graph of 1e5 vertices: 44 us alone, 74 us by fours).
 template <bool FOUR>
 __global__ void __launch_bounds__(RLR_THREADS, 6) k_relabel_rows(RelabelArgs A) {
@@ -669,16 +671,17 @@ __global__ void __launch_bounds__(RLR_THREADS, 6) k_relabel_rows(RelabelArgs A) 
         int H[RLR_THREADS / 32][NCLASS];
         LongRowSmem S;
     } sm;
-    if (A.counters[CNT_BAD_OFFSETS]) return;
+    const int stop = A.counters[CNT_BAD_OFFSETS], bound = A.coff[A.long_class * A.ntiles];   // (loaded together)
+    if (stop) return;
     int bad = 0;
-    for (int r = A.coff[A.long_class * A.ntiles] + blockIdx.x; r < A.n; r += gridDim.x) bad |= relabel_long(A, r, sm.S);
+    for (int r = bound + blockIdx.x; r < A.n; r += gridDim.x) bad |= relabel_long(A, r, sm.S);
     const int lane = lane_id();
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     auto row = [&](int x, int r, int d, int ob) {
         if (d <= 32) bad |= relabel_group<32>(A, x, r, d, ob, true);
         else if (d <= 64) bad |= relabel_two(A, x, r, d, ob);
-        else bad |= relabel_row(A, x, r, d, ob, sm.H[threadIdx.x >> 5]);
+        else bad |= relabel_row<!FOUR>(A, x, r, d, ob, sm.H[threadIdx.x >> 5]);
     };
     for (int x = FOUR ? A.n : gw; x < A.n; x += nw) {
         const int2 vx = A.vinfo[x];   // new id, degree
