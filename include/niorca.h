@@ -84,7 +84,8 @@ niorca_status niorca_count(const int32_t *rowptr, const int32_t *colidx, int32_t
  * no staging copy: the kernels that read the CSR (the degree-class pass and
  * the row relabelling, each reading it once in order) load it across the
  * host link, and the orbit solve stores the counts into `out` in blocks of
- * 32 contiguous rows. On GB300 (Grace host, NVLink-C2C) the transfers thus
+ * 32 contiguous rows (a row at a time for vertices whose degree is far above
+ * the mean, and in graphs of few vertices). On GB300 (Grace host, NVLink-C2C) the transfers thus
  * overlap the kernels instead of preceding and following them.
  *   rowptr  host int32[n + 1], colidx host int32[m], out host int64[n * 15],
  *           same meaning and layout as niorca_count; each must be

@@ -87,6 +87,9 @@ __device__ __forceinline__ void to_induced(long long *p) {
 // (3840 contiguous bytes) with coalesced stores through shared memory, which
 // also suits an output buffer in host memory. With long_class 0 (a graph
 // with fewer vertices than the grid has warps) every vertex takes a warp.
+// Vertices from SOLVE_CTA_CLASS on take a CTA: with a warp each, one vertex of
+// 1e6 neighbours was the kernel's 4.4 ms (3.4 ms with another unrolling of the
+// same loop), 0.6 ms so.
 __device__ __forceinline__ void solve_write(long long d, const VAcc &a, long long sS1, long long sA1, int induced,
                                             long long *o) {
     long long psi[15];
@@ -97,13 +100,19 @@ __device__ __forceinline__ void solve_write(long long d, const VAcc &a, long lon
 }
 
 constexpr int SOLVE_WARPS = 8;
-// Degree class (of degree 64) from which a vertex has a warp to itself.
+// Least degree class (of degree 64) from which a vertex has a warp to itself.
 // Vertices of high degree are often neighbours in the caller's order too, and
 // a warp that sums 32 of them in turn is the kernel's tail: with the line at
 // degrees 512, 128, 64 it took 84, 37, 25 us on a power-law graph of 1e5
-// vertices, 41, 27, 20 on R-MAT 14 and 1321, 1233, 1137 on R-MAT 22 (R-MAT
-// 18, with one vertex of 25254 neighbours: 83, 110, 95).
+// vertices, 41, 27, 20 on R-MAT 14 and 1321, 1233, 1137 on R-MAT 22. Where
+// most vertices have such degrees there is no tail, and 32 at a time is the
+// cheaper way, above all into host memory: the line is at 2.5 times the mean
+// degree or above (G(1e6, mean degree 70): 583 us with a warp for every
+// vertex, 377 so; G(4e5, 80) into host memory 1221, 316), in graphs with 20
+// groups of 32 vertices and more a multiprocessor (G(1e5, 100): 72 us with
+// warps, 70; G(50000, 200): 58, 75).
 constexpr int SOLVE_WARP_CLASS = 20;
+constexpr int SOLVE_CTA_CLASS = 40;   // degree 2048
 
 __global__ void __launch_bounds__(SOLVE_WARPS * 32) k_solve(Graph g, const VAcc *vacc, const int *perm,
                                                             const int2 *vinfo, long long *out, int induced,
@@ -116,20 +125,49 @@ __global__ void __launch_bounds__(SOLVE_WARPS * 32) k_solve(Graph g, const VAcc 
     long long *ob = obuf[threadIdx.x >> 5];
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
-    const int bound = min(coff[long_class * ntiles], g.n);
-    // highest degrees first, on different CTAs
-    const int spread = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-    for (int x = g.n - 1 - spread; x >= bound; x -= nw) {
-        const int4 rx = g.rinfo[x];
-        long long sS1 = 0, sA1 = 0;
-        for (int p = rx.x + lane; p < rx.z; p += 32) {
+    const int bound = min(coff[long_class * ntiles], g.n), top = min(coff[SOLVE_CTA_CLASS * ntiles], g.n);
+    auto sums = [&](const int4 &rx, int first, int stride, long long &sS1, long long &sA1) {
+        sS1 = sA1 = 0;
+        for (int p = rx.x + first; p < rx.z; p += stride) {
             const longlong2 sa = *reinterpret_cast<const longlong2 *>(&vacc[g.ncol[p]]);
             sS1 += sa.x;
             sA1 += sa.y;
         }
         sS1 = warp_sum(sS1);
         sA1 = warp_sum(sA1);
-        if (lane == 0) solve_write(rx.z - rx.x, vacc[x], sS1, sA1, induced, out + (size_t)perm[x] * 15);
+    };
+    auto write = [&](int x, const int4 &rx, long long sS1, long long sA1) {   // one warp
+        if (lane == 0) solve_write(rx.z - rx.x, vacc[x], sS1, sA1, induced, ob);
+        __syncwarp();
+        if (lane < 15) out[(size_t)perm[x] * 15 + lane] = ob[lane];
+        __syncwarp();
+    };
+    for (int x = g.n - 1 - (int)blockIdx.x; x >= top; x -= gridDim.x) {
+        const int4 rx = g.rinfo[x];
+        long long sS1, sA1;
+        sums(rx, threadIdx.x, SOLVE_WARPS * 32, sS1, sA1);
+        if (lane == 0) {
+            ob[16] = sS1;
+            ob[17] = sA1;
+        }
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            sS1 = sA1 = 0;
+            for (int w = 0; w < SOLVE_WARPS; ++w) {
+                sS1 += obuf[w][16];
+                sA1 += obuf[w][17];
+            }
+            write(x, rx, sS1, sA1);
+        }
+        __syncthreads();
+    }
+    // highest degrees first, on different CTAs
+    const int spread = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    for (int x = top - 1 - spread; x >= bound; x -= nw) {
+        const int4 rx = g.rinfo[x];
+        long long sS1, sA1;
+        sums(rx, lane, 32, sS1, sA1);
+        write(x, rx, sS1, sA1);
     }
     for (int xo0 = gw * 32; long_class > 0 && xo0 < g.n; xo0 += nw * 32) {
         const int xo = xo0 + lane;   // caller id
@@ -183,7 +221,9 @@ void launch_solve(Work &w, long long *out, cudaStream_t st) {
     const int grid = w.num_sms * w.tune[TUNE_GRID_SOLVE];
     // a graph with no more vertices than the grid has warps: one warp per
     // vertex (long_class 0), so that no warp solves 32 vertices in turn
-    const int lc = (long long)w.n <= (long long)grid * SOLVE_WARPS ? 0 : min(w.tune[TUNE_LONG_ROW_CLASS], SOLVE_WARP_CLASS);
+    const int mean = w.n >= 640ll * w.num_sms ? (int)min(5ll * w.m / (2ll * w.n), (long long)MAX_DEGREE) : 0;   // 2.5 times
+    const int line = min(min(w.tune[TUNE_LONG_ROW_CLASS], max(SOLVE_WARP_CLASS, deg_class(mean))), SOLVE_CTA_CLASS);
+    const int lc = (long long)w.n <= (long long)grid * SOLVE_WARPS ? 0 : line;
     launch_pdl(k_solve, grid, SOLVE_WARPS * 32, 0, st,
         g, w.vacc, w.perm, w.vinfo, out, w.induced, w.coff, w.ntiles, lc, w.counters);
     after_launch(st, K_SOLVE);
