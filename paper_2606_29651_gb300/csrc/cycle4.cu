@@ -1039,12 +1039,10 @@ constexpr size_t CC_SMEM = cq_smem(CC_THREADS, CC_SLOTS, CC_MAXW);
 __global__ void __launch_bounds__(CM_THREADS) k_c4_mid(Graph g, VAcc *vacc, const int *lists, int *counters,
                                                        int cb) {
     pdl_begin();
-    if (call_stopped(counters)) return;
-    c4_queue<CM_THREADS, CM_SLOTS, CM_MAXW, true>(g, vacc, lists + 5 * (size_t)g.n,
-                                                  counters[CNT_C4_MIDP] + counters[CNT_C4_MIDP_LEFT],
-                                                  counters + CNT_C4_MIDP_NEXT, cb);
-    c4_queue<CM_THREADS, CM_SLOTS, CM_MAXW, false>(g, vacc, lists + 2 * (size_t)g.n, counters[CNT_C4_MID],
-                                                   counters + CNT_C4_MID_NEXT, cb);
+    const int np = counters[CNT_C4_MIDP] + counters[CNT_C4_MIDP_LEFT], nm = counters[CNT_C4_MID];   // (0 in a stopped call)
+    if (np == 0 && nm == 0) return;
+    c4_queue<CM_THREADS, CM_SLOTS, CM_MAXW, true>(g, vacc, lists + 5 * (size_t)g.n, np, counters + CNT_C4_MIDP_NEXT, cb);
+    c4_queue<CM_THREADS, CM_SLOTS, CM_MAXW, false>(g, vacc, lists + 2 * (size_t)g.n, nm, counters + CNT_C4_MID_NEXT, cb);
 }
 
 __global__ void __launch_bounds__(CC_THREADS) k_c4_cta(Graph g, VAcc *vacc, const int *lists, int *counters,
