@@ -220,8 +220,16 @@ int32_t niorca_version(void);
  *   0..4  CTAs per SM of the relabel, triangle, edge-aggregate, 4-cycle and
  *         solve kernels (1..64; defaults 16, 8, 8, 8, 8)
  *   5     degree class from which a row is relabelled by a whole CTA
- *         (1..127; default 32, i.e. degree >= 512)
- *   6     largest wedge count W of a 4-cycle root handled by one warp (2..1536)
+ *         (1..127; default 32, i.e. degree >= 512); also the highest class
+ *         from which the orbit solve gives a vertex at least a warp of its
+ *         own (it does so from degree 64, or 2.5 times the mean, on)
+ *   6     largest wedge count W of a 4-cycle root that one warp counts in a
+ *         table (2..1536; default 1536; a table holds at most 1152, or 768 in
+ *         graphs of more than 2^21 vertices, and 32 in graphs of up to 32
+ *         vertices a multiprocessor). The filter that settles roots without a
+ *         table takes those up to 4/3 of it. In graphs of up to 2048 vertices
+ *         a multiprocessor, up to 8192 roots that it leaves are counted by
+ *         four warps each
  *   7     largest out-degree of a triangle root handled by one warp (2..64)
  *   8     largest out-degree of a CTA-tier triangle root that keeps the bit
  *         matrix of its out-neighbourhood (2..1152; default 1152)

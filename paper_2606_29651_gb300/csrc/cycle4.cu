@@ -940,7 +940,10 @@ __global__ void __launch_bounds__(CW_WARPS * 32, SPLIT ? 6 : 8) k_c4_warp_left(G
 // about 60 instructions per 32 wedges.
 constexpr int CF_WARPS = 8;
 constexpr int CF_LOG = 10;
-constexpr int CF_MAXW = 2048;   // two keys per word: about 8 of them may be falsely taken for repeats
+// W that the filter takes, for tables of up to maxw: 2048 at the default of
+// 1536. That is two keys per word of the filter, of which about 8 may be
+// falsely taken for repeats.
+__device__ __forceinline__ int cf_maxw(int maxw) { return maxw * 4 / 3; }
 
 struct __align__(16) C4FilterSmem {
     unsigned t[1 << CF_LOG];
@@ -959,7 +962,7 @@ __global__ void __launch_bounds__(CF_WARPS * 32, 5) k_c4_filter(Graph g, VAcc *v
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     const C4Limits<SPLIT> lim(maxw, cb, ck_min_wedges(coff, ntiles, g.n, teamw));
-    const long long most = min(maxw < CW_MAXW ? (long long)maxw : CF_MAXW, lim.team);   // (lowered knobs hold here too)
+    const long long most = min((long long)cf_maxw(maxw), lim.team);
     for (int i = lane; i < (1 << CF_LOG) / 4; i += 32) reinterpret_cast<uint4 *>(S.t)[i] = make_uint4(EMPTY, EMPTY, EMPTY, EMPTY);
     __syncwarp();
     auto do_root = [&](int u, const int4 &ru, int2 s0) {
@@ -973,7 +976,7 @@ __global__ void __launch_bounds__(CF_WARPS * 32, 5) k_c4_filter(Graph g, VAcc *v
     };
     // ids of low degree: four roots at a time, eight lanes each
     const int2 Z2 = make_int2(0, 0);
-    const int low = maxw >= 256 ? low_degree_ids(g.n, nw, coff, ntiles) : 0;
+    const int low = most >= 8 * SMALL_ROW ? low_degree_ids(g.n, nw, coff, ntiles) : 0;
     for (long long u0 = 4ll * gw; u0 < low; u0 += 4ll * nw) {
         const int u = (int)u0 + (lane >> 3), l = lane & 7;
         int4 ru = make_int4(0, 0, 0, 0);
