@@ -1624,7 +1624,7 @@ void launch_cycle4(Work &w, cudaStream_t st) {
     if (filter) {
         launch_pdl(packed ? k_c4_filter<false> : k_c4_filter<true>, w.num_sms * min(w.tune[TUNE_GRID_C4], occ_f),
                    CF_WARPS * 32, CF_SMEM, st, g, w.vacc, w.lists, w.counters, maxw, cb, teamw, w.coff, w.ntiles);
-        after_launch(st, K_C4_WARP);
+        after_launch(st, K_C4_FILTER);
         launch_pdl(packed ? k_c4_warp_left<false> : k_c4_warp_left<true>, w.num_sms * (packed ? occ_l : occ_ls),
                    CW_WARPS * 32, 0, st, g, w.vacc, w.lists, w.counters, maxw, cb, few, teamw, w.coff, w.ntiles);
         after_launch(st, K_C4_WARP_LEFT);

@@ -158,7 +158,8 @@ void launch_validate(const int *rowptr, const int *colidx, int n, int m, int *st
 enum KernelId {
     K_CLASS_HIST, K_SCAN, K_CLASS_SCATTER, K_RELABEL, K_BATCH_SETUP,
     K_TRI_WARP, K_TRI_CTA, K_AGG_WARP, K_AGG_CTA, K_C4_WARP, K_C4_CTA, K_C4_PLAN, K_C4_TILED,
-    K_SOLVE, K_VALIDATE, K_C4_MID, K_TRI_BIG, K_AGG_BIG, K_C4_WARP_LEFT, K_C4_WEDGE_LEN, K_ADJ_BITS, K_COUNT
+    K_SOLVE, K_VALIDATE, K_C4_MID, K_TRI_BIG, K_AGG_BIG, K_C4_WARP_LEFT, K_C4_WEDGE_LEN, K_ADJ_BITS, K_C4_FILTER,
+    K_COUNT
 };
 const char *kernel_name(int id);
 

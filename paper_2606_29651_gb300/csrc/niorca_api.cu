@@ -39,7 +39,7 @@ const char *const kNames[K_COUNT] = {
     "k_class_hist", "k_scan", "k_class_scatter", "k_relabel_rows", "k_batch_setup",
     "k_tri_warp", "k_tri_cta", "k_agg_warp", "k_agg_cta", "k_c4_warp", "k_c4_cta", "k_c4_tiled_plan",
     "k_c4_tiled", "k_solve", "k_validate", "k_c4_mid", "k_tri_big", "k_agg_big",
-    "k_c4_warp_left", "k_c4_wedge_len", "k_adj_bits"};
+    "k_c4_warp_left", "k_c4_wedge_len", "k_adj_bits", "k_c4_filter"};
 }  // namespace
 
 const char *kernel_name(int id) { return (id >= 0 && id < K_COUNT) ? kNames[id] : "?"; }
