@@ -73,6 +73,8 @@ def deg_class(d: np.ndarray) -> np.ndarray:
 # niorca_set_tuning): triangle roots by out-degree, 4-cycle roots by wedges.
 TRI_WARP_MAXD, TRI_CTA_MAXD, TRI_BITS_MAXD, TRI_HASH_MAXD = 64, 256, 1152, 8192
 C4_MID_MAXW, C4_CTA_MAXW = 3072, 12288
+C4_TABLE_MAXW = {True: 1152, False: 768}   # a warp's table, packed or split
+C4_SMALL_MAXW = 32   # the same in graphs of at most 32 vertices per SM
 WL_MAXD = 1024   # roots with more in-neighbours go to the key-tiled tier
 
 
@@ -113,9 +115,11 @@ class Shape:
         self.din = np.bincount(rd[sel], minlength=n)
 
     def c4_tiers(self, c4_warp_ub: int = 1536, num_sms: int = 152) -> dict:
-        """Relabelled ids of the roots of every 4-cycle kernel (a graph with
-        fewer vertices than 32 warps per SM keeps roots above 256 wedges out
-        of the warp tiers)."""
+        """Relabelled ids of the 4-cycle roots by their wedges alone: what one
+        warp can count (in two sizes; up to 256 wedges in a graph with fewer
+        vertices than 32 per SM), four warps, a CTA and the key-tiled tier.
+        Samples of roots of every size come from these classes; which kernel
+        takes a root is c4_routes."""
         n, w = self.n, self.w_root
         if n <= 32 * num_sms:
             c4_warp_ub = min(c4_warp_ub, 256)
@@ -128,12 +132,7 @@ class Shape:
         warp = live & ~hub & (w <= warp_lim)
         wbig = live & ~hub & ~warp & (w <= big_lim)
         rest = live & ~warp & ~wbig
-        # counters of the key-tiled tier: words per zone of degrees, a CTA holds 48K of them
-        words = 0
-        for lo, hi, bits in ((1024, None, 16), (256, 1024, 10), (64, 256, 8), (32, 64, 6), (16, 32, 5), (8, 16, 4),
-                             (4, 8, 3), (2, 4, 2)):
-            ids = int(((self.d >= lo) & (self.d < (hi or 1 << 62))).sum())
-            words += (-(-ids // (32 // bits)) + 3) & ~3
+        words = self.key_words()
         min_team = C4_MID_MAXW if words <= 48 << 10 else 2 * C4_MID_MAXW if words <= 192 << 10 else C4_CTA_MAXW
         team = rest & ((w > min_team) | hub)
         midp = rest & ~team & (w <= 2 * C4_MID_MAXW) & (w <= pack_lim)
@@ -141,6 +140,44 @@ class Shape:
         cta = rest & ~team & ~midp & ~mid
         return {"k_c4_warp": warp, "k_c4_warp_big": wbig, "k_c4_midp": midp, "k_c4_mid": mid, "k_c4_cta": cta,
                 "k_c4_tiled": team}
+
+    def key_words(self) -> int:
+        """Counter words of the key-tiled tier (a CTA holds 48K of them)."""
+        words = 0
+        for lo, hi, bits in ((1024, None, 16), (256, 1024, 10), (64, 256, 8), (32, 64, 6), (16, 32, 5), (8, 16, 4),
+                             (4, 8, 3), (2, 4, 2)):
+            ids = int(((self.d >= lo) & (self.d < (hi or 1 << 62))).sum())
+            words += (-(-ids // (32 // bits)) + 3) & ~3
+        return words
+
+    def c4_routes(self, maxw: int = 1536, teamw: int = C4_CTA_MAXW, num_sms: int = 152) -> dict:
+        """Relabelled ids of the roots that every 4-cycle kernel takes first, in
+        a single graph in which at most a third of the pairs of neighbours
+        are edges. `k_c4_filter` hands the roots with more than 32 possible
+        repeats on to `k_c4_warp_left` (or, when they are few in a graph of at
+        most 2048 vertices per SM, to `k_c4_mid`), which only the keys tell:
+        they are listed where they go first."""
+        n, w = self.n, self.w_root
+        hub = self.din > WL_MAXD   # the key-tiled tier, whatever W
+        live = (self.din >= 2) & ((w >= 2) | hub)
+        pack = (1 << (32 - int(max(n - 1, 1)).bit_length())) - 2   # packed tables hold counts below this
+        packed = pack >= maxw
+        table = min(maxw, C4_TABLE_MAXW[packed])
+        words = self.key_words()
+        team = min(teamw, C4_MID_MAXW if words <= 48 << 10 else 2 * C4_MID_MAXW if words <= 192 << 10 else teamw)
+        res, rest = {}, live & ~hub
+        if n > 32 * num_sms:
+            filt = rest & (self.din <= 64) & (w <= min(maxw * 4 // 3, team)) & (w * w <= 48 * n)
+            left = rest & ~filt & (w <= table)
+            res = {"k_c4_filter": filt, "k_c4_warp_left": left}
+            rest = rest & ~filt & ~left
+        else:
+            res = {"k_c4_warp": rest & (w <= min(table, C4_SMALL_MAXW))}
+            rest = rest & ~res["k_c4_warp"]
+        tiled = rest & (w > team)
+        rest = rest & ~tiled
+        mid = rest & (((w <= 2 * C4_MID_MAXW) & (w <= pack)) | (w <= C4_MID_MAXW))
+        return {**res, "k_c4_mid": mid, "k_c4_cta": rest & ~mid, "k_c4_tiled": tiled | (live & hub)}
 
     def tri_tiers(self, warp_maxd: int = TRI_WARP_MAXD) -> dict:
         """Relabelled ids of the roots of every triangle / aggregate kernel
@@ -211,8 +248,9 @@ def algorithmic_bytes(rowptr: np.ndarray, colidx: np.ndarray, c4_warp_ub: int = 
             min(d+w, |N+(u) ∩ N+(v)|)  (None when too costly to list),
     B_c4  = 4 * number of wedges u - v - w with v, w below u (cycle roots),
     B_out = 120 n.
-    A root's wedges (or triangle probes) count for the tier kernel that
-    takes it (Shape.c4_tiers, Shape.tri_tiers).
+    Triangle probes count for the tier kernel that takes their root
+    (Shape.tri_tiers), wedges for the class of their root's size
+    (Shape.c4_tiers; by kernel: launched_bytes).
     """
     sh = shape if shape is not None else Shape(rowptr, colidx)
     n, m = sh.n, sh.m
@@ -235,14 +273,12 @@ def algorithmic_bytes(rowptr: np.ndarray, colidx: np.ndarray, c4_warp_ub: int = 
     return res
 
 
-def launched_bytes(ab: dict, n: int) -> dict:
-    """ab["per_kernel"] by the kernels that run on a large graph: k_c4_filter
-    walks every root that fits a table of one warp."""
-    per = dict(ab["per_kernel"])
-    big = per.pop("k_c4_warp_big")
-    per["k_c4_filter"] = per.pop("k_c4_warp")
-    if 48 * n >= 1536 ** 2:   # the filter's limit on the repeats it expects
-        per["k_c4_filter"] += big
+def launched_bytes(ab: dict, shape: "Shape", c4_warp_ub: int = 1536) -> dict:
+    """ab["per_kernel"] with the 4-cycle wedges by the kernel that takes their
+    root first (Shape.c4_routes)."""
+    per = {k: v for k, v in ab["per_kernel"].items() if not k.startswith("k_c4")}
+    for k, msk in shape.c4_routes(c4_warp_ub).items():
+        per[k] = 4 * int(shape.w_root[msk].sum())
     return per
 
 
@@ -530,7 +566,7 @@ def run_rmat(ni, torch, dev, stream, timer, steps, scale, peak) -> dict:
     _, pairs, _ = sh.k4_bytes(max_pairs=0)
     ab["k4_pairs_checked"] = pairs
     rl = roofline_terms(ab, ms, peak)
-    per = launched_bytes(ab, len(rp) - 1)
+    per = launched_bytes(ab, sh)
     rl["per_kernel_frac"] = {k: round(per[k] / (kern[k][0] * 1e-3) / 1e9 / peak, 4) for k in per if k in kern and per[k]}
     return {"workload": f"R-MAT scale {scale}, edge factor 16, (.57,.19,.19,.05), seed 1; loops and duplicates removed",
             "n": len(rp) - 1, "edges": edges, "steps": len(step_ms), "ms_per_call": ms, "edges_per_s": edges / (ms * 1e-3),
@@ -773,7 +809,7 @@ def run_ours(args) -> None:
     tun = ni.get_tuning()
     sh = Shape(rp, ci)
     ab = algorithmic_bytes(rp, ci, tun["c4_warp_maxw"], tun["warp_maxd"], shape=sh)
-    alg = launched_bytes(ab, len(rp) - 1).get(top_name)
+    alg = launched_bytes(ab, sh, tun["c4_warp_maxw"]).get(top_name)
     achieved = alg / (top_avg_ms * 1e-3) / 1e9 if alg else None
     roofline = {
         "bound": "hbm", "kernel": top_name, "achieved": achieved, "peak": peak, "unit": "GB/s",
