@@ -172,23 +172,16 @@ __device__ __forceinline__ int wedge_chunk(const Graph &g, int u, int b, int din
 
 // Wedge segments of a root's first two chunks of in-neighbours, held in
 // registers by the warp (lane p: in-neighbours p and 32 + p) so that its
-// walks search no row again. With one chunk (din <= 32) its segment table
-// may be built already (built0: pre0 and total0 are the lane's).
+// walks search no row again.
 struct RootChunks {
     int have = 0;          // chunks held: 0, 1 or 2 (warp-uniform)
-    bool built0 = false;   // the warp's segment table holds chunk 0
     int v0 = -1, st0 = 0, len0 = 0, v1 = -1, st1 = 0, len1 = 0;
-    int pre0 = 0, total0 = 0;
 };
 
 // Segment table of chunk c (in-neighbours 32c ...) of root u, from the
 // registers of rc when it holds the chunk, else by searching the rows.
 __device__ __forceinline__ int root_chunk(const Graph &g, int u, int b, int din, int c, SegTab &T,
                                           const RootChunks &rc, int &v, int &len, int &pre) {
-    if (c == 0 && rc.built0) {
-        v = rc.v0, len = rc.len0, pre = rc.pre0;
-        return rc.total0;
-    }
     if (c < rc.have) {
         v = c == 0 ? rc.v0 : rc.v1;
         len = c == 0 ? rc.len0 : rc.len1;
@@ -440,18 +433,18 @@ __device__ __forceinline__ void c4_root(const Graph &g, VAcc *vacc, int u, int b
         }
     }
     if (sweep) {
-        long long su = 0;
-        for (int i = tid; i < (CTA ? nt : 0); i += nthreads) {
-            const int slot = CTA ? T.touched[i] : i;
-            if (!CTA && T.empty(slot)) continue;
-            const int c = T.cnt(slot);
-            if (c >= 2) {
-                su += c2(c);
-                add64(&vacc[T.key(slot)].C4, c2(c));
+        if (CTA) {   // (a warp's credits are done)
+            long long su = 0;
+            for (int i = tid; i < nt; i += nthreads) {
+                const int slot = T.touched[i], c = T.cnt(slot);
+                if (c >= 2) {
+                    su += c2(c);
+                    add64(&vacc[T.key(slot)].C4, c2(c));
+                }
             }
+            su = warp_sum(su);
+            if (lane == 0 && su) add64(&vacc[u].C4, su);
         }
-        su = warp_sum(su);
-        if (CTA && lane == 0 && su) add64(&vacc[u].C4, su);
         // middle vertices: each wedge through v adds c_w - 1
         if (tid < 32) pv[tid] = 0;
         sync();
