@@ -1133,13 +1133,14 @@ __device__ __forceinline__ CkPlan ck_plan(int *region, const CkZone *z, int word
 
 // CTA 0: root order of the key-tiled tier: the queued roots (list 4, their
 // wedge counts in list 1) sorted by decreasing wedge count (64 buckets, two
-// per octave) into list 0, and the prefix sums of their in-degrees into list
-// 2. Every other CTA: enc, ends and index.
+// per octave) into list 0. Their in-degrees sum to more than m / 2 only in a
+// CSR that is not symmetric, which is reported. Every other CTA: enc, ends and
+// index.
 __global__ void __launch_bounds__(1024) k_c4_tiled_plan(Graph g, int *lists, int *counters, const int *coff, int ntiles,
-                                                        int words, int *region) {
+                                                        int words, int *region, int *status) {
     pdl_begin();
     __shared__ int hist[64], base[64];
-    __shared__ int wsum[32];
+    __shared__ long long degrees;
     __shared__ CkZone z[CK_ZONES + 1];
     __shared__ int glo[CK_MAX_GROUPS];
     if (call_stopped(counters)) return;
@@ -1188,13 +1189,14 @@ __global__ void __launch_bounds__(1024) k_c4_tiled_plan(Graph g, int *lists, int
         }
         return;
     }
-    int *sorted = lists, *offs = lists + 2 * (size_t)g.n;
+    int *sorted = lists;
     auto bucket = [](int w) {
         const int e = 31 - __clz(max(w, 1));
         const int half = e > 0 ? (w >> (e - 1)) & 1 : 0;
         return 63 - min(63, 2 * e + half);
     };
     if (threadIdx.x < 64) hist[threadIdx.x] = 0;
+    if (threadIdx.x == 0) degrees = 0;
     __syncthreads();
     for (int i = threadIdx.x; i < nt; i += blockDim.x) atomicAdd(&hist[bucket(wts[i])], 1);
     __syncthreads();
@@ -1205,26 +1207,17 @@ __global__ void __launch_bounds__(1024) k_c4_tiled_plan(Graph g, int *lists, int
         base[2 * threadIdx.x + 1] = ex + a;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < nt; i += blockDim.x) sorted[atomicAdd(&base[bucket(wts[i])], 1)] = roots[i];
-    __syncthreads();
-    int carry = 0;
-    for (int j0 = 0; j0 < nt; j0 += blockDim.x) {
-        const int j = j0 + threadIdx.x;
-        int din = 0;
-        if (j < nt) {
-            const int4 r = g.rinfo[sorted[j]];
-            din = r.y - r.x;
-        }
-        const int incl = warp_inclusive_scan(din);
-        if (lane_id() == 31) wsum[threadIdx.x >> 5] = incl;
-        __syncthreads();
-        if (threadIdx.x < 32) wsum[threadIdx.x] = warp_inclusive_scan(wsum[threadIdx.x]);
-        __syncthreads();
-        const int before = (threadIdx.x >= 32 ? wsum[(threadIdx.x >> 5) - 1] : 0) + incl - din;
-        if (j < nt) offs[j] = carry + before;
-        carry += wsum[31];
-        __syncthreads();
+    long long din = 0;
+    for (int i = threadIdx.x; i < nt; i += blockDim.x) {
+        const int u = roots[i];
+        sorted[atomicAdd(&base[bucket(wts[i])], 1)] = u;
+        const int4 ru = g.rinfo[u];
+        din += ru.y - ru.x;
     }
+    din = warp_sum(din);
+    if (lane_id() == 0) add64(&degrees, din);
+    __syncthreads();
+    if (threadIdx.x == 0 && degrees > g.m / 2) set_status(status, ST_ENOTSIMPLE);
 }
 
 // What a CTA keeps in shared memory.
@@ -1521,13 +1514,12 @@ __device__ __forceinline__ void c4_wide_top(const Graph &g, VAcc *vacc, int u, i
     if (lane == 0 && su) add64(&vacc[u].C4, su);
 }
 
-// Roots from the work queue. The prefix sums of the roots' in-degrees pass
-// m / 2 only for a CSR that is not symmetric: such a root stops with
-// ENOTSIMPLE.
+// Roots from the work queue. Every access stays in range for any CSR with
+// sorted rows or not: runs lie within their rows, and every entry of `enc` is
+// a counter of the CTA.
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1)
-    k_c4_tiled(Graph g, VAcc *vacc, const int *lists, int *counters, const int *coff, int ntiles, int words, int *region,
-               int *status) {
+    k_c4_tiled(Graph g, VAcc *vacc, const int *lists, int *counters, const int *coff, int ntiles, int words, int *region) {
     pdl_begin();
     extern __shared__ __align__(16) unsigned char dsm[];
     CkShared S;
@@ -1546,7 +1538,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1)
     if (call_stopped(counters)) return;
     const int nt = counters[CNT_C4_TEAM];
     if (nt == 0) return;
-    const int *sorted = lists, *offs = lists + 2 * (size_t)g.n;
+    const int *sorted = lists;
     for (int i = threadIdx.x; i <= words / 4; i += THREADS) reinterpret_cast<uint4 *>(S.cnt)[i] = make_uint4(0, 0, 0, 0);
     if (threadIdx.x == 0) {
         ck_zones(coff, ntiles, g.n, S.z);
@@ -1563,10 +1555,6 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1)
         if (j >= nt) break;
         const int u = sorted[j];
         const int4 ru = g.rinfo[u];
-        if ((long long)offs[j] + (ru.y - ru.x) > g.m / 2 || offs[j] < 0) {
-            if (threadIdx.x == 0) set_status(status, ST_ENOTSIMPLE);
-            continue;
-        }
         const bool wide = ru.y - ru.x > CK_NARROW_MAXD;
         if (wide) c4_wide_top<THREADS>(g, vacc, u, words, S);
         c4_tiled_root<THREADS>(g, vacc, u, wide ? min(u, S.z[0].lo) : u, words, P, S);
@@ -1639,16 +1627,16 @@ void launch_cycle4(Work &w, cudaStream_t st) {
     const bool small = w.n <= CK_SMALL_N;
     const int words = small ? (w.n / 2 + 4 * CK_ZONES + 4) & ~3 : CK_WORDS;
     launch_pdl(k_c4_tiled_plan, 1 + min(2 * w.num_sms, w.m / 4096 + 1), 1024, 0, st, g, w.lists, w.counters, w.coff, w.ntiles, words,
-               w.tcnt);
+               w.tcnt, w.status);
     after_launch(st, K_C4_PLAN);
     if (small) {
         const size_t smem = ck_smem(256, words);
         const int occ = (int)min((size_t)4, (size_t)(227 * 1024) / (smem + 1024));
         launch_pdl(k_c4_tiled<256>, w.num_sms * occ, 256, smem, st, g, w.vacc, w.lists, w.counters, w.coff, w.ntiles, words,
-                   w.tcnt, w.status);
+                   w.tcnt);
     } else {
         launch_pdl(k_c4_tiled<1024>, w.num_sms, 1024, ck_smem(1024, words), st, g, w.vacc, w.lists, w.counters, w.coff,
-                   w.ntiles, words, w.tcnt, w.status);
+                   w.ntiles, words, w.tcnt);
     }
     after_launch(st, K_C4_TILED);
 }

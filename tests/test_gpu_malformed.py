@@ -45,3 +45,16 @@ def test_overlapping_rows_stop_the_call(ni, lib, n, m):  # noqa: F811
     assert int(status.item()) == 1 << Status.EINVAL
     good = gg.rmat(10, 8, seed=2)
     assert_same(gpu_count(ni, *good), oracle.count(*good), "the next call")
+
+
+def test_too_many_in_neighbours_are_reported(ni):  # noqa: F811
+    # 60 rows of 2000 entries whose vertices do not list them back: roots of
+    # the key-tiled 4-cycle tier with more in-entries than half of the CSR
+    from paper_2606_29651_gb300 import Status
+    n, hubs = 6000, 60
+    rp = np.concatenate([np.zeros(n - hubs + 1, np.int32), 2000 * np.arange(1, hubs + 1, dtype=np.int32)])
+    ci = np.tile(np.arange(0, 4000, 2, dtype=np.int32), hubs)
+    dev = torch.device("cuda:0")
+    ni.last_status()
+    ni.count(torch.from_numpy(rp).to(dev), torch.from_numpy(ci).to(dev))
+    assert ni.last_status() == Status.ENOTSIMPLE
