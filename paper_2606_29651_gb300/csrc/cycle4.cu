@@ -108,7 +108,7 @@ constexpr int SAMPLE_CTAS = 8;
 enum { C4_FILTER = 1, C4_TABLES = 2 };
 template <int L>
 __global__ void __launch_bounds__(256, 8) k_c4_wedge_len(Graph g, int2 *wl, const VAcc *vacc, int *counters,
-                                                         const int *coff, int ntiles, int sample) {
+                                                         const int *coff, int ntiles, int sample, int mode) {
     pdl_begin();
     if (call_stopped(counters)) return;
     auto row = [&](int u, int first, int stride) {
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(256, 8) k_c4_wedge_len(Graph g, int2 *wl, cons
     };
     const int bound = min(coff[deg_class(WL_LONG) * ntiles], g.n);
     const int ctas = gridDim.x - sample;
-    if (sample == 0 && blockIdx.x == 0 && threadIdx.x == 0) counters[CNT_C4_MODE] = C4_FILTER;
+    if (sample == 0 && blockIdx.x == 0 && threadIdx.x == 0) counters[CNT_C4_MODE] = mode;
     if ((int)blockIdx.x >= ctas) {   // CTAs of their own for the sample, a vertex of degree below WL_LONG per thread
         const long long at = (long long)(blockIdx.x - ctas) * blockDim.x + threadIdx.x;
         const int u = (int)(at * bound / (sample * (int)blockDim.x));
@@ -1580,9 +1580,19 @@ void launch_cycle4(Work &w, cudaStream_t st) {
     // 320 with the limit below; 357 graphs of 18 to 180: 138, 160, 141).
     const bool tiny = w.graphs > 1 && w.n / w.graphs < 150 && w.n > w.num_sms * 32;
     const bool filter = w.n > w.num_sms * 32 && !tiny;
-    const int sample = filter && w.m >= 12ll * w.n ? SAMPLE_CTAS : 0;
+    // Batches of random graphs in which the average root (d^2 / 3 wedges at
+    // mean degree d, over the n / graphs keys of its graph) repeats eight keys
+    // and more: the tables at once too. Larger single graphs of that kind are
+    // better off with the filter, whose rule knows their size (us a call,
+    // filter first / tables at once: 100 graphs G(700, 0.03), 15 repeats,
+    // 408 / 377; 200 graphs G(300, 0.1), 150, 597 / 548; 1000 graphs
+    // G(300, 0.05), 9, 943 / 932; 8192 power-law graphs, 0.2, 11966 / 13446;
+    // one G(8000, mean degree 40), 18, 192 / 209).
+    const double mean = (double)w.m / w.n;
+    const bool repeats = w.graphs > 1 && mean * mean * mean * mean / 9 >= 2.0 * 8 * w.n / w.graphs;
+    const int sample = filter && !repeats && w.m >= 12ll * w.n ? SAMPLE_CTAS : 0;
     launch_pdl((long long)w.m < 16ll * w.n ? k_c4_wedge_len<8> : k_c4_wedge_len<16>, w.num_sms * 8 + sample, 256, 0, st, g, wl,
-               w.vacc, w.counters, w.coff, w.ntiles, sample);
+               w.vacc, w.counters, w.coff, w.ntiles, sample, repeats ? C4_TABLES : C4_FILTER);
     after_launch(st, K_C4_WEDGE_LEN);
     const int cb = packed_count_bits(w.n);
     // a packed word holds counts up to 2^cb - 2; with many vertices (large

@@ -86,3 +86,18 @@ def test_lowered_limit_of_the_warp_tables(tuning):  # noqa: F811
     for maxw in (2, 33, 200):
         tuning.set_tuning(c4_warp_maxw=maxw)
         assert_same(gpu_count(tuning, rp, ci), exp, f"c4_warp_maxw {maxw}")
+
+
+@pytest.mark.parametrize("graphs,n,p", [(40, 300, 0.1), (30, 700, 0.02), (20, 700, 0.04)])
+def test_batches_of_random_graphs(ni, graphs, n, p):  # noqa: F811
+    # eight and more repeated keys per root of (n p)^2 / 3 wedges, and fewer
+    gs = [gg.er(n, p, 30 + i) for i in range(graphs)]
+    assert (((n * p) ** 2 / 3) ** 2 / (2 * n) >= 8) == (p > 0.03) and graphs * n > 32 * 152
+    rowptr, colidx, vo, eo = gg.pack(gs)
+    dev = torch.device("cuda:0")
+    out = ni.count_batch(torch.from_numpy(rowptr.astype(np.int32)).to(dev), torch.from_numpy(colidx).to(dev),
+                         torch.from_numpy(vo).to(dev), torch.from_numpy(eo).to(dev))
+    ni.check()
+    got = out.cpu().numpy()
+    for i, (rp, ci) in enumerate(gs):
+        assert_same(got[vo[i]:vo[i + 1]], oracle.count(rp, ci), f"graph {i}")
