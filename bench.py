@@ -74,7 +74,7 @@ def deg_class(d: np.ndarray) -> np.ndarray:
 TRI_WARP_MAXD, TRI_CTA_MAXD, TRI_BITS_MAXD, TRI_HASH_MAXD = 64, 256, 1152, 8192
 C4_MID_MAXW, C4_CTA_MAXW = 3072, 12288
 C4_TABLE_MAXW = {True: 1152, False: 768}   # a warp's table, packed or split
-C4_SMALL_MAXW = 32   # the same in graphs of at most 32 vertices per SM
+C4_SMALL_MAXW = {True: 32, False: 128}   # the same in graphs of at most 16 vertices per SM, and of at most 32
 WL_MAXD = 1024   # roots with more in-neighbours go to the key-tiled tier
 
 
@@ -172,7 +172,7 @@ class Shape:
             res = {"k_c4_filter": filt, "k_c4_warp_left": left}
             rest = rest & ~filt & ~left
         else:
-            res = {"k_c4_warp": rest & (w <= min(table, C4_SMALL_MAXW))}
+            res = {"k_c4_warp": rest & (w <= min(table, C4_SMALL_MAXW[n <= 16 * num_sms]))}
             rest = rest & ~res["k_c4_warp"]
         tiled = rest & (w > team)
         rest = rest & ~tiled

@@ -225,8 +225,8 @@ int32_t niorca_version(void);
  *         own (it does so from degree 64, or 2.5 times the mean, on)
  *   6     largest wedge count W of a 4-cycle root that one warp counts in a
  *         table (2..1536; default 1536; a table holds at most 1152, or 768 in
- *         graphs of more than 2^21 vertices, and 32 in graphs of up to 32
- *         vertices a multiprocessor). The filter that settles roots without a
+ *         graphs of more than 2^21 vertices, and 32 or 128 in graphs of up
+ *         to 16 or 32 vertices a multiprocessor). The filter that settles roots without a
  *         table takes those up to 4/3 of it. In graphs of up to 2048 vertices
  *         a multiprocessor, up to 8192 roots that it leaves are counted by
  *         four warps each

@@ -37,7 +37,8 @@ constexpr int CW_WARPS = 4;
 constexpr int CW_WORDS = 1536;      // table words per warp of k_c4_warp: 6 KB, 8 CTAs of 4 warps per SM
 constexpr int CWB_WORDS = 2048;     // split tables: 8 KB, 6 CTAs per SM
 constexpr int CW_MAXW = 1536;       // largest W of a root in the warp tiers
-constexpr int CW_SMALL_MAXW = 32;   // the same, for graphs of up to 32 vertices a multiprocessor
+constexpr int CW_SMALL_MAXW = 32;   // the same, for graphs of up to 16 vertices a multiprocessor
+constexpr int CW_FEW_MAXW = 128;    // and of up to 32
 constexpr int CW_DUPS = 32;         // repeated keys a warp credits by search at most
 constexpr int CW_LEFT_LIST = 0;     // list slot of the roots of k_c4_warp_left: the triangle heavy list,
                                     // which nothing reads after that stage
@@ -1611,7 +1612,11 @@ void launch_cycle4(Work &w, cudaStream_t st) {
     // what it leaves. Below, every warp has one root, and nearly all (W above
     // CW_SMALL_MAXW) go to the 4-warp tier at once, where the slowest walk is
     // shorter: with the filter in front, G(400, mean degree 20) took 67 us a
-    // call instead of 63, G(2000, 20) 75 instead of 71.
+    // call instead of 63, G(2000, 20) 75 instead of 71. From 16 vertices a
+    // multiprocessor on the 4-warp tier has several roots for each of its CTAs,
+    // and the line is higher (at 32 / 128 wedges: G(4800, 16) 104 / 99 us a
+    // call, a ring of 4800 vertices of degree 16 with 10% rewired 111 / 100;
+    // G(400, 20) 63 / 64, G(1000, 20) 67 / 68).
     if (filter) {
         launch_pdl(packed ? k_c4_filter<false> : k_c4_filter<true>, w.num_sms * min(w.tune[TUNE_GRID_C4], occ_f),
                    CF_WARPS * 32, CF_SMEM, st, g, w.vacc, w.lists, w.counters, maxw, cb, teamw, w.coff, w.ntiles);
@@ -1622,7 +1627,8 @@ void launch_cycle4(Work &w, cudaStream_t st) {
     } else {
         launch_pdl(packed ? k_c4_warp<false> : k_c4_warp<true>,
                    w.num_sms * min(w.tune[TUNE_GRID_C4], packed ? occ_w : occ_ws), CW_WARPS * 32, 0, st, g, w.vacc, w.lists,
-                   w.counters, tiny ? maxw : min(maxw, CW_SMALL_MAXW), cb, teamw, w.coff, w.ntiles);
+                   w.counters, tiny ? maxw : min(maxw, w.n > w.num_sms * 16 ? CW_FEW_MAXW : CW_SMALL_MAXW), cb, teamw,
+                   w.coff, w.ntiles);
         after_launch(st, K_C4_WARP);
     }
     static const int occ_m = resident_ctas((const void *)k_c4_mid, CM_THREADS, CM_SMEM);

@@ -17,7 +17,8 @@ def _padded(rp, ci, n):
 
 
 @pytest.mark.parametrize("name,make", [
-    ("small", lambda: gg.er_mean_degree(3000, 48, 5)),
+    ("small", lambda: gg.er_mean_degree(2400, 48, 5)),
+    ("few", lambda: gg.er_mean_degree(3000, 48, 5)),
     ("packed tables", lambda: gg.er_mean_degree(9000, 50, 6)),
     ("split tables", lambda: _padded(*gg.er_mean_degree(9000, 50, 6), (1 << 21) + 9)),
     ("hubs", lambda: gg.rmat(14, 16, seed=3)),
@@ -27,9 +28,10 @@ def test_every_root_goes_to_one_kernel(name, make):
     w, routes = sh.w_root, sh.c4_routes()
     live = (sh.din >= 2) & (w >= 2)
     assert (sum(m.astype(int) for m in routes.values()) == live).all(), name
-    if name == "small":
+    if name in ("small", "few"):
+        limit = 32 if name == "small" else 128
         assert set(routes) == {"k_c4_warp", "k_c4_mid", "k_c4_cta", "k_c4_tiled"}
-        assert w[routes["k_c4_warp"]].max() == 32 and w[routes["k_c4_mid"]].min() == 33
+        assert w[routes["k_c4_warp"]].max() <= limit < w[routes["k_c4_mid"]].min()
         return
     f, left = routes["k_c4_filter"], routes["k_c4_warp_left"]
     assert (w[f] ** 2 <= 48 * sh.n).all() and w[f].max() <= 2048 and sh.din[f].max() <= 64

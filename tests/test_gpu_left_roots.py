@@ -101,3 +101,10 @@ def test_batches_of_random_graphs(ni, graphs, n, p):  # noqa: F811
     got = out.cpu().numpy()
     for i, (rp, ci) in enumerate(gs):
         assert_same(got[vo[i]:vo[i + 1]], oracle.count(rp, ci), f"graph {i}")
+
+
+@pytest.mark.parametrize("n", [16 * 152, 16 * 152 + 1, 32 * 152, 32 * 152 + 1])   # small graphs' lines (152 multiprocessors)
+@pytest.mark.parametrize("k", [12, 24])
+def test_small_graphs(ni, n, k):  # noqa: F811
+    rp, ci = _ring(n, k, n)
+    assert_same(gpu_count(ni, rp, ci), oracle.count(rp, ci), f"ring {n}, {k}")
