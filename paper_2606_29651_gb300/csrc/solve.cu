@@ -136,10 +136,10 @@ __global__ void __launch_bounds__(SOLVE_WARPS * 32) k_solve(Graph g, const VAcc 
         sS1 = warp_sum(sS1);
         sA1 = warp_sum(sA1);
     };
-    auto write = [&](int x, const int4 &rx, long long sS1, long long sA1) {   // one warp
-        if (lane == 0) solve_write(rx.z - rx.x, vacc[x], sS1, sA1, induced, ob);
+    auto write = [&](int xo, long long d, const VAcc &a, long long sS1, long long sA1) {   // one warp
+        if (lane == 0) solve_write(d, a, sS1, sA1, induced, ob);
         __syncwarp();
-        if (lane < 15) out[(size_t)perm[x] * 15 + lane] = ob[lane];
+        if (lane < 15) out[(size_t)xo * 15 + lane] = ob[lane];
         __syncwarp();
     };
     for (int x = g.n - 1 - (int)blockIdx.x; x >= top; x -= gridDim.x) {
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(SOLVE_WARPS * 32) k_solve(Graph g, const VAcc 
                 sS1 += obuf[w][16];
                 sA1 += obuf[w][17];
             }
-            write(x, rx, sS1, sA1);
+            write(perm[x], rx.z - rx.x, vacc[x], sS1, sA1);
         }
         __syncthreads();
     }
@@ -165,9 +165,11 @@ __global__ void __launch_bounds__(SOLVE_WARPS * 32) k_solve(Graph g, const VAcc 
     const int spread = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     for (int x = top - 1 - spread; x >= bound; x -= nw) {
         const int4 rx = g.rinfo[x];
+        const int xo = perm[x];
+        const VAcc a = vacc[x];   // in flight during the sums
         long long sS1, sA1;
         sums(rx, lane, 32, sS1, sA1);
-        write(x, rx, sS1, sA1);
+        write(xo, rx.z - rx.x, a, sS1, sA1);
     }
     for (int xo0 = gw * 32; long_class > 0 && xo0 < g.n; xo0 += nw * 32) {
         const int xo = xo0 + lane;   // caller id
