@@ -1427,7 +1427,7 @@ __device__ __forceinline__ void c4_tiled_root(const Graph &g, VAcc *vacc, int u,
                         }
                     }
                     if (MID) {
-                        sum -= (unsigned)ln;   // (sums of c - 1 over a root's wedges are below W <= m)
+                        sum -= (unsigned)ln;   // (32 counts of at most 65535; 32 such windows fit run_add too)
                         su += sum;
                         run_add(&vacc[S.v[j]].C4, j, sum);
                     }

@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(TW_WARPS * 32, 6) k_tri_warp(Graph g, AdjBits 
 // ------------------------------------------------------------ CTA tiers
 
 // Roots with out-degree above the warp tier get a CTA each, in two sizes:
-// k_tri_cta (256 threads, dp <= TS_MAXD) needs about 18 KB of shared memory,
+// k_tri_cta (256 threads, dp <= TS_MAXD) needs 26 KB of shared memory,
 // so several CTAs share an SM; k_tri_big (1024 threads) takes the rest with
 // the bit matrix R up to TB_BITMAT_MAXD (hash of N+(u) capped at 4096 slots),
 // a 16384-slot hash up to TB_HASH_MAXD, and binary searches beyond.
