@@ -633,6 +633,7 @@ __device__ __forceinline__ int relabel_long(const RelabelArgs &A, int r, LongRow
         load(k, left, y, vi);
 #pragma unroll
         for (int h = 0; h < U; ++h) {
+            if (32 * h >= left) break;
             const bool act = 32 * h + lane < left;
             const int c = act ? deg_class(vi[h].y) : NCLASS + lane;   // inactive lanes match only themselves
             const unsigned peers = __match_any_sync(FULL, c);
