@@ -572,11 +572,11 @@ constexpr int C4_SEARCH = 128;
 // Roots that k_c4_filter leaves, in graphs of up to 2048 vertices a
 // multiprocessor: up to C4_FEW_LEFT of them are a few warps' walks in a row
 // at the end of the stage, so four warps walk each (k_c4_mid); more have work
-// for every warp, and one warp each is the cheaper way (300 power-law graphs
-// of 150 to 1500 vertices: 462 us a call with the line at 4000, 447 at 8000;
-// G(20000, mean degree 16) rewired from a ring: 163 at 8000, 223 at 16000;
-// none of them left to the warps: 100 graphs G(700, 0.03) 482 us, 417 with
-// the line).
+// for every warp, and one warp each is the cheaper way (us a call: 300
+// power-law graphs of 150 to 1500 vertices 453 with four warps for all, 462
+// with the line at 4000, 447 at 8000; one of 2e5 vertices, mean degree 20,
+// 1250 with four warps for all, 1235; G(6000, mean degree 30) 175 with the
+// line at 1000, 140 from 2000 on).
 constexpr int C4_FEW_LEFT = 8192;
 __device__ __forceinline__ int c4_mode(const int *counters) {
     return *reinterpret_cast<const volatile int *>(counters + CNT_C4_MODE);
@@ -1577,8 +1577,8 @@ void launch_cycle4(Work &w, cudaStream_t st) {
     int maxw = w.tune[TUNE_C4_WARP_MAXW] < CW_MAXW ? w.tune[TUNE_C4_WARP_MAXW] : CW_MAXW;
     // Batches of graphs of under 150 vertices on average: their roots have many
     // repeated keys and short walks, so all go to a warp's table at once (1756
-    // graphs of 18 to 144 vertices: 315 us a call; 359 with the filter first,
-    // 320 with the limit below; 357 graphs of 18 to 180: 138, 160, 141).
+    // graphs of 18 to 144 vertices: 315 us a call; 359 with the filter first;
+    // 357 graphs of 18 to 180: 138, 160).
     const bool tiny = w.graphs > 1 && w.n / w.graphs < 150 && w.n > w.num_sms * 32;
     const bool filter = w.n > w.num_sms * 32 && !tiny;
     // Batches of random graphs in which the average root (d^2 / 3 wedges at
